@@ -74,7 +74,8 @@ struct PrecDev : PrecBase {
   int nsm = 0;
   int64_t nlast = 0;
   DBuf<double> work;
-  DBuf<int32_t> flags;
+  DBuf<unsigned char> rec;  // the sweeps' records and unknowns
+  int64_t rec_bytes = 0;    // one sweep's records
   DBuf<unsigned long long> tick;
   DBuf<int> abort_flag;
   DBuf<double> fwork;  // fixed values on the levels (apply_fixed)

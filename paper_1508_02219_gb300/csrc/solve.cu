@@ -11,7 +11,6 @@
 namespace vb {
 namespace {
 
-constexpr int SW = 8;
 constexpr int TRI_R = 4;  // scalar rows per lane in the triangular solves (blocks up to 128)
 
 template <typename T>
@@ -37,11 +36,6 @@ __global__ void k_scatter_scale(int64_t n, const int32_t* __restrict__ sp, const
   }
 }
 
-__global__ void k_mul(int64_t n, const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ y) {
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x)
-    y[q] = __dmul_rn(a[q], b[q]);
-}
-
 // u <- L^{-1} P u per pivot block (one thread per block).
 template <typename TL>
 __device__ void pivot_forward(const TL* lu, const int32_t* pv, int m, double* u) {
@@ -62,30 +56,6 @@ __device__ void pivot_backward(const TL* lu, int m, double* u) {
     for (int k = i + 1; k < m; ++k) s = __dsub_rn(s, __dmul_rn(ld(lu + i * m + k), u[k]));
     u[i] = __ddiv_rn(s, ld(lu + i * m + i));
   }
-}
-
-// u <- U^{-1} L^{-1} P u for an FP32 pivot block in FP32 arithmetic (the
-// mixed factor applies its FP32 factors in FP32; vectors stay FP64).  m <= 32.
-__device__ void pivot_solve_f32(const float* lu, const int32_t* pv, int m, double* u) {
-  float x[32];
-  for (int k = 0; k < m; ++k) x[k] = (float)u[k];
-  for (int k = 0; k < m; ++k)
-    if (pv[k] != k) {
-      const float t = x[k];
-      x[k] = x[pv[k]];
-      x[pv[k]] = t;
-    }
-  for (int i = 1; i < m; ++i) {
-    float s = x[i];
-    for (int k = 0; k < i; ++k) s = __fmaf_rn(-lu[i * m + k], x[k], s);
-    x[i] = s;
-  }
-  for (int i = m - 1; i >= 0; --i) {
-    float s = x[i];
-    for (int k = i + 1; k < m; ++k) s = __fmaf_rn(-lu[i * m + k], x[k], s);
-    x[i] = __fdiv_rn(s, lu[i * m + i]);
-  }
-  for (int k = 0; k < m; ++k) u[k] = (double)x[k];
 }
 
 __global__ void k_pivot_fwd(int64_t nD, const int32_t* __restrict__ sz, const int64_t* __restrict__ roff,
@@ -172,165 +142,753 @@ __global__ void k_rowblk(int64_t nbr, const int64_t* __restrict__ roff, int64_t*
     for (int64_t q = roff[I] + lane; q < roff[I + 1]; q += 32) rowblk[q] = I;
 }
 
-// Bounded wait until row k is published (wait_flag); false when the wait gave
-// up or row k failed (a failed row publishes 2).
-__device__ __forceinline__ bool wait_row(const int32_t* done, int64_t k, int* abort, unsigned long long limit,
-                                         int* st) {
-  return wait_flag(done + k, abort, limit, st) == 1;
+// ---------------------------------------------------------------------------
+// The last level's triangular sweeps.
+//
+// Publication.  A row's unknowns are their own flags: the sweep's records
+// start as kTriEmpty in every word, a row stores its finished values there
+// with relaxed stores, and a dependant polls exactly the values that it needs
+// until none is empty.  No other data hangs on them, so neither side takes a
+// fence, and a link of the dependency chain costs one store and one load
+// through L2 (0.53 us measured from warp to warp) instead of store, fence,
+// flag, poll, fence and load.  The empty word is a NaN that no operation
+// produces; a value that carries those bits all the same (an input's payload)
+// is stored as the canonical NaN.
+//
+// Records are of type R.  The FP32 sweeps publish each unknown rounded to
+// FP32, the form its dependants use (a conversion from FP64 costs a dependant
+// 100 cycles a value on this part), beside the FP64 value (dbl), which block
+// rows of more than TRI_MR scalars read.  With R = double the record serves
+// both; that form needs less memory and is the one of the fixed-scratch solve.
+// A record starts on a 16-byte boundary: with w = 16 / sizeof(R), row k's at
+// coff[k] + (w - 1) k rounded down to a multiple of w.
+template <typename R>
+__device__ __forceinline__ int64_t tri_rec(int64_t off, int64_t k) {
+  constexpr int64_t w = 16 / sizeof(R);
+  return (off + (w - 1) * k) & ~(w - 1);
+}
+template <typename R>
+int64_t rec_words(int64_t n_last, int64_t p) {  // a whole number of 16-byte groups
+  constexpr int64_t w = 16 / sizeof(R);
+  return (n_last + (w - 1) * p + w - 1) & ~(w - 1);
 }
 
-constexpr int TRI_MR = 16;      // block rows up to this size use the lane-per-block path
+__device__ __forceinline__ bool tri_ready(double v) { return __double_as_longlong(v) != -1LL; }
+__device__ __forceinline__ bool tri_ready(float v) { return __float_as_int(v) != -1; }
+__device__ __forceinline__ void tri_publish(double* p, double v) {
+  if (!tri_ready(v)) v = __longlong_as_double(0x7ff8000000000000LL);
+  asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
+}
+__device__ __forceinline__ void tri_publish(float* p, float v) {
+  if (!tri_ready(v)) v = __int_as_float(0x7fc00000);
+  asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
+}
+__device__ __forceinline__ double tri_load(const double* p) {
+  double v;
+  asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
+
+constexpr int TRI_W = 4;         // warps per block
+constexpr int TRI_MR = 16;       // block rows up to this size use the lane-per-block path
+constexpr int TRI_MP = 32;       // pivot blocks up to this size are solved from shared memory
 constexpr int TRI_STAGE = 1024;  // values of a row staged in shared memory per warp
-constexpr int TRI_XQ = 16;       // dependency values loaded in one batch
+constexpr int TRI_XQ = 8;        // dependency values polled at once
 
-constexpr int TRI_PIV = 72;  // per warp: an FP32 pivot LU of up to 8 x 8 and its 8 interchanges
+// Blocks per SM.  The chain of rows bounds the sweeps, not the number of rows
+// in flight: 8 warps an SM with all their registers measured 82.5 ms on the
+// FGMRES of 720 000 unknowns, 12 warps 85.3 and 16 (128 registers) 95.9.
+constexpr int TRI_B = 2;
 
+// Shared memory of one warp.
 template <typename T>
-constexpr size_t tri_smem() {
-  return (size_t)SW * TRI_STAGE * sizeof(T) + (size_t)SW * 32 * TRI_R * sizeof(double) +
-         (size_t)SW * TRI_PIV * sizeof(float);
+struct alignas(16) TriSmem {
+  T stage[TRI_STAGE];           // the row's block values (a row of more than TRI_MR
+  T part[32 * TRI_MR];          //   scalars: up to the end of part); part: per block
+                                //   of the row (modulo 32), its product
+  // the factored pivot block and the reciprocals of its diagonal (tri_recip):
+  // up to TRI_MP rows of T, or up to TRI_MP / 2 rows of a tagged FP64 block
+  T lu[TRI_MP * (TRI_MP + 1)];
+  T ry[TRI_MP], rz[TRI_MP];
+};
+
+// The wait of one warp between two polls: a short sleep, the abort word and
+// the time budget every 16th poll.  False when the wait gave up.
+struct TriWait {
+  unsigned it = 0;
+  unsigned long long t0 = 0;
+  __device__ __forceinline__ bool pause(int* abort, unsigned long long limit, int* st) {
+    if (it == 0) t0 = global_ns();
+    ++it;
+    __nanosleep(32);
+    if ((it & 15) == 0) {
+      if (*((volatile int*)abort) != 0) return false;
+      if (global_ns() - t0 > limit) {
+        dev_fail(st, DEV_ETIMEOUT);
+        atomicExch(abort, 1);
+        return false;
+      }
+    }
+    return true;
+  }
+};
+
+// The first cnt (1 to TRI_XQ) values of a record into x; false while one of
+// them is still empty.
+template <typename TA>
+__device__ __forceinline__ bool tri_take(const double* p, int cnt, TA* x) {
+  bool ok = true;
+#pragma unroll
+  for (int q = 0; q < TRI_XQ; q += 2)
+    if (q < cnt) {
+      double a, b;
+      asm volatile("ld.relaxed.gpu.global.v2.f64 {%0, %1}, [%2];" : "=d"(a), "=d"(b) : "l"(p + q) : "memory");
+      ok = ok && tri_ready(a) && (q + 1 >= cnt || tri_ready(b));
+      x[q] = (TA)a;
+      x[q + 1] = (TA)b;
+    }
+  return ok;
+}
+__device__ __forceinline__ bool tri_take(const float* p, int cnt, float* x) {
+  bool ok = true;
+#pragma unroll
+  for (int q = 0; q < TRI_XQ; q += 4)
+    if (q < cnt) {
+      asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                   : "=f"(x[q]), "=f"(x[q + 1]), "=f"(x[q + 2]), "=f"(x[q + 3])
+                   : "l"(p + q)
+                   : "memory");
+#pragma unroll
+      for (int u = 0; u < 4; ++u) ok = ok && (q + u >= cnt || tri_ready(x[q + u]));
+    }
+  return ok;
 }
 
-// The calling warp's pivot-block buffer in the sweep's shared memory.
+// a / b correctly rounded from y = RN(1/b) and z, the rest of 1/b (tri_recip):
+// q0 = a y + a z is within one ulp of a / b, a - b q0 is exact, and the
+// correction by it rounds to RN(a / b) (Markstein's theorem; exact remainder
+// and correctly rounded reciprocal).  Four operations instead of a division's
+// 84 (FP32) or 560 (FP64) cycles.  Operands outside the range where no
+// intermediate can underflow or overflow (y = 0 marks such a b) are divided.
+__device__ __forceinline__ void tri_recip(float b, float& y, float& z) {
+  y = 0.f, z = 0.f;
+  if (fabsf(b) >= 0x1p-40f && fabsf(b) <= 0x1p40f) {
+    y = __frcp_rn(b);
+    z = __fmul_rn(__fmaf_rn(-b, y, 1.f), y);
+  }
+}
+__device__ __forceinline__ void tri_recip(double b, double& y, double& z) {
+  y = 0.0, z = 0.0;
+  if (fabs(b) >= 0x1p-300 && fabs(b) <= 0x1p300) {
+    y = __drcp_rn(b);
+    z = __dmul_rn(__fma_rn(-b, y, 1.0), y);
+  }
+}
+__device__ __forceinline__ double tri_div(double a, double b, double y, double z) {
+  const unsigned e = ((unsigned)__double2hiint(a) >> 20) & 0x7ff;  // |a| in [2^-300, 2^300): integer compares
+  if (__double2hiint(y) != 0 && e >= 1023 - 300 && e < 1023 + 300) {
+    const double q = __fma_rn(a, y, __dmul_rn(a, z));
+    return __fma_rn(__fma_rn(-b, q, a), y, q);
+  }
+  return __ddiv_rn(a, b);
+}
+
+// (double)v by integer operations (normal values; the conversion instruction
+// takes the FP64 unit).
+__device__ __forceinline__ double tri_widen(float v) {
+  const unsigned u = (unsigned)__float_as_int(v);
+  if ((u & 0x7f800000u) - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+  return (double)v;
+}
+__device__ __forceinline__ double tri_widen(double v) { return v; }
+
+// RN32(RN64(R - s)) for an FP64 R and an FP32 s by FP32 operations: R is held
+// as the exact sum h + m + l of three floats; t + e = h - s and f + e2 = t + w
+// exactly (Knuth's two-sum), w = e + m.  f is the answer when e2 and all that
+// was rounded or left out (2^-24 |w| + |l| + 2^-53 |f|, less than 2^-8 of half
+// an ulp of f under the two range conditions) stay within half an ulp, which
+// is not asked of a power of two.  Otherwise (one row in some hundred) the
+// FP64 unit is used: a subtraction between two conversions, 290 cycles on the
+// chain against 100.
+struct TriSplit {
+  float h, m, l;
+  bool ok;
+};
+__device__ __forceinline__ TriSplit tri_split(double R) {
+  TriSplit p;
+  p.h = (float)R;
+  const double d = R - (double)p.h;
+  p.m = (float)d;
+  p.l = (float)(d - (double)p.m);
+  p.ok = fabsf(p.h) >= 0x1p-40f && fabsf(p.h) <= 0x1p40f;
+  return p;
+}
+__device__ __forceinline__ float tri_sub32(double R, const TriSplit& p, float s, bool wanted) {
+  const float t = __fsub_rn(p.h, s);
+  const float tb = __fsub_rn(t, p.h);
+  const float e = __fadd_rn(__fsub_rn(p.h, __fsub_rn(t, tb)), __fsub_rn(-s, tb));
+  const float w = __fadd_rn(e, p.m);
+  const float f = __fadd_rn(t, w);
+  const float fb = __fsub_rn(f, t);
+  const float e2 = __fadd_rn(__fsub_rn(t, __fsub_rn(f, fb)), __fsub_rn(w, fb));
+  const unsigned u = (unsigned)__float_as_int(f);
+  const float lead = __int_as_float((int)(u & 0x7f800000u));  // 2^ef
+  const bool ok = p.ok && (u & 0x7fffffu) != 0 && fabsf(f) >= 0x1p-60f && fabsf(w) <= lead * 0x1p-10f &&
+                  fabsf(p.h) <= lead * 0x1p10f && fabsf(e2) <= lead * (0x1p-24f - 0x1p-32f);
+  return ok || !wanted ? f : (float)(R - (double)s);
+}
+
+// The block row that a warp works on.
 template <typename T>
-__device__ __forceinline__ float* tri_piv_buf(unsigned char* sm) {
-  return (float*)(sm + (size_t)SW * TRI_STAGE * sizeof(T) + (size_t)SW * 32 * TRI_R * sizeof(double)) +
-         (size_t)(threadIdx.x >> 5) * TRI_PIV;
+struct TriRow {
+  const int32_t* bcol;  // its blocks' columns and value offsets
+  const int64_t* voff;
+  const int32_t* csz;   // the matrix's column partition
+  const int64_t* coff;
+  int64_t v0;           // its first value
+  int nb, ni;           // blocks, scalar rows
+};
+
+// sum_b B_ib x_b of the calling warp's block row (ni <= G rows, G = 8 or 16),
+// row a's sum on lane a.  Lane l owns the blocks l, l + 32, ... of the row, in
+// units of up to TRI_XQ columns, and polls for its next two units; as soon as
+// some lanes' units have arrived, all lanes multiply those (G lanes to a
+// unit, one per row), so that when the last dependency arrives only its own
+// product is left.  The products are kept per owner lane, each element's
+// additions in the order of its blocks and columns, and then summed over the
+// owners as a butterfly over lane ^ 16, 8, 4, 2, 1 would.  An FP64 operation
+// occupies the unit of a warp's quarter of the SM for 64 cycles whatever the
+// number of lanes, so the additions of owners that do not exist (+0.0) are
+// left out there; the one effect they have, -0.0 becoming +0.0, is applied.
+template <int G, typename T, typename R>
+__device__ __forceinline__ bool tri_row(const TriRow<T>& row, const T* sval, const R* rec, T* part, int* abort,
+                                        unsigned long long limit, int* st, int lane, T* sum) {
+  const int nb = row.nb, ni = row.ni;
+  constexpr int NG = 32 / G;
+  const int g = lane / G, a = lane % G;
+  // the lane's units: the generator's block and column, then unit A and unit B
+  int gb = lane - 32, gq = 0, gnk = 0, gvo = 0;
+  const R* gx = rec;
+  auto next = [&](int& meta, int& vo, const R*& x) {
+    if (gq + TRI_XQ < gnk) {
+      gq += TRI_XQ;
+    } else {
+      gb += 32;
+      gq = 0;
+      gnk = 0;
+      if (gb < nb) {
+        const int32_t k = row.bcol[gb];
+        gnk = row.csz[k];
+        gvo = (int)(row.voff[gb] - row.v0);
+        gx = rec + tri_rec<R>(row.coff[k], k);
+      }
+    }
+    meta = gnk ? min(TRI_XQ, gnk - gq) | (gb < 32 && gq == 0 ? 16 : 0) | gnk << 8 : 0;
+    vo = gvo + gq;
+    x = gx + gq;
+  };
+  // a unit: its columns cnt, the block's columns nk, whether it opens its
+  // owner's sum, and its first value's place
+  int metaA, voA, metaB, voB;
+  bool okA = false, okB = false;
+  const R *pA, *pB;
+  T xA[TRI_XQ], xB[TRI_XQ];
+  next(metaA, voA, pA);
+  next(metaB, voB, pB);
+  int units = 0;  // of all lanes, still to come
+  for (int b = lane; b < nb; b += 32) units += (row.csz[row.bcol[b]] + TRI_XQ - 1) / TRI_XQ;
+  units = __reduce_add_sync(0xffffffffu, units);
+  TriWait w;
+  while (units > 0) {
+    if (metaA && !okA) okA = tri_take(pA, metaA & 15, xA);
+    if (metaB && !okB) okB = tri_take(pB, metaB & 15, xB);
+    const unsigned arrived = __ballot_sync(0xffffffffu, okA);
+    if (!arrived) {
+      const bool go = w.pause(abort, limit, st);
+      if (!__all_sync(0xffffffffu, go)) return false;
+      continue;
+    }
+    for (unsigned left = arrived; left;) {
+      unsigned mine = left;  // the group's owner: the g-th lowest lane left
+#pragma unroll
+      for (int j = 0; j < NG; ++j) {
+        if (j < g) mine &= mine - 1;
+        left &= left - 1;
+      }
+      const int o = mine ? __ffs(mine) - 1 : 0;
+      const int meta = __shfl_sync(0xffffffffu, metaA, o);
+      const int vo = __shfl_sync(0xffffffffu, voA, o);
+      const int cnt = mine != 0 && a < ni ? meta & 15 : 0;
+      const int nk = meta >> 8;
+      T acc = cnt && !(meta & 16) ? part[o * G + a] : (T)0;
+      const T* v = sval + vo + a * nk;
+      if constexpr (sizeof(T) == sizeof(double)) {
+        const int most = __reduce_max_sync(0xffffffffu, cnt);
+#pragma unroll
+        for (int q = 0; q < TRI_XQ; ++q) {
+          if (q >= most) break;
+          const T x = __shfl_sync(0xffffffffu, xA[q], o);
+          if (q < cnt) acc = fma(v[q], x, acc);
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < TRI_XQ; ++q) {
+          const T x = __shfl_sync(0xffffffffu, xA[q], o);
+          if (q < cnt) acc = fma(v[q], x, acc);
+        }
+      }
+      if (cnt) part[o * G + a] = acc;
+      __syncwarp();
+    }
+    units -= __popc(arrived);
+    if (units == 0) break;
+    if (okA) {
+#pragma unroll
+      for (int q = 0; q < TRI_XQ; ++q) xA[q] = xB[q];
+      metaA = metaB, voA = voB, pA = pB, okA = okB;
+      okB = false;
+      next(metaB, voB, pB);
+    }
+  }
+  // owners l = g + NG j in lane group g: j ^ (16 / NG) ... j ^ 1 within the
+  // lane, then g ^ (NG / 2) ... g ^ 1 by shuffles
+  constexpr int J = 32 / NG;
+  const int own = min(nb, 32);
+  T p[J];
+#pragma unroll
+  for (int j = 0; j < J; ++j) p[j] = a < ni && g + NG * j < own ? part[(g + NG * j) * G + a] : (T)0;
+  if constexpr (sizeof(T) == sizeof(double)) {
+    if (own <= 16) {
+#pragma unroll
+      for (int j = 0; j < J; ++j)
+        if (__double_as_longlong(p[j]) == (long long)0x8000000000000000ULL) p[j] = 0.0;
+    }
+#pragma unroll
+    for (int h = J / 2; h >= 1; h >>= 1)
+      if (own > h * NG) {
+#pragma unroll
+        for (int j = 0; j < h; ++j) p[j] = p[j] + p[j + h];
+      }
+#pragma unroll
+    for (int h = NG / 2; h >= 1; h >>= 1)
+      if (own > h) p[0] += __shfl_xor_sync(0xffffffffu, p[0], h * G);
+  } else {
+#pragma unroll
+    for (int h = J / 2; h >= 1; h >>= 1)
+#pragma unroll
+      for (int j = 0; j < h; ++j) p[j] = p[j] + p[j + h];
+#pragma unroll
+    for (int h = NG / 2; h >= 1; h >>= 1) p[0] += __shfl_xor_sync(0xffffffffu, p[0], h * G);
+  }
+  *sum = p[0];
+  return true;
+}
+
+// The row of up to TRI_MR scalars that is not the common one (9 rows or more,
+// or values that did not fit on chip): kept out of line, as are the large rows
+// and the larger pivot blocks below, so that the common row's code stays
+// small (inlined, they made it 1.5 times slower).
+template <typename T, typename R>
+__device__ __noinline__ bool tri_row16(TriRow<T> row, const T* sval, const R* rec, T* part, int* abort,
+                                       unsigned long long limit, int* st, int lane, T* sum) {
+  return tri_row<16>(row, sval, rec, part, abort, limit, st, lane, sum);
+}
+
+// s[t] -= sum_b B_ib x_b for the rows lane + 32 t of a block row of more than
+// TRI_MR scalars: FP64 sums in the order of the blocks and columns.  Every lane
+// polls its own block's first unknowns; the blocks are taken in their order,
+// each as soon as it has arrived.  xw: the FP64 unknowns, record k at
+// coff[k] (dense) or at tri_rec.
+template <typename T>
+__device__ __noinline__ bool tri_large(TriRow<T> row, const T* sval, const double* xw, bool dense, double* s,
+                                       int* abort, unsigned long long limit, int* st, int lane) {
+  const int nb = row.nb, ni = row.ni;
+  for (int base = 0; base < nb; base += 32) {
+    // lane l: block base + l, its first unknown and its values
+    int nk = 0, vo = 0;
+    const double* xk = nullptr;
+    if (base + lane < nb) {
+      const int32_t k = row.bcol[base + lane];
+      nk = row.csz[k];
+      vo = (int)(row.voff[base + lane] - row.v0);
+      xk = xw + (dense ? row.coff[k] : tri_rec<double>(row.coff[k], k));
+    }
+    // every lane polls its own block's first unknowns; the blocks are
+    // taken in their order, each as soon as it has arrived
+    double x[TRI_XQ];
+    bool ok = nk == 0;
+    TriWait w;
+    const int cnt = min(32, nb - base);
+    for (int b = 0; b < cnt;) {
+      if (!ok) {
+        ok = true;
+#pragma unroll
+        for (int q = 0; q < TRI_XQ; ++q)
+          if (q < nk) {
+            x[q] = tri_load(xk + q);
+            ok = ok && tri_ready(x[q]);
+          }
+        for (int q = TRI_XQ; q < nk; ++q) ok = ok && tri_ready(tri_load(xk + q));
+      }
+      const unsigned arrived = __ballot_sync(0xffffffffu, ok);
+      if (!(arrived >> b & 1)) {
+        const bool go = w.pause(abort, limit, st);
+        if (!__all_sync(0xffffffffu, go)) return false;
+        continue;
+      }
+      for (; b < cnt && (arrived >> b & 1); ++b) {
+        const int bk = __shfl_sync(0xffffffffu, nk, b), bv = __shfl_sync(0xffffffffu, vo, b);
+        const double* bx = (const double*)__shfl_sync(0xffffffffu, (unsigned long long)xk, b);
+        for (int q0 = 0; q0 < bk; q0 += TRI_XQ) {
+          T v[TRI_XQ];
+          double xq[TRI_XQ];
+#pragma unroll
+          for (int q = 0; q < TRI_XQ; ++q)
+            if (q0 + q < bk) xq[q] = q0 == 0 ? __shfl_sync(0xffffffffu, x[q], b) : tri_load(bx + q0 + q);
+#pragma unroll
+          for (int t = 0; t < TRI_R; ++t) {
+            if (32 * t >= ni) break;
+            const int a = lane + 32 * t;
+#pragma unroll
+            for (int q = 0; q < TRI_XQ; ++q)
+              if (a < ni && q0 + q < bk) v[q] = sval[bv + a * bk + q0 + q];
+#pragma unroll
+            for (int q = 0; q < TRI_XQ; ++q) {
+              if (q0 + q >= bk) break;
+              if (a < ni) s[t] = fma(-tri_widen(v[q]), xq[q], s[t]);
+            }
+          }
+        }
+      }
+    }
+  }
+  return true;
+}
+
+// Row stride of a staged pivot block of m rows.
+__device__ __forceinline__ int tri_stride(int m, bool f32) {
+  if (!f32) return m | 1;
+  return m <= 8 ? 8 : m <= 12 ? 12 : m <= 16 ? 16 : m <= 20 ? 20 : 32;
+}
+
+// U^{-1} L^{-1} P u of a staged FP32 pivot block of m <= M rows (row stride S,
+// a multiple of 4; the block is padded to M rows with those of the identity),
+// the operations of the sequential solve in their order: lane a holds u_a and
+// gets x_a, src is the lane's interchanged source row.  Every lane solves the
+// whole block in registers: its operations form one serial chain (each row of
+// U starts with the unknown found last), which no split shortens; the block's
+// entries come as broadcast 16-byte loads that do not depend on it.  The
+// padding adds -0.0 to the rows of the block, which changes none of them.
+// FAST divides as tri_div does; *ok tells whether all dividends were in its
+// range.
+template <int M, int S, bool FAST>
+__device__ __forceinline__ float tri_pivot_f32(const float* lu, const float* ry, const float* rz, int m, int src,
+                                               float u, int lane, bool* ok) {
+  const float up = __shfl_sync(0xffffffffu, u, src);
+  float x[M];
+#pragma unroll
+  for (int k = 0; k < M; ++k) x[k] = __shfl_sync(0xffffffffu, up, k);
+#pragma unroll
+  for (int i = 1; i < M; ++i) {
+#pragma unroll
+    for (int k4 = 0; k4 < i; k4 += 4) {
+      const float4 l = *reinterpret_cast<const float4*>(lu + i * S + k4);
+      const float lv[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+      for (int k = k4; k < i && k < k4 + 4; ++k) x[i] = __fmaf_rn(-lv[k - k4], x[k], x[i]);
+    }
+    if (i >= m) x[i] = 0.f;  // also where the block's unknowns are infinite
+  }
+  float lo = 1.f, hi = 1.f;
+#pragma unroll
+  for (int i = M - 1; i >= 0; --i) {
+#pragma unroll
+    for (int k4 = (i + 1) & ~3; k4 < M; k4 += 4) {
+      const float4 l = *reinterpret_cast<const float4*>(lu + i * S + k4);
+      const float lv[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+      for (int k = k4; k < M && k < k4 + 4; ++k)
+        if (k > i) x[i] = __fmaf_rn(-lv[k - k4], x[k], x[i]);
+    }
+    if (FAST) {
+      const float s = fabsf(x[i]), q = __fmaf_rn(x[i], ry[i], __fmul_rn(x[i], rz[i]));
+      if (i < m) lo = fminf(lo, s == s ? s : 0.f), hi = fmaxf(hi, s);
+      x[i] = __fmaf_rn(__fmaf_rn(-lu[i * S + i], q, x[i]), ry[i], q);
+      if (i >= m) x[i] = 0.f;
+    } else {
+      x[i] = i < m ? __fdiv_rn(x[i], lu[i * S + i]) : 0.f;
+    }
+  }
+  *ok = lo >= 0x1p-40f && hi <= 0x1p40f;
+  float r = x[0];
+#pragma unroll
+  for (int k = 1; k < M; ++k)
+    if (lane == k) r = x[k];
+  return r;
+}
+
+// The same in FP64, lane a with row a: L column by column over all rows at
+// once; in U the products with the newest unknown are formed for all rows at
+// once, so that only the subtractions of one row stay serial.  (An FP64
+// operation takes 64 cycles for one lane as for 32.)
+template <int M>
+__device__ __forceinline__ double tri_pivot_f64(const double* lu, const double* ry, const double* rz, int m, int S,
+                                                int src, double u, int lane) {
+  double y = __shfl_sync(0xffffffffu, u, src);
+  const double* row = lu + (lane < m ? lane : 0) * S;
+  double prod[M];  // k < a: l_ak, k >= a: u_ak, then its product with x_k
+#pragma unroll
+  for (int k = 0; k < M; ++k) prod[k] = k < m ? row[k] : 0.0;
+  const double d = lu[(lane < m ? lane : 0) * (S + 1)], dy = ry[lane < m ? lane : 0], dz = rz[lane < m ? lane : 0];
+#pragma unroll
+  for (int k = 0; k + 1 < M; ++k)
+    if (k + 1 < m) {
+      const double yk = __shfl_sync(0xffffffffu, y, k);
+      if (lane > k && lane < m) y = __dsub_rn(y, __dmul_rn(prod[k], yk));
+    }
+#pragma unroll
+  for (int i = M - 1; i >= 0; --i)
+    if (i < m) {
+      if (lane == i) {
+#pragma unroll
+        for (int k = i + 1; k < M; ++k)
+          if (k < m) y = __dsub_rn(y, prod[k]);
+        y = tri_div(y, d, dy, dz);
+      }
+      const double x = __shfl_sync(0xffffffffu, y, i);
+      if (lane < i) prod[i] = __dmul_rn(prod[i], x);
+    }
+  return y;
+}
+
+// The FP64 solve for m <= TRI_MP rows, in loops; the products take the place
+// of the entries above the diagonal in shared memory.
+__device__ __noinline__ double tri_pivot_f64_wide(double* lu, const double* ry, const double* rz, int m, int S,
+                                                     int src, double u, int lane) {
+  double y = __shfl_sync(0xffffffffu, u, src);
+  for (int k = 0; k + 1 < m; ++k) {
+    const double yk = __shfl_sync(0xffffffffu, y, k);
+    if (lane > k && lane < m) y = __dsub_rn(y, __dmul_rn(lu[lane * S + k], yk));
+  }
+  for (int i = m - 1; i >= 0; --i) {
+    if (lane == i) {
+#pragma unroll 4
+      for (int k = i + 1; k < m; ++k) y = __dsub_rn(y, lu[i * S + k]);
+      y = tri_div(y, lu[i * S + i], ry[i], rz[i]);
+    }
+    const double x = __shfl_sync(0xffffffffu, y, i);
+    if (lane < i) lu[lane * S + i] = __dmul_rn(lu[lane * S + i], x);
+    __syncwarp();
+  }
+  return y;
+}
+
+// The FP32 solve for m <= TRI_MP rows; fast: every diagonal entry has its
+// reciprocal (tri_recip).
+template <int M, int S>
+__device__ __forceinline__ float tri_pivot_any(const float* lu, const float* ry, const float* rz, int m, int src,
+                                               bool fast, float u, int lane) {
+  bool ok;
+  if (fast) {
+    const float x = tri_pivot_f32<M, S, true>(lu, ry, rz, m, src, u, lane, &ok);
+    if (ok) return x;
+  }
+  return tri_pivot_f32<M, S, false>(lu, ry, rz, m, src, u, lane, &ok);
+}
+__device__ __noinline__ float tri_pivot_f32_wide(const float* lu, const float* ry, const float* rz, int m, int src,
+                                                 bool fast, float u, int lane) {
+  return m <= 8    ? tri_pivot_any<8, 8>(lu, ry, rz, m, src, fast, u, lane)
+         : m <= 12 ? tri_pivot_any<12, 12>(lu, ry, rz, m, src, fast, u, lane)
+         : m <= 16 ? tri_pivot_any<16, 16>(lu, ry, rz, m, src, fast, u, lane)
+         : m <= 20 ? tri_pivot_any<20, 20>(lu, ry, rz, m, src, fast, u, lane)
+                   : tri_pivot_any<32, 32>(lu, ry, rz, m, src, fast, u, lane);
 }
 
 // Sync-free block triangular sweep over the last-level factors, one warp per
 // block row, rows handed out in level order (order[ticket]): every dependency
 // of a row sits in an earlier level and so holds an earlier ticket.
-//   forward  (BWD = false): y_i <- y_i - sum_{k<i} L_ik y_k        (in place)
+//   forward  (BWD = false): y_i <- r_i g_i - sum_{k<i} L_ik y_k
+//                           (rhs g, scl r; y to out and the records)
 //   backward (BWD = true):  x_i <- D_i^{-1} (y_i - sum_{j>i} U_ij x_j)
-//                           (rows flagged in fixed keep the x_i in out)
-// Rows of up to TRI_MR scalars: the row's block values (static) are staged in
-// shared memory before any wait; every lane then owns some blocks of the row,
-// waits for its own dependency, loads that dependency's values in one batch
-// and accumulates its products privately; a warp reduction forms the update.
-// The row's latency is its slowest dependency plus one batched load and a
-// reduction.  Larger rows use lanes over scalar rows.
-template <typename T, bool BWD>
-__global__ void __launch_bounds__(SW * 32)
+//                           (rhs y; x to the records, c_i x_i to out, scl c;
+//                           rows flagged in fixed take x_i = fixv_i / c_i)
+// rec: the records; dbl: the FP64 unknowns (R = float; forward: out).  Both
+// start as 0xff bytes.  Rows of up to TRI_MR scalars: everything static (the
+// row's values, the pivot LU, its interchanges and its diagonal's
+// reciprocals) is on chip before the first poll; then tri_row.  Larger rows
+// (FP64 sums, block by block) use a lane per scalar row.
+//
+// Bound: the levels of the dependency DAG times the latency of a link.  A
+// publication reaches a poller in 0.53 us; a link's own work is then about
+// 0.35 us forward and 0.8 us backward in FP32 (products of the last arrival
+// 330 cycles, sum over the owners 160, subtraction 100, pivot solve 700), and
+// several times that in FP64, whose operations take 64 cycles each.  One
+// application, with flags, fences and one-lane pivot solves before and now:
+// 3.0 million unknowns FP32 (2 650 levels each way) 34.9 and 11.6 ms; 48 000
+// unknowns at tau 0.9 FP32 (5 100 and 6 190 levels) 60.6 and 17.1 ms; 360 000
+// unknowns FP64 (1 930 levels) 51.8 and 15.6 ms; 18 000 FP64 10.2 and 3.3 ms.
+template <typename T, bool BWD, typename R>
+__global__ void __launch_bounds__(TRI_W * 32, TRI_B)
     k_tri(VBView<T> M, const int64_t* __restrict__ dgoff, const double* __restrict__ lu64,
           const float* __restrict__ lu32, const int32_t* __restrict__ ptag, const int32_t* __restrict__ piv,
-          const double* __restrict__ rhs, double* __restrict__ out, const int32_t* __restrict__ order,
-          int32_t* __restrict__ done, unsigned long long* ticket, int* abort, unsigned long long wait_limit,
-          int* st, const int32_t* __restrict__ fixed) {
+          const double* __restrict__ rhs, const double* __restrict__ scl, R* rec, double* dbl, double* out,
+          const int32_t* __restrict__ order, unsigned long long* ticket, int* abort, unsigned long long wait_limit,
+          int* st, const int32_t* __restrict__ fixed, const double* __restrict__ fixv) {
   extern __shared__ __align__(16) unsigned char tri_sm[];
-  T* stage = (T*)tri_sm + (size_t)(threadIdx.x >> 5) * TRI_STAGE;
-  double* sv = (double*)(tri_sm + (size_t)SW * TRI_STAGE * sizeof(T)) + (size_t)(threadIdx.x >> 5) * 32 * TRI_R;
   const int lane = threadIdx.x & 31;
+  TriSmem<T>& sm = reinterpret_cast<TriSmem<T>*>(tri_sm)[threadIdx.x >> 5];
+  // the finished unknown a of row i, whose scalars start at r0
+  auto publish = [&](int64_t i, int64_t r0, int a, double x, double sc) {
+    R* ri = rec + tri_rec<R>(r0, i);
+    if constexpr (std::is_same<R, float>::value) tri_publish(ri + a, (float)x);
+    if constexpr (std::is_same<R, double>::value) tri_publish(ri + a, x);
+    if (std::is_same<R, float>::value) tri_publish(dbl + r0 + a, x);
+    if (BWD)
+      out[r0 + a] = __dmul_rn(sc, x);
+    else if (std::is_same<R, double>::value)
+      out[r0 + a] = x;
+  };
   for (;;) {
     long long t0 = 0;
     if (lane == 0) t0 = (long long)atomicAdd(ticket, 1ULL);
     t0 = __shfl_sync(0xffffffffu, t0, 0);
     if (t0 >= M.nbr) break;
     const int64_t i = order[t0];
-    if (BWD && fixed && fixed[i]) {  // the caller gave this row's unknowns (already in out)
-      if (lane == 0) atomicExch(&done[i], 1);
-      continue;
-    }
     const int ni = M.rsz[i];
     const int64_t r0 = M.roff[i];
-    bool failed = false;
-    // backward sweep, FP32 pivot block of at most 8 rows: the pivot LU and its
-    // interchanges are static, so they come into shared memory before the
-    // waits below and the final solve reads them on chip
-    if (BWD && lu32 && ni <= 8 && !ptag[i]) {
-      float* slu = tri_piv_buf<T>(tri_sm);
-      const int64_t lo = dgoff[i];
-      for (int e = lane; e < ni * ni; e += 32) slu[e] = lu32[lo + e];
-      if (lane < ni) reinterpret_cast<int32_t*>(slu + 64)[lane] = piv[r0 + lane];
+    if (BWD && fixed && fixed[i]) {  // the caller gave this row's unknowns
+      for (int a = lane; a < ni; a += 32) publish(i, r0, a, __ddiv_rn(fixv[r0 + a], scl[r0 + a]), scl[r0 + a]);
+      continue;
     }
-    if (ni <= TRI_MR) {
-      const int64_t b0 = M.bptr[i], b1 = M.bptr[i + 1];
-      const int64_t v0 = M.voff[b0];
-      const int64_t nv = M.voff[b1] - v0;
-      const bool staged = nv <= TRI_STAGE;
-      if (staged) {
-#pragma unroll 4
-        for (int64_t e = lane; e < nv; e += 32) stage[e] = M.val[v0 + e];
+    const int64_t b0 = M.bptr[i], b1 = M.bptr[i + 1];
+    const int nb = (int)(b1 - b0);
+    // the pivot block: applied in FP32 (f32p) or FP64, from shared memory (sp)
+    const bool f32p = BWD && lu32 && !ptag[i];
+    const int S = tri_stride(ni, f32p);
+    const bool sp = BWD && ni <= (f32p || sizeof(T) == sizeof(double) ? TRI_MP : TRI_MP / 2);
+    int src = lane;     // interchanged source row
+    bool fast = false;  // every diagonal entry of the FP32 block has its reciprocal
+    if (sp) {
+      const int64_t lo = dgoff[i];
+      if (f32p) {
+        for (int e = lane; e < S * S; e += 32) {
+          const int a = e / S, c = e - a * S;
+          reinterpret_cast<float*>(sm.lu)[e] = a < ni && c < ni ? lu32[lo + a * ni + c] : a == c ? 1.f : 0.f;
+        }
+      } else {
+        for (int e = lane; e < ni * ni; e += 32) {
+          const int a = e / ni;
+          reinterpret_cast<double*>(sm.lu)[a * S + (e - a * ni)] = lu64[lo + e];
+        }
       }
-      const double r_self = lane < ni ? rhs[r0 + lane] : 0.0;
+      const int pv = lane < ni ? piv[r0 + lane] : lane;
+      for (int k = 0; k < ni; ++k) {
+        const int pk = __shfl_sync(0xffffffffu, pv, k);
+        const int vk = __shfl_sync(0xffffffffu, src, k), vp = __shfl_sync(0xffffffffu, src, pk & 31);
+        if (lane == k) src = vp;
+        if (lane == pk) src = vk;
+      }
       __syncwarp();
-      // FP32 factors are applied in FP32 (the products and their sums), FP64
-      // ones in FP64; the row's result is formed in FP64
-      using TA = typename std::conditional<sizeof(T) == sizeof(float), float, double>::type;
-      TA part[TRI_MR];
-#pragma unroll
-      for (int a = 0; a < TRI_MR; ++a) part[a] = 0.0;
-      for (int64_t b = b0 + lane; b < b1; b += 32) {
-        const int32_t k = M.bcol[b];
-        const int nk = M.csz[k];
-        const T* v = staged ? stage + (M.voff[b] - v0) : M.val + M.voff[b];
-        if (!wait_row(done, k, abort, wait_limit, st)) {
-          failed = true;
-          break;
-        }
-        const double* xk = out + M.coff[k];
-        for (int q0 = 0; q0 < nk; q0 += TRI_XQ) {
-          TA xq[TRI_XQ];
-#pragma unroll
-          for (int q = 0; q < TRI_XQ; ++q) xq[q] = q0 + q < nk ? (TA)__ldcg(xk + q0 + q) : (TA)0;
-#pragma unroll
-          for (int q = 0; q < TRI_XQ; ++q) {
-            if (q0 + q >= nk) break;
-#pragma unroll
-            for (int a = 0; a < TRI_MR; ++a)
-              if (a < ni) part[a] = fma((TA)v[a * nk + q0 + q], xq[q], part[a]);
-          }
-        }
+      if (f32p) {
+        float y = 1.f, z = 0.f;
+        if (lane < ni) tri_recip(reinterpret_cast<float*>(sm.lu)[lane * (S + 1)], y, z);
+        reinterpret_cast<float*>(sm.ry)[lane] = y;
+        reinterpret_cast<float*>(sm.rz)[lane] = z;
+        fast = __all_sync(0xffffffffu, y != 0.f);
+      } else if (lane < ni) {
+        double y, z;
+        tri_recip(reinterpret_cast<double*>(sm.lu)[lane * (S + 1)], y, z);
+        reinterpret_cast<double*>(sm.ry)[lane] = y;
+        reinterpret_cast<double*>(sm.rz)[lane] = z;
       }
-      failed = __any_sync(0xffffffffu, failed);
-#pragma unroll
-      for (int a = 0; a < TRI_MR; ++a)
-        for (int o = 16; o > 0; o >>= 1) part[a] += __shfl_xor_sync(0xffffffffu, part[a], o);
-      if (!failed && lane < ni) {
-        double sa = 0.0;
-#pragma unroll
-        for (int a = 0; a < TRI_MR; ++a)
-          if (a == lane) sa = part[a];
-        sv[lane] = r_self - sa;
-      }
-    } else {
-      double s[TRI_R];
-#pragma unroll
-      for (int t = 0; t < TRI_R; ++t) s[t] = lane + 32 * t < ni ? rhs[r0 + lane + 32 * t] : 0.0;
-      if (ni > 32 * TRI_R) {
-        if (lane == 0) dev_fail(st, DEV_INTERNAL);
-        failed = true;
-      }
-      for (int64_t b = M.bptr[i]; b < M.bptr[i + 1] && !failed; ++b) {
-        const int32_t k = M.bcol[b];
-        bool ok = true;
-        if (lane == 0) ok = wait_row(done, k, abort, wait_limit, st);
-        failed = !__shfl_sync(0xffffffffu, ok, 0);
-        if (failed) break;
-        const int nk = M.csz[k];
-        const double* xk = out + M.coff[k];
-#pragma unroll
-        for (int t = 0; t < TRI_R; ++t) {
-          const int a = lane + 32 * t;
-          if (a < ni) {
-            const T* v = M.val + M.voff[b] + (int64_t)a * nk;
-            for (int q = 0; q < nk; ++q) s[t] = fma(-ld(v + q), __ldcg(xk + q), s[t]);
-          }
-        }
-      }
-#pragma unroll
-      for (int t = 0; t < TRI_R; ++t)
-        if (!failed && lane + 32 * t < ni) sv[lane + 32 * t] = s[t];
+    }
+    const int64_t v0 = M.voff[b0];
+    const int64_t nv = M.voff[b1] - v0;
+    const bool staged = nv <= TRI_STAGE + (ni > TRI_MR ? 32 * TRI_MR : 0);
+    if (staged) {
+#pragma unroll 4
+      for (int64_t e = lane; e < nv; e += 32) sm.stage[e] = M.val[v0 + e];
+    }
+    const T* sval = staged ? sm.stage : M.val + v0;
+    const TriRow<T> row{M.bcol + b0, M.voff + b0, M.csz, M.coff, v0, nb, ni};
+    double u = 0.0, sc = 0.0;  // lane a: row a's unknown, its scale
+    if (lane < ni) {
+      sc = scl[r0 + lane];
+      u = BWD ? rhs[r0 + lane] : __dmul_rn(sc, rhs[r0 + lane]);
     }
     __syncwarp();
-    if (!failed) {
+    TriSplit us{0.f, 0.f, 0.f, false};
+    constexpr bool narrow = std::is_same<R, float>::value;
+    if constexpr (narrow) us = tri_split(u);
+    float uf = 0.f;   // u rounded to FP32 (FP32 records)
+    double s[TRI_R];  // rows lane + 32 t of a large row
+    if (ni <= TRI_MR) {
+      // FP32 factors are applied in FP32 (the products and their sums), FP64
+      // ones in FP64; the row's result is formed in FP64
+      T sa;
+      const bool ok = ni <= 8 && staged
+                          ? tri_row<8>(row, sm.stage, rec, sm.part, abort, wait_limit, st, lane, &sa)
+                          : tri_row16<T, R>(row, sval, rec, sm.part, abort, wait_limit, st, lane, &sa);
+      if (!ok) return;
+      if constexpr (narrow) uf = tri_sub32(u, us, sa, lane < ni);
+      if (!narrow || (BWD && !f32p)) u = lane < ni ? u - (double)sa : 0.0;
+      if constexpr (narrow && !BWD) {  // the record first: the FP64 unknown is not on the chain
+        if (lane < ni) {
+          tri_publish(rec + tri_rec<R>(r0, i) + lane, uf);
+          tri_publish(dbl + r0 + lane, u - (double)sa);
+        }
+        __syncwarp();  // the staged data is read no more
+        continue;
+      }
+    } else {
+      if (ni > 32 * TRI_R) {
+        if (lane == 0) {
+          dev_fail(st, DEV_INTERNAL);
+          atomicExch(abort, 1);
+        }
+        return;
+      }
+      s[0] = u;
+#pragma unroll
+      for (int t = 1; t < TRI_R; ++t) {
+        const int64_t q = r0 + lane + 32 * t;
+        s[t] = lane + 32 * t < ni ? (BWD ? rhs[q] : __dmul_rn(scl[q], rhs[q])) : 0.0;
+      }
+      const bool dense = std::is_same<R, float>::value;
+      if (!tri_large<T>(row, sval, dense ? dbl : (const double*)rec, dense, s, abort, wait_limit, st, lane)) return;
+      u = s[0];
+    }
+    if (ni <= TRI_MP && (!BWD || sp)) {
+      if (BWD) {
+        if (f32p) {
+          if (!narrow || ni > TRI_MR) uf = (float)u;
+          if constexpr (sizeof(T) == sizeof(float)) {  // FP32 pivot blocks belong to FP32 factors only
+            bool ok = false;
+            float x = 0.f;
+            if (ni <= 6 && fast) x = tri_pivot_f32<6, 8, true>(sm.lu, sm.ry, sm.rz, ni, src, uf, lane, &ok);
+            if (!ok) x = tri_pivot_f32_wide(sm.lu, sm.ry, sm.rz, ni, src, fast, uf, lane);
+            if constexpr (narrow)
+              if (lane < ni) tri_publish(rec + tri_rec<R>(r0, i) + lane, x);
+            u = (double)x;
+          }
+        } else {
+          double* l = reinterpret_cast<double*>(sm.lu);
+          const double* ry = reinterpret_cast<const double*>(sm.ry);
+          const double* rz = reinterpret_cast<const double*>(sm.rz);
+          u = sizeof(T) == sizeof(double) && ni <= 8 ? tri_pivot_f64<8>(l, ry, rz, ni, S, src, u, lane)
+                                                     : tri_pivot_f64_wide(l, ry, rz, ni, S, src, u, lane);
+        }
+      }
+      if (lane < ni) publish(i, r0, lane, u, sc);
+    } else {  // pivot blocks of more than TRI_MP rows: one lane
+      double* sv = reinterpret_cast<double*>(sm.part);
+#pragma unroll
+      for (int t = 0; t < TRI_R; ++t)
+        if (lane + 32 * t < ni) sv[lane + 32 * t] = ni <= TRI_MR ? u : s[t];
+      __syncwarp();
       if (BWD && lane == 0) {
-        if (lu32 && ni <= 8 && !ptag[i]) {  // the pivot block staged on chip before the waits
-          const float* slu = tri_piv_buf<T>(tri_sm);
-          pivot_solve_f32(slu, reinterpret_cast<const int32_t*>(slu + 64), ni, sv);
-        } else if (lu32 && !ptag[i] && ni <= 32) {
-          pivot_solve_f32(lu32 + dgoff[i], piv + r0, ni, sv);
-        } else if (lu32 && !ptag[i]) {
+        if (f32p) {
           pivot_forward<float>(lu32 + dgoff[i], piv + r0, ni, sv);
           pivot_backward<float>(lu32 + dgoff[i], ni, sv);
         } else {
@@ -339,11 +897,9 @@ __global__ void __launch_bounds__(SW * 32)
         }
       }
       __syncwarp();
-      for (int a = lane; a < ni; a += 32) out[r0 + a] = sv[a];
+      for (int a = lane; a < ni; a += 32) publish(i, r0, a, sv[a], scl[r0 + a]);
     }
-    __threadfence();  // every lane's writes before the flag
-    __syncwarp();
-    if (lane == 0) atomicExch(&done[i], failed ? 2 : 1);
+    __syncwarp();  // the staged data is read no more
   }
 }
 
@@ -510,8 +1066,15 @@ void tri_attributes() {
   int dev = 0;
   VB_CUDA(cudaGetDevice(&dev));
   if (dev >= 0 && dev < 64 && set_on[dev]) return;
-  VB_CUDA(cudaFuncSetAttribute(k_tri<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_smem<T>()));
-  VB_CUDA(cudaFuncSetAttribute(k_tri<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_smem<T>()));
+  auto opt_in = [](auto kernel) {
+    VB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TRI_W * sizeof(TriSmem<T>))));
+  };
+  opt_in(k_tri<T, false, double>);
+  opt_in(k_tri<T, true, double>);
+  if constexpr (sizeof(T) == sizeof(float)) {
+    opt_in(k_tri<T, false, float>);
+    opt_in(k_tri<T, true, float>);
+  }
   if (dev >= 0 && dev < 64) set_on[dev] = true;
 }
 
@@ -529,9 +1092,12 @@ void PrecDev<T>::prepare_apply() {
     if (M.nf > 0) make_rowblk(L.W.nbr, L.W.roff.p, M.nf, M.wrow, s);
   }
   nlast = last.A.nbr ? last.A.nrows_scalar(s) : 0;
-  total += 2 * nlast;
   work.alloc(std::max<int64_t>(total, 1), s);
-  flags.alloc(2 * std::max<int64_t>(last.A.nbr, 1), s);
+  // the sweeps' records and FP64 unknowns, cleared together: FP32 records
+  // twice, y and x, or FP64 records twice and y
+  const bool narrow = sizeof(T) == sizeof(float);
+  rec_bytes = narrow ? rec_words<float>(nlast, last.A.nbr) * 4 : rec_words<double>(nlast, last.A.nbr) * 8;
+  rec.alloc(2 * rec_bytes + (narrow ? 2 : 1) * nlast * 8 + 16, s);
   tick.alloc(2, s);
   abort_flag.alloc(1, s);
   int dev = 0;
@@ -550,9 +1116,12 @@ struct SolveBufs {
   const int64_t* grow[kMaxLev]; // scalar row -> block row of G
   const int64_t* wrow[kMaxLev]; // scalar row -> block row of W
   double* fv[kMaxLev + 1];      // fixed values per level (fv[0]: the caller's)
-  double* yy;                   // last level: S_1 g, then L^{-1} S_1 g
-  double* xx;                   // last level: U^{-1} L^{-1} S_1 g
-  int32_t* flags;               // 2 p_last completion flags
+  double* yy;                   // last level: L^{-1} S_1 g
+  void* recf;                   // records of the forward sweep
+  void* recb;                   // records of the backward sweep (may be recf)
+  double* xx;                   // FP32 records: the FP64 unknowns of the backward sweep (else NULL)
+  void* clear;                  // what starts as 0xff bytes: recf, and all else but a recb that is recf
+  size_t clear_bytes;
   unsigned long long* tick;     // 2 tickets
   int* abort;
   int nsm;
@@ -568,13 +1137,28 @@ __global__ void k_fix_down(int64_t n, const int32_t* __restrict__ sp, const doub
   }
 }
 
-// Last level: the fixed rows' unknowns before the column scaling.
-__global__ void k_fix_last(int64_t p, const int64_t* __restrict__ roff, const int32_t* __restrict__ fixed,
-                           const double* __restrict__ fv, const double* __restrict__ c, double* __restrict__ xx) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p; i += (int64_t)gridDim.x * blockDim.x) {
-    if (!fixed[i]) continue;
-    for (int64_t q = roff[i]; q < roff[i + 1]; ++q) xx[q] = __ddiv_rn(fv[q], c[q]);
-  }
+// The last level's two sweeps: z = S2 (L U)^{-1} S1 g, with records of type R.
+template <typename T, typename R>
+void sweep_last(const PrecDev<T>& P, const SolveBufs& B, const double* g, double* z, int64_t n, const int32_t* fixed,
+                const double* fixv) {
+  cudaStream_t s = P.s;
+  const auto& last = P.last;
+  const int64_t p = last.A.nbr;
+  // the buffers keep the previous call's contents
+  VB_CUDA(cudaMemsetAsync(B.clear, 0xff, B.clear_bytes, s));
+  VB_CUDA(cudaMemsetAsync(B.tick, 0, 2 * sizeof(unsigned long long), s));
+  VB_CUDA(cudaMemsetAsync(B.abort, 0, sizeof(int), s));
+  const unsigned nb =
+      (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)B.nsm * TRI_B, (p + TRI_W - 1) / TRI_W));
+  const size_t smem = TRI_W * sizeof(TriSmem<T>);
+  launch(k_tri<T, false, R>, nb, TRI_W * 32, smem, s, last.L.view(), nullptr, nullptr, nullptr, nullptr, nullptr, g,
+         last.r.p, (R*)B.recf, B.yy, B.yy, last.lorder.p, B.tick, B.abort, (unsigned long long)P.wait_limit,
+         P.status.p, nullptr, nullptr);
+  if (B.recb == B.recf) VB_CUDA(cudaMemsetAsync(B.recb, 0xff, rec_words<R>(n, p) * sizeof(R), s));
+  launch(k_tri<T, true, R>, nb, TRI_W * 32, smem, s, last.U.view(), last.Dg.voff.p, last.Dg.val.p,
+         sizeof(T) == sizeof(float) ? last.Dg32.val.p : nullptr, last.ptag.p, last.piv.p, B.yy, last.c.p, (R*)B.recb,
+         B.xx, z, last.uorder.p, B.tick + 1, B.abort, (unsigned long long)P.wait_limit, P.status.p, fixed, fixv);
+  VB_LAUNCH_CHECK();
 }
 
 // Alg. 2 over all levels, in the factorization's own numbering; enqueues
@@ -612,24 +1196,14 @@ void solve_core(const PrecDev<T>& P, const double* in, double* out, const SolveB
     const double* g = nl == 0 ? in : B.bh[nl - 1] + P.maps[nl - 1].nf;
     double* z = nl == 0 ? out : B.xh[nl - 1] + P.maps[nl - 1].nf;
     if (nl_last) {
-      launch(k_mul, grid_for(nl_last, 256), 256, 0, s, nl_last, last.r.p, g, B.yy);
-      const int64_t p = last.A.nbr;
-      const int32_t* fixed = fixv ? last.fixed.p : nullptr;
-      if (fixed)
-        launch(k_fix_last, grid_for(p, 256), 256, 0, s, p, last.A.roff.p, fixed, nl == 0 ? fixv : B.fv[nl],
-               last.c.p, B.xx);
-      // the buffers keep the previous call's contents: clear what starts at 0
-      VB_CUDA(cudaMemsetAsync(B.flags, 0, 2 * p * sizeof(int32_t), s));
-      VB_CUDA(cudaMemsetAsync(B.tick, 0, 2 * sizeof(unsigned long long), s));
-      VB_CUDA(cudaMemsetAsync(B.abort, 0, sizeof(int), s));
-      const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)B.nsm * 2, (p + SW - 1) / SW));
-      launch(k_tri<T, false>, nb, SW * 32, tri_smem<T>(), s, last.L.view(), nullptr, nullptr, nullptr, nullptr,
-             nullptr, B.yy, B.yy, last.lorder.p, B.flags, B.tick, B.abort, (unsigned long long)P.wait_limit,
-             P.status.p, nullptr);
-      launch(k_tri<T, true>, nb, SW * 32, tri_smem<T>(), s, last.U.view(), last.Dg.voff.p, last.Dg.val.p,
-             mixed ? last.Dg32.val.p : nullptr, last.ptag.p, last.piv.p, B.yy, B.xx, last.uorder.p, B.flags + p,
-             B.tick + 1, B.abort, (unsigned long long)P.wait_limit, P.status.p, fixed);
-      launch(k_mul, grid_for(nl_last, 256), 256, 0, s, nl_last, last.c.p, B.xx, z);
+      if constexpr (sizeof(T) == sizeof(float)) {
+        if (B.xx)
+          sweep_last<T, float>(P, B, g, z, nl_last, fixv ? last.fixed.p : nullptr, nl == 0 ? fixv : B.fv[nl]);
+        else
+          sweep_last<T, double>(P, B, g, z, nl_last, fixv ? last.fixed.p : nullptr, nl == 0 ? fixv : B.fv[nl]);
+      } else {
+        sweep_last<T, double>(P, B, g, z, nl_last, fixv ? last.fixed.p : nullptr, nl == 0 ? fixv : B.fv[nl]);
+      }
       VB_LAUNCH_CHECK();
     }
   }
@@ -681,8 +1255,13 @@ void PrecDev<T>::apply_fixed(const double* x, double* y, const double* fixv) {
     B.grow[l] = maps[l].grow.p;
     B.wrow[l] = maps[l].wrow.p;
   }
-  B.yy = wp;
-  B.xx = wp + nlast;
+  const bool narrow = sizeof(T) == sizeof(float);
+  B.recf = rec.p;
+  B.recb = rec.p + rec_bytes;
+  B.yy = (double*)(rec.p + 2 * rec_bytes);
+  B.xx = narrow ? B.yy + nlast : nullptr;
+  B.clear = rec.p;
+  B.clear_bytes = 2 * rec_bytes + (narrow ? 2 : 0) * nlast * 8;
   if (fixv) {
     const int64_t nf = fixed_work(*this);
     if ((int64_t)fwork.n < nf) fwork.alloc(std::max<int64_t>(nf, 1), s);
@@ -692,7 +1271,6 @@ void PrecDev<T>::apply_fixed(const double* x, double* y, const double* fixv) {
       fp += maps[l].n - maps[l].nf;
     }
   }
-  B.flags = flags.p;
   B.tick = tick.p;
   B.abort = abort_flag.p;
   B.nsm = nsm;
@@ -701,13 +1279,15 @@ void PrecDev<T>::apply_fixed(const double* x, double* y, const double* fixv) {
 
 // ---- the same solve with caller-provided scratch (no allocation) ----------
 // Layout of the scratch, each piece 256-byte aligned: the permuted x and y
-// (n doubles each), the per-level work vectors (2 n_l doubles each), the
-// last-level vectors (2 n_last doubles), the row->block maps of G and W
-// (n_l int64 per level), the last-level flags (2 p_last int32), two tickets,
-// the abort word, and (factorizations with fixed rows) the fixed-value work.
+// (n doubles each), the records of the sweeps (both use the same n_last +
+// p_last doubles, in turn: p_last doubles, then the first n_last doubles of
+// the next piece), the work vectors (n_last doubles of records, then the
+// last level's y, then 2 n_l doubles per level), the row->block maps of G and
+// W (n_l int64 per level), two tickets, the abort word, and (factorizations
+// with fixed rows) the fixed-value work.
 namespace {
 struct ScratchPlan {
-  size_t xp, yp, work, maps, flags, tick, abort, fwork, total;
+  size_t xp, yp, rec, work, maps, tick, abort, fwork, total;
 };
 
 inline size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -727,12 +1307,12 @@ ScratchPlan plan_scratch(const PrecDev<T>& P) {
   o = align256(o + (size_t)P.n * 8);
   sp.yp = o;
   o = align256(o + (size_t)P.n * 8);
+  sp.rec = o;
+  o = align256(o + (size_t)P.last.A.nbr * 8);
   sp.work = o;
   o = align256(o + (size_t)nwork * 8);
   sp.maps = o;
   o = align256(o + (size_t)nmap * 8);
-  sp.flags = o;
-  o = align256(o + (size_t)(2 * P.last.A.nbr) * 4);
   sp.tick = o;
   o = align256(o + 2 * 8);
   sp.abort = o;
@@ -766,10 +1346,16 @@ void PrecDev<T>::solve_scratch(const double* x, double* y, unsigned char* scratc
   const int nl = (int)lev.size();
   if (nl > kMaxLev) fail(VB_EINVAL, "more than 64 levels");
   if (fixv && !last.fixed.p) fail(VB_EINVAL, "the factorization has no fixed rows");
-  double* wp = (double*)(scratch + sp.work);
+  const int64_t nl_last = maps.empty() ? n : maps.back().n - maps.back().nf;
+  double* wp = (double*)(scratch + sp.work) + nl_last;  // its first n_last doubles belong to the records
   int64_t* mp = (int64_t*)(scratch + sp.maps);
   double* fp = (double*)(scratch + sp.fwork);
   SolveBufs B{};
+  // FP64 records, shared by the two sweeps: no more scratch than their flags took
+  B.recf = B.recb = B.clear = scratch + sp.rec;
+  B.clear_bytes = rec_words<double>(nl_last, last.A.nbr) * 8;
+  B.yy = wp;
+  wp += nl_last;
   for (int l = 0; l < nl; ++l) {
     B.bh[l] = wp;
     wp += maps[l].n;
@@ -790,10 +1376,6 @@ void PrecDev<T>::solve_scratch(const double* x, double* y, unsigned char* scratc
       fp += maps[l].n - maps[l].nf;
     }
   }
-  const int64_t nl_last = maps.empty() ? n : maps.back().n - maps.back().nf;
-  B.yy = wp;
-  B.xx = wp + nl_last;
-  B.flags = (int32_t*)(scratch + sp.flags);
   B.tick = (unsigned long long*)(scratch + sp.tick);
   B.abort = (int*)(scratch + sp.abort);
   B.nsm = nsm_dev;
