@@ -19,15 +19,27 @@
 // For each column k it needs row k's factored pivot block and its U row:
 // row k publishes them as one record (below) and a 64-bit word in done[k]
 // telling where the record lies, so the dependant waits for one word and
-// brings the record on chip with one bulk asynchronous copy (completing on an
-// mbarrier); the record of the next pending column is fetched ahead while
-// the current step computes.  After the last column the warp thresholds its U
-// part, applies lfil to L and U (radix selection of the lfil largest norms),
+// brings the record on chip with its own asynchronous copies; the record of
+// the next pending column is fetched ahead while the current step computes.
+// After the last column the warp thresholds its U part, applies lfil to it,
 // sorts the kept blocks by column, factors its diagonal block (GEPP) and
-// publishes.  Per element, the operation order is the oracle's, so FP64
-// results match it bit for bit; the mixed factor keeps its drop sums, drop
-// tests and diagonal GEPP in FP32 (a block whose condition estimate exceeds
-// the threshold is factored again in FP64).
+// publishes; the L part, which no other row reads, is written after that.  Per
+// element, the operation order is the oracle's, so FP64 results match it bit
+// for bit; the mixed factor keeps its drop sums, drop tests and diagonal GEPP
+// in FP32 (a block whose condition estimate exceeds the threshold is factored
+// again in FP64).
+//
+// Bound: the chain of dependent rows times a link's latency (a dependant's step
+// for the column it waited on, then its finish).  With 16 warps an SM, stages
+// of 2 KB and 128 registers, the records of more than about ten U blocks (FP64:
+// four) were read in place from L2, one dependent load after another, and half
+// of the rows worked in global memory: 32 us a link (FP64 42 to 66).  Now 7
+// warps an SM (FP64 5, wide rows 3) have all their registers and keep records
+// and rows on chip; a step's update takes a column per lane, divisions by pivot
+// entries are corrected products with their reciprocals, the pivot search and
+// the reciprocals overlap, and FP64 drop tests are decided in FP32 where that
+// is certain.  The kernel's time before and now: 3.0 million unknowns FP32 710
+// and 416 ms, 360 000 FP64 498 and 270 ms, 48 000 at tau 0.9 786 and 270 ms.
 //
 // A wait that runs out sets VB_ETIMEOUT and raises an abort flag; a row that
 // failed publishes kRowFailed so that its dependants stop too.  Overflowing a
@@ -51,35 +63,47 @@ enum : int { SL_LIVE = 0, SL_LKEPT = 1, SL_DEAD = 2 };
 
 // ---------------------------------------------------------------------------
 // Published rows.  Row k's record, in the U pool, 16-byte aligned:
-//   int32 head[4]         ucnt (U blocks), nk, lu64 (1: the pivot LU is stored
-//                         in FP64, else in the factor's type), nval (U values)
-//   int32 piv[nk]         GEPP interchanges of the pivot block
-//   TL lu[nk * nk]        the factored pivot block, row-major
+//   int32 head[4]         ucnt (U blocks), nk, 2 depth + lu64 (lu64 = 1: the
+//                         pivot LU is stored in FP64, else in the factor's
+//                         type TL; depth: rows on the longest chain of waits
+//                         that ends at the row), ncol (U columns)
+//   int32 perm[nk]        row of the pivot block that GEPP brought to each place
+//   TL lu[nk * S]         the factored pivot block, rows S = lu_stride apart
+//   TL ry[nk], rz[nk]     reciprocals of its diagonal (recip_rn)
 //   int32 ucol[ucnt]      U block columns, ascending
-//   int32 urel[ucnt]      each U block's first value within val
+//   int32 ucst[ucnt]      each U block's first column within the row's U part
 //   int32 unj[ucnt]       each U block's column count
-//   T val[nval]           the U blocks, row-major, in column order
+//   T val[ncol * nk]      the U blocks, row-major, in column order (block q's
+//                         values start at nk ucst[q])
 // every part starting on a 16-byte boundary.  done[k] = (offset << 24) |
 // length, both in 16-byte units, once the record is complete; kRowFailed when
 // the row failed; 0 before.
 constexpr unsigned long long kRowFailed = ~0ull;
 constexpr int64_t kRecMaxUnits = (1LL << 24) - 1;
 
-__host__ __device__ __forceinline__ int64_t pad16(int64_t b) { return (b + 15) & ~(int64_t)15; }
+// Row stride of a record's pivot LU: FP32 blocks of at most 8 rows are read by
+// unrolled code with fixed offsets.
+__host__ __device__ __forceinline__ int lu_stride(int nk, int lu64, int tsize) {
+  return !lu64 && tsize == 4 && nk <= 8 ? 8 : nk;
+}
 
+template <typename I>
 struct RecLayout {
-  int64_t piv, lu, ucol, urel, unj, val, bytes;
+  I perm, lu, rcp, ucol, ucst, unj, val, bytes;
 };
-
-__host__ __device__ __forceinline__ RecLayout rec_layout(int ucnt, int nk, int lu64, int64_t nval, int tsize) {
-  RecLayout L;
-  L.piv = 16;
-  L.lu = L.piv + pad16(4LL * nk);
-  L.ucol = L.lu + pad16((int64_t)nk * nk * (lu64 ? 8 : tsize));
-  L.urel = L.ucol + pad16(4LL * ucnt);
-  L.unj = L.urel + pad16(4LL * ucnt);
-  L.val = L.unj + pad16(4LL * ucnt);
-  L.bytes = L.val + pad16(nval * tsize);
+// I = int for a published record (at most 2^28 bytes), int64_t to size a new one.
+template <typename I>
+__host__ __device__ __forceinline__ RecLayout<I> rec_layout(int ucnt, int nk, int lu64, int ncol, int tsize) {
+  RecLayout<I> L;
+  const I tl = lu64 ? 8 : tsize, uc = ((I)ucnt * 4 + 15) & ~(I)15;
+  L.perm = 16;
+  L.lu = L.perm + (((I)nk * 4 + 15) & ~(I)15);
+  L.rcp = L.lu + (((I)nk * lu_stride(nk, lu64, tsize) * tl + 15) & ~(I)15);
+  L.ucol = L.rcp + ((2 * (I)nk * tl + 15) & ~(I)15);
+  L.ucst = L.ucol + uc;
+  L.unj = L.ucst + uc;
+  L.val = L.unj + uc;
+  L.bytes = L.val + (((I)ncol * nk * tsize + 15) & ~(I)15);
   return L;
 }
 
@@ -137,21 +161,29 @@ std::map<long long, struct IlutGeom> g_geom;
 constexpr int64_t kTuneMinRows = 65536;
 
 constexpr int PVMAX = 64;
-struct IlutMisc {
-  unsigned long long mbar[2];  // completion of the bulk copy into stage buffer b
-  unsigned long long nvals;
-  long long wdst[32];  // destination offset of each block of a copied chunk
-  int hist[256];       // radix selection of the lfil cut
-  int qoff[32];        // workspace value offset of each U block's target
-  int quo[32];         // value offset of the U block within the record values
-  int qnj[32];
-  int qpre[33];        // element prefix of a chunk's blocks
-  int pv[PVMAX];       // GEPP interchanges of the row's own diagonal block
-  float lu32[64];      // the row's FP32 pivot LU (at most 8 x 8) for its record
-  float mbuf[64];      // a step's FP32 multiplier (at most 64 values) for its update
-  int nl, nslots, flag, pad;
-};
+constexpr int NSMALL = 8;   // FP32 pivot blocks up to this size are factored and applied in registers
+constexpr int NPIV = 32;    // and up to this factored in registers
+constexpr int MCOLS = 512;  // columns of a chunk of U blocks that the column update maps
 
+// Per-warp scratch.  buf serves, one after the other: the lfil cut's histogram
+// (256 int), a multiplier being formed, a chunk's column map (MCOLS bytes) and
+// block descriptors (32 int4), the general update's tables.
+template <typename T>
+struct alignas(16) IlutMisc {
+  int buf[256];
+  T mt[1024 / sizeof(T)];  // rows of a step's multiplier, transposed: row a of column r at r * np + a
+  T lu[NSMALL * NSMALL];   // the row's own small pivot LU (FP32)
+  T ry[NPIV], rz[NPIV];    // reciprocals of its diagonal (FP32)
+  int pv[PVMAX];           // GEPP interchanges of the row's own diagonal block
+  int perm[PVMAX];         // and the rows they brought to each place
+};
+struct CopyTab {  // tables of the general update, in IlutMisc::buf
+  int qpre[33];   // element prefix of a chunk's blocks
+  int qoff[32];   // workspace value offset of each U block's target
+  int quo[32];    // value offset of the U block within the record's values
+  int qnj[32];
+};
+static_assert(sizeof(CopyTab) <= 1024, "tables exceed the scratch");
 
 template <typename T>
 __device__ __forceinline__ T msub(T acc, T a, T b);
@@ -183,38 +215,45 @@ __device__ __forceinline__ bool drop_rule_f(float f2, int m, int n, float t) {
 __device__ __forceinline__ long long norm_key(double f2) { return __double_as_longlong(f2); }
 __device__ __forceinline__ long long norm_key(float f2) { return (long long)__float_as_int(f2); }
 
-template <typename T>
-__device__ __forceinline__ double fro2_seq(const T* v, int n) {
-  double s = 0.0;
-  for (int e = 0; e < n; ++e) {
-    const double x = (double)v[e];
-    s = __dadd_rn(s, __dmul_rn(x, x));
+// x[perm[j]] <- x[j] for one row of length m, in place: every cycle of the
+// permutation is turned from its smallest place.
+template <typename T, typename F>
+__device__ __forceinline__ void row_permute(T* x, int m, F&& perm) {
+#pragma unroll 1
+  for (int j = 0; j < m; ++j) {
+    int q = perm(j);
+    while (q > j && q < m) q = perm(q);
+    if (q != j) continue;  // j is not the smallest place of its cycle
+    T v = x[j];
+#pragma unroll 1
+    for (q = perm(j); q != j && q >= 0 && q < m; q = perm(q)) {
+      const T t = x[q];
+      x[q] = v;
+      v = t;
+    }
+    x[j] = v;
   }
-  return s;
 }
 
 // x (one row of length m) <- x (P^T L U)^{-1} = x U^{-1} L^{-1} P, with the
 // factored pivot block read through L2 (written by another warp).
 template <typename T, typename TL>
-__device__ void ainv_right_row(const TL* lu, const int32_t* pv, int m, T* x) {
+__device__ __noinline__ void ainv_right_row(const TL* lu, int S, const int32_t* pv, int m, T* x) {
+#pragma unroll 1
   for (int j = 0; j < m; ++j) {
     TL s = (TL)x[j];
-    for (int q = 0; q < j; ++q) s = msub<TL>(s, (TL)x[q], __ldcg(lu + q * m + j));
-    x[j] = (T)(s / __ldcg(lu + j * m + j));
+#pragma unroll 1
+    for (int q = 0; q < j; ++q) s = msub<TL>(s, (TL)x[q], __ldcg(lu + q * S + j));
+    x[j] = (T)(s / __ldcg(lu + j * S + j));
   }
+#pragma unroll 1
   for (int j = m - 1; j >= 0; --j) {
     TL s = (TL)x[j];
-    for (int q = j + 1; q < m; ++q) s = msub<TL>(s, (TL)x[q], __ldcg(lu + q * m + j));
+#pragma unroll 1
+    for (int q = j + 1; q < m; ++q) s = msub<TL>(s, (TL)x[q], __ldcg(lu + q * S + j));
     x[j] = (T)s;
   }
-  for (int k = m - 1; k >= 0; --k) {
-    const int p = __ldcg(pv + k);
-    if (p > k && p < m) {  // GEPP interchanges satisfy k <= p < m
-      const T t = x[k];
-      x[k] = x[p];
-      x[p] = t;
-    }
-  }
+  row_permute(x, m, [&](int j) { return __ldcg(pv + j); });
 }
 
 // Workspace hash: keys[h] = -2 - slot, -1 = empty; the column of a slot is
@@ -222,6 +261,7 @@ __device__ void ainv_right_row(const TL* lu, const int32_t* pv, int m, T* x) {
 // __syncwarp), and the columns inserted in one phase are distinct.
 __device__ __forceinline__ int ws_place(int* keys, uint32_t mask, int slot, int col) {
   uint32_t h = hmix((uint32_t)col) & mask;
+#pragma unroll 1
   for (uint32_t probe = 0; probe <= mask; ++probe) {
     if (atomicCAS(&keys[h], -1, -2 - slot) == -1) return (int)h;
     h = (h + 1) & mask;
@@ -231,6 +271,7 @@ __device__ __forceinline__ int ws_place(int* keys, uint32_t mask, int slot, int 
 
 __device__ __forceinline__ int ws_lookup(const int* keys, const int* scol, uint32_t mask, int col) {
   uint32_t h = hmix((uint32_t)col) & mask;
+#pragma unroll 1
   for (uint32_t probe = 0; probe <= mask; ++probe) {
     const int kv = keys[h];
     if (kv == -1) return -1;
@@ -241,28 +282,12 @@ __device__ __forceinline__ int ws_lookup(const int* keys, const int* scol, uint3
   return -1;
 }
 
-// Claim a new slot of sz values for column col; returns the slot or -1.
-__device__ __forceinline__ int ws_new_slot(int smax, int64_t vmax, int* keys, int* hpos, int* scol, int* soff,
-                                           int* sstate, int* sncl, int* nslots, unsigned long long* nvals,
-                                           uint32_t hmask, int col, int ncl, int sz) {
-  const int slot = atomicAdd(nslots, 1);
-  const long long off = (long long)atomicAdd(nvals, (unsigned long long)sz);
-  if (slot >= smax) return -1;
-  hpos[slot] = -1;  // the end-of-row reset skips slots that were never placed
-  if (off + sz > vmax) return -1;
-  scol[slot] = col;
-  soff[slot] = (int)off;
-  sstate[slot] = SL_LIVE;
-  sncl[slot] = ncl;
-  hpos[slot] = ws_place(keys, hmask, slot, col);
-  return hpos[slot] < 0 ? -1 : slot;
-}
-
 constexpr int MAX_SLOTS = 4096;  // largest workspace (blocks of one working row)
 
 // Warp-cooperative copy with eight independent loads in flight per lane.
 template <typename T>
-__device__ __forceinline__ void warp_copy(T* __restrict__ dst, const T* __restrict__ src, int64_t n, int lane) {
+__device__ __noinline__ void warp_copy(T* __restrict__ dst, const T* __restrict__ src, int64_t n, int lane) {
+#pragma unroll 1
   for (int64_t e0 = lane; e0 < n; e0 += 32 * 8) {
     T v[8];
 #pragma unroll
@@ -281,8 +306,9 @@ __device__ __forceinline__ void warp_copy(T* __restrict__ dst, const T* __restri
 // Squared Frobenius norm in row-major order (the oracle's summation order),
 // with the loads issued eight at a time.
 template <typename T>
-__device__ __forceinline__ double fro2_batched(const T* __restrict__ v, int n) {
+__device__ __noinline__ double fro2_batched(const T* __restrict__ v, int n) {
   double s = 0.0;
+#pragma unroll 1
   for (int e0 = 0; e0 < n; e0 += 8) {
     T x[8];
 #pragma unroll
@@ -301,6 +327,7 @@ __device__ __forceinline__ double fro2_batched(const T* __restrict__ v, int n) {
 template <typename T>
 __device__ __forceinline__ float fro2_f32(const T* __restrict__ v, int n) {
   float s = 0.f;
+#pragma unroll 1
   for (int e0 = 0; e0 < n; e0 += 16) {  // sixteen loads in flight, summed in element order
     float x[16];
 #pragma unroll
@@ -315,25 +342,22 @@ __device__ __forceinline__ float fro2_f32(const T* __restrict__ v, int n) {
 // x (one row of length m) <- x (P^T L U)^{-1} from a staged pivot block
 // (values of type TS, arithmetic in TL); x lives in shared memory.
 template <typename T, typename TL, typename TS>
-__device__ void ainv_right_row_sh(const TS* lu, const int* pv, int m, T* x) {
+__device__ __noinline__ void ainv_right_row_sh(const TS* lu, int S, const int* pv, int m, T* x) {
+#pragma unroll 1
   for (int j = 0; j < m; ++j) {
     TL s = (TL)x[j];
-    for (int q = 0; q < j; ++q) s = msub<TL>(s, (TL)x[q], (TL)lu[q * m + j]);
-    x[j] = (T)(s / (TL)lu[j * m + j]);
+#pragma unroll 1
+    for (int q = 0; q < j; ++q) s = msub<TL>(s, (TL)x[q], (TL)lu[q * S + j]);
+    x[j] = (T)(s / (TL)lu[j * S + j]);
   }
+#pragma unroll 1
   for (int j = m - 1; j >= 0; --j) {
     TL s = (TL)x[j];
-    for (int q = j + 1; q < m; ++q) s = msub<TL>(s, (TL)x[q], (TL)lu[q * m + j]);
+#pragma unroll 1
+    for (int q = j + 1; q < m; ++q) s = msub<TL>(s, (TL)x[q], (TL)lu[q * S + j]);
     x[j] = (T)s;
   }
-  for (int k = m - 1; k >= 0; --k) {
-    const int p = pv[k];
-    if (p > k && p < m) {
-      const T t = x[k];
-      x[k] = x[p];
-      x[p] = t;
-    }
-  }
+  row_permute(x, m, [&](int j) { return pv[j]; });
 }
 
 // |x| as an integer key: non-negative IEEE values order like their bit
@@ -359,10 +383,12 @@ __device__ __forceinline__ float div_rn<float>(float a, float b) {
 // Pivot rows go to gpiv (and pvs when not null).  Returns false when a pivot
 // column is exactly zero.
 template <typename TL>
-__device__ bool gepp_warp(TL* a, int n, int* pvs, int32_t* gpiv, int lane) {
+__device__ __noinline__ bool gepp_warp(TL* a, int n, int* pvs, int32_t* gpiv, int lane) {
+#pragma unroll 1
   for (int kk = 0; kk < n; ++kk) {
     long long key = -1;
     int idx = 0x7fffffff;
+#pragma unroll 1
     for (int ii = kk + lane; ii < n; ii += 32) {
       const long long v = abs_key(a[ii * n + kk]);
       if (v > key) {
@@ -385,6 +411,7 @@ __device__ bool gepp_warp(TL* a, int n, int* pvs, int32_t* gpiv, int lane) {
       if (pvs) pvs[kk] = pr;
     }
     if (pr != kk)
+#pragma unroll 1
       for (int jj = lane; jj < n; jj += 32) {
         const TL t = a[kk * n + jj];
         a[kk * n + jj] = a[pr * n + jj];
@@ -393,11 +420,13 @@ __device__ bool gepp_warp(TL* a, int n, int* pvs, int32_t* gpiv, int lane) {
     __syncwarp();
     const TL d = a[kk * n + kk];
     const int w = n - kk - 1;
+#pragma unroll 1
     for (int r = lane; r < w; r += 32) {
       TL* l = a + (kk + 1 + r) * n + kk;
       *l = div_rn<TL>(*l, d);
     }
     __syncwarp();
+#pragma unroll 1
     for (int e = lane; e < w * w; e += 32) {
       const int r = e / w, c = e - r * w;
       const int ii = kk + 1 + r, jj = kk + 1 + c;
@@ -411,11 +440,13 @@ __device__ bool gepp_warp(TL* a, int n, int* pvs, int32_t* gpiv, int lane) {
 // ||B^{-1}||_1 of a GEPP-factored FP32 block (n <= 32): lane c solves
 // B x = e_c through the interchanges, L and U; the result is the largest
 // column sum, on every lane.
-__device__ float inv_norm1_f32(const float* a, int n, const int* pv, int lane) {
+__device__ __noinline__ float inv_norm1_f32(const float* a, int n, const int* pv, int lane) {
   float cs = 0.f;
   if (lane < n) {
     float x[32];
+#pragma unroll 1
     for (int ii = 0; ii < n; ++ii) x[ii] = ii == lane ? 1.f : 0.f;
+#pragma unroll 1
     for (int kk = 0; kk < n; ++kk) {
       const int pk = pv[kk];
       if (pk != kk) {
@@ -424,260 +455,368 @@ __device__ float inv_norm1_f32(const float* a, int n, const int* pv, int lane) {
         x[pk] = t;
       }
     }
+#pragma unroll 1
     for (int ii = 1; ii < n; ++ii) {
       float sum = x[ii];
+#pragma unroll 1
       for (int kk = 0; kk < ii; ++kk) sum = __fmaf_rn(-a[ii * n + kk], x[kk], sum);
       x[ii] = sum;
     }
+#pragma unroll 1
     for (int ii = n - 1; ii >= 0; --ii) {
       float sum = x[ii];
+#pragma unroll 1
       for (int kk = ii + 1; kk < n; ++kk) sum = __fmaf_rn(-a[ii * n + kk], x[kk], sum);
       x[ii] = __fdiv_rn(sum, a[ii * n + ii]);
     }
+#pragma unroll 1
     for (int ii = 0; ii < n; ++ii) cs += fabsf(x[ii]);
   }
   for (int o = 16; o > 0; o >>= 1) cs = fmaxf(cs, __shfl_xor_sync(0xffffffffu, cs, o));
   return cs;
 }
 
-// ---- pivot blocks of at most 8 rows (FP32), held in registers ---------------
-// The block size is a template argument, so every loop is unrolled and no
-// array is indexed at run time.  Each routine gives every element the
-// operations of its generic counterpart (ainv_right_row_sh, gepp_warp,
-// inv_norm1_f32) in the same order, so the results are identical bit for
-// bit; only the latency of the dependent chain changes.
+// ---- division by a pivot entry -------------------------------------------
+// a / b correctly rounded from y = RN(1/b) and z, the rest of 1/b: q = a y +
+// a z is within one ulp of a / b, a - b q is exact, and the correction by it
+// rounds to RN(a / b) (Markstein's theorem: exact remainder, correctly rounded
+// reciprocal).  Valid while no intermediate can underflow or overflow, which
+// the exponent ranges below ensure; y = 0 marks a b outside of its range.
+__device__ __forceinline__ void recip_rn(float b, float& y, float& z) {
+  y = 0.f, z = 0.f;
+  if (fabsf(b) >= 0x1p-40f && fabsf(b) <= 0x1p40f) {
+    y = __frcp_rn(b);
+    z = __fmul_rn(__fmaf_rn(-b, y, 1.f), y);
+  }
+}
+__device__ __forceinline__ void recip_rn(double b, double& y, double& z) {
+  y = 0.0, z = 0.0;
+  if (fabs(b) >= 0x1p-300 && fabs(b) <= 0x1p300) {
+    y = __drcp_rn(b);
+    z = __dmul_rn(__fma_rn(-b, y, 1.0), y);
+  }
+}
+__device__ __forceinline__ float div_recip(float a, float b, float y, float z) {
+  const float q = __fmaf_rn(a, y, __fmul_rn(a, z));
+  return __fmaf_rn(__fmaf_rn(-b, q, a), y, q);
+}
+__device__ __forceinline__ double div_recip(double a, double b, double y, double z) {
+  const double q = __fma_rn(a, y, __dmul_rn(a, z));
+  return __fma_rn(__fma_rn(-b, q, a), y, q);
+}
+__device__ __forceinline__ bool div_range(float a, float y) {
+  return y != 0.f && fabsf(a) >= 0x1p-40f && fabsf(a) <= 0x1p40f;
+}
+__device__ __forceinline__ bool div_range(double a, double y) {
+  const unsigned e = ((unsigned)__double2hiint(a) >> 20) & 0x7ff;
+  return __double2hiint(y) != 0 && e >= 1023 - 300 && e < 1023 + 300;
+}
 
-// x (one row of length N, shared or global memory) <- x (P^T L U)^{-1}.
+// ---- FP32 pivot blocks held in registers -----------------------------------
+// The block's entries are read up front by broadcast 16-byte loads (rows N
+// floats apart), so that only the chain of operations itself is left; a size n
+// below N costs a uniform branch per row.  Each routine gives every element the
+// operations of its generic counterpart (ainv_right_row_sh, gepp_warp,
+// inv_norm1_f32) in the same order, so the results are identical bit for bit.
+// A 6 x 6 block, one warp alone: multiplier 1 900 cycles with the entries read
+// where they are used, factorization with condition estimate 6 200.
+
 template <int N>
-__device__ __forceinline__ void ainv_right_row_n(const float* lu, const int* pv, float* x, float* x2) {
-  float r[N];
+__device__ __forceinline__ void load_lu(const float* lu, float* L) {
 #pragma unroll
-  for (int j = 0; j < N; ++j) r[j] = x[j];
+  for (int e = 0; e < N * N; e += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(lu + e);
+    L[e] = v.x, L[e + 1] = v.y, L[e + 2] = v.z, L[e + 3] = v.w;
+  }
+}
+
+// r <- r (P^T L U)^{-1} for one row x[0, n), n <= 8; the result goes, permuted,
+// to the row m and (unless NULL) to mt with stride np.
+__device__ __forceinline__ void mult_row_small(const float* lu, const float* ry, const float* rz, const int* perm,
+                                               int n, const float* x, float* m, float* mt, int np) {
+  constexpr int N = NSMALL;
+  float L[N * N], r[N], y[N], z[N];
+  int c[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) r[j] = j < n ? x[j] : 0.f;
+  load_lu<N>(lu, L);
 #pragma unroll
   for (int j = 0; j < N; ++j) {
-    float s = r[j];
-#pragma unroll
-    for (int q = 0; q < j; ++q) s = msub<float>(s, r[q], lu[q * N + j]);
-    r[j] = s / lu[j * N + j];
+    y[j] = j < n ? ry[j] : 1.f;
+    z[j] = j < n ? rz[j] : 0.f;
+    c[j] = j < n ? perm[j] : 0;
   }
-#pragma unroll
-  for (int j = N - 1; j >= 0; --j) {
-    float s = r[j];
-#pragma unroll
-    for (int q = j + 1; q < N; ++q) s = msub<float>(s, r[q], lu[q * N + j]);
-    r[j] = s;
-  }
-#pragma unroll
-  for (int k = N - 1; k >= 0; --k) {
-    const int p = pv[k];
-#pragma unroll
-    for (int q = k + 1; q < N; ++q)
-      if (q == p) {
-        const float t = r[k];
-        r[k] = r[q];
-        r[q] = t;
-      }
-  }
-#pragma unroll
-  for (int j = 0; j < N; ++j) x[j] = r[j];
-  if (x2) {
-#pragma unroll
-    for (int j = 0; j < N; ++j) x2[j] = r[j];
-  }
-}
-
-// GEPP of the N x N row-major block a (shared memory), row i in lane i's
-// registers: the pivot is the largest |a_ik| (lowest row on ties) found by a
-// warp max-reduction of the keys and a ballot; interchanges and the pivot
-// row travel by shuffles.  Pivot rows go to gpiv (and pvs when not null).
-template <int N>
-__device__ __forceinline__ bool gepp_n(float* a, int* pvs, int32_t* gpiv, int lane) {
-  float r[N];
-#pragma unroll
-  for (int j = 0; j < N; ++j) r[j] = lane < N ? a[lane * N + j] : 0.f;
   bool ok = true;
 #pragma unroll
-  for (int k = 0; k < N; ++k) {
-    const unsigned key = (lane >= k && lane < N) ? (unsigned)abs_key(r[k]) + 1u : 0u;
-    const unsigned mk = __reduce_max_sync(0xffffffffu, key);
-    if (mk <= 1u) {  // the pivot column is exactly zero
-      ok = false;
-      break;
-    }
-    const int p = __ffs(__ballot_sync(0xffffffffu, key == mk)) - 1;
-    if (lane == 0) {
-      gpiv[k] = p;
-      if (pvs) pvs[k] = p;
-    }
-    if (p != k) {
+  for (int q = 0; q < N; ++q)
+    if (q < n) {  // x_q is complete: divide, then take it out of the columns to its right
+      ok = ok && div_range(r[q], y[q]);
+      r[q] = div_recip(r[q], L[q * N + q], y[q], z[q]);
 #pragma unroll
-      for (int j = 0; j < N; ++j) {
-        const float vk = __shfl_sync(0xffffffffu, r[j], k);
-        const float vp = __shfl_sync(0xffffffffu, r[j], p);
-        if (lane == k) r[j] = vp;
-        if (lane == p) r[j] = vk;
+      for (int j = q + 1; j < N; ++j) r[j] = msub<float>(r[j], r[q], L[q * N + j]);
+    }
+  if (!ok) {  // a dividend or a divisor outside of the range: divide
+#pragma unroll
+    for (int j = 0; j < N; ++j) r[j] = j < n ? x[j] : 0.f;
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (q < n) {
+        r[q] = __fdiv_rn(r[q], L[q * N + q]);
+#pragma unroll
+        for (int j = q + 1; j < N; ++j) r[j] = msub<float>(r[j], r[q], L[q * N + j]);
+      }
+  }
+#pragma unroll
+  for (int j = N - 2; j >= 0; --j) {
+#pragma unroll
+    for (int q = j + 1; q < N; ++q)
+      if (q < n) r[j] = msub<float>(r[j], r[q], L[q * N + j]);
+  }
+#pragma unroll
+  for (int j = 0; j < N; ++j)
+    if (j < n) {
+      m[c[j]] = r[j];
+      if (mt) mt[c[j] * np] = r[j];
+    }
+}
+
+// GEPP of the n x n row-major FP32 block at src (n <= N), row i in lane i's
+// registers: the pivot is the largest |a_ik| (the lowest position on ties)
+// found by a warp max-reduction of the keys and a ballot, while every lane
+// forms the reciprocal of its own candidate, so that the multipliers need no
+// division.  Rows are not exchanged: pos is the position that a lane's row has
+// come to.  The factored block goes to lu (rows N apart), its diagonal's
+// reciprocals to ry and rz, the interchanges to pvs and gpiv, the rows' order
+// to perm.  Then, on every lane, ||B^{-1}||_1 by solving B x = e_c on lane c.
+// False when a pivot column is exactly zero.
+template <int N>
+__device__ __noinline__ bool gepp_cond(const float* src, int n, float* lu, float* ry, float* rz, int* pvs, int* perm,
+                                       int32_t* gpiv, int lane, float* inv1) {
+  float r[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) r[j] = lane < n && j < n ? src[lane * n + j] : 0.f;
+  int pos = lane < n ? lane : 64;
+  float yd = 0.f, zd = 0.f;  // the reciprocal of the pivot that a lane's row supplied
+  bool done = lane >= n;
+#pragma unroll
+  for (int k = 0; k < N; ++k)
+    if (k < n) {
+      const unsigned key = done ? 0u : (unsigned)abs_key(r[k]) + 1u;
+      float yc, zc;
+      recip_rn(r[k], yc, zc);
+      const unsigned mk = __reduce_max_sync(0xffffffffu, key);
+      if (mk <= 1u) return false;  // the pivot column is exactly zero
+      unsigned who = __ballot_sync(0xffffffffu, key == mk);
+      if (who & (who - 1)) {
+        const int pm = (int)__reduce_min_sync(0xffffffffu, key == mk ? (unsigned)pos : 64u);
+        who = __ballot_sync(0xffffffffu, key == mk && pos == pm);
+      }
+      const int from = __ffs(who) - 1;
+      float u[N];
+#pragma unroll
+      for (int j = k; j < N; ++j) u[j] = __shfl_sync(0xffffffffu, r[j], from);
+      const float yp = __shfl_sync(0xffffffffu, yc, from), zp = __shfl_sync(0xffffffffu, zc, from);
+      const int p = __shfl_sync(0xffffffffu, pos, from);
+      if (lane == from) {
+        pos = k;
+        yd = yp, zd = zp;
+        done = true;
+      } else if (pos == k) {
+        pos = p;
+      }
+      if (lane == 0) {
+        gpiv[k] = p;
+        pvs[k] = p;
+      }
+      if (!done) {
+        const float l = div_range(r[k], yp) ? div_recip(r[k], u[k], yp, zp) : __fdiv_rn(r[k], u[k]);
+        r[k] = l;
+#pragma unroll
+        for (int j = k + 1; j < N; ++j) r[j] = msub<float>(r[j], l, u[j]);
       }
     }
-    float u[N];
+  if (lane < n) {
+    perm[pos] = lane;
+    ry[pos] = yd;
+    rz[pos] = zd;
 #pragma unroll
-    for (int j = k; j < N; ++j) u[j] = __shfl_sync(0xffffffffu, r[j], k);
-    if (lane > k && lane < N) {
-      const float l = div_rn<float>(r[k], u[k]);
-      r[k] = l;
-#pragma unroll
-      for (int j = k + 1; j < N; ++j) r[j] = msub<float>(r[j], l, u[j]);
-    }
-  }
-  if (lane < N) {
-#pragma unroll
-    for (int j = 0; j < N; ++j) a[lane * N + j] = r[j];
+    for (int j = 0; j < N; ++j) lu[pos * N + j] = r[j];
   }
   __syncwarp();
-  return ok;
-}
-
-// ||B^{-1}||_1 of a GEPP-factored N x N block: lane c solves B x = e_c in
-// registers; the largest column sum, on every lane.
-template <int N>
-__device__ __forceinline__ float inv_norm1_n(const float* a, const int* pv, int lane) {
+  // x = P e_c: one at the place that row c was brought to (lanes without a
+  // column follow lane 0's kind, so that they stay on the common path)
   float cs = 0.f;
-  if (lane < N) {
-    float x[N];
+  float x[N];
+  const int pc = lane < n ? pos : 0;
 #pragma unroll
-    for (int ii = 0; ii < N; ++ii) x[ii] = ii == lane ? 1.f : 0.f;
+  for (int i = 0; i < N; ++i) x[i] = i == pc ? 1.f : 0.f;
+  if (N <= 8) {
+    float L[N * N], y[N], z[N];
+    load_lu<N>(lu, L);
 #pragma unroll
-    for (int kk = 0; kk < N; ++kk) {
-      const int pk = pv[kk];
+    for (int i = 0; i < N; ++i) y[i] = i < n ? ry[i] : 1.f, z[i] = i < n ? rz[i] : 0.f;
 #pragma unroll
-      for (int q = kk + 1; q < N; ++q)
-        if (q == pk) {
-          const float t = x[kk];
-          x[kk] = x[q];
-          x[q] = t;
+    for (int i = 1; i < N; ++i) {
+#pragma unroll
+      for (int k = 0; k < i; ++k)
+        if (i < n) x[i] = __fmaf_rn(-L[i * N + k], x[k], x[i]);
+    }
+#pragma unroll
+    for (int i = N - 1; i >= 0; --i)
+      if (i < n) {
+#pragma unroll
+        for (int k = i + 1; k < N; ++k)
+          if (k < n) x[i] = __fmaf_rn(-L[i * N + k], x[k], x[i]);
+        x[i] = div_range(x[i], y[i]) ? div_recip(x[i], L[i * (N + 1)], y[i], z[i])
+                                     : __fdiv_rn(x[i], L[i * (N + 1)]);
+      }
+  } else {
+#pragma unroll
+    for (int i = 1; i < N; ++i)
+      if (i < n) {
+#pragma unroll
+        for (int k4 = 0; k4 < i; k4 += 4) {
+          const float4 v = *reinterpret_cast<const float4*>(lu + i * N + k4);
+          const float l[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int k = k4; k < i && k < k4 + 4; ++k) x[i] = __fmaf_rn(-l[k - k4], x[k], x[i]);
         }
-    }
+      }
 #pragma unroll
-    for (int ii = 1; ii < N; ++ii) {
-      float sum = x[ii];
+    for (int i = N - 1; i >= 0; --i)
+      if (i < n) {
 #pragma unroll
-      for (int kk = 0; kk < ii; ++kk) sum = __fmaf_rn(-a[ii * N + kk], x[kk], sum);
-      x[ii] = sum;
-    }
+        for (int k4 = (i + 1) & ~3; k4 < N; k4 += 4) {
+          const float4 v = *reinterpret_cast<const float4*>(lu + i * N + k4);
+          const float l[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int ii = N - 1; ii >= 0; --ii) {
-      float sum = x[ii];
-#pragma unroll
-      for (int kk = ii + 1; kk < N; ++kk) sum = __fmaf_rn(-a[ii * N + kk], x[kk], sum);
-      x[ii] = __fdiv_rn(sum, a[ii * N + ii]);
-    }
-#pragma unroll
-    for (int ii = 0; ii < N; ++ii) cs += fabsf(x[ii]);
+          for (int k = k4; k < N && k < k4 + 4; ++k)
+            if (k > i && k < n) x[i] = __fmaf_rn(-l[k - k4], x[k], x[i]);
+        }
+        x[i] = div_range(x[i], ry[i]) ? div_recip(x[i], lu[i * (N + 1)], ry[i], rz[i])
+                                      : __fdiv_rn(x[i], lu[i * (N + 1)]);
+      }
   }
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (i < n) cs += fabsf(x[i]);
+  if (lane >= n) cs = 0.f;
   for (int o = 16; o > 0; o >>= 1) cs = fmaxf(cs, __shfl_xor_sync(0xffffffffu, cs, o));
-  return cs;
+  *inv1 = cs;
+  return true;
 }
 
-// Dispatch on the block size (false / a negative norm: larger than 8, the
-// caller takes the generic routine).
-__device__ __forceinline__ bool ainv_right_row_small(const float* lu, const int* pv, int m, float* x, float* x2) {
-  switch (m) {
-    case 1: ainv_right_row_n<1>(lu, pv, x, x2); return true;
-    case 2: ainv_right_row_n<2>(lu, pv, x, x2); return true;
-    case 3: ainv_right_row_n<3>(lu, pv, x, x2); return true;
-    case 4: ainv_right_row_n<4>(lu, pv, x, x2); return true;
-    case 5: ainv_right_row_n<5>(lu, pv, x, x2); return true;
-    case 6: ainv_right_row_n<6>(lu, pv, x, x2); return true;
-    case 7: ainv_right_row_n<7>(lu, pv, x, x2); return true;
-    case 8: ainv_right_row_n<8>(lu, pv, x, x2); return true;
-    default: return false;
+// The same for any n and either type, in loops, the row held in shared memory
+// at w[j * nw].
+template <typename T>
+__device__ __noinline__ void mult_row_loop(const T* lu, const T* ry, const T* rz, const int* perm, int n, T* w, int nw,
+                                           T* m, T* mt, int np) {
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) w[j * nw] = m[j];
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) {
+    T s = w[j * nw];
+#pragma unroll 4
+    for (int q = 0; q < j; ++q) s = msub<T>(s, w[q * nw], lu[q * n + j]);
+    w[j * nw] = div_range(s, ry[j]) ? div_recip(s, lu[j * n + j], ry[j], rz[j]) : div_rn<T>(s, lu[j * n + j]);
+  }
+#pragma unroll 1
+  for (int j = n - 2; j >= 0; --j) {
+    T s = w[j * nw];
+#pragma unroll 4
+    for (int q = j + 1; q < n; ++q) s = msub<T>(s, w[q * nw], lu[q * n + j]);
+    w[j * nw] = s;
+  }
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) {
+    const int c = perm[j];
+    m[c] = w[j * nw];
+    if (mt) mt[c * np] = w[j * nw];
   }
 }
-__device__ __forceinline__ bool gepp_small(float* a, int n, int* pvs, int32_t* gpiv, int lane) {
-  switch (n) {
-    case 1: return gepp_n<1>(a, pvs, gpiv, lane);
-    case 2: return gepp_n<2>(a, pvs, gpiv, lane);
-    case 3: return gepp_n<3>(a, pvs, gpiv, lane);
-    case 4: return gepp_n<4>(a, pvs, gpiv, lane);
-    case 5: return gepp_n<5>(a, pvs, gpiv, lane);
-    case 6: return gepp_n<6>(a, pvs, gpiv, lane);
-    case 7: return gepp_n<7>(a, pvs, gpiv, lane);
-    default: return gepp_n<8>(a, pvs, gpiv, lane);
+
+// perm from the interchanges pvs of a block of n <= PVMAX rows (pvs and perm in
+// shared memory).
+__device__ __noinline__ void perm_of(const int* pvs, int n, int* perm, int lane) {
+  if (lane == 0) {
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) perm[k] = k;
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+      const int p = pvs[k], t = perm[k];
+      perm[k] = perm[p];
+      perm[p] = t;
+    }
   }
+  __syncwarp();
 }
-__device__ __forceinline__ float inv_norm1_small(const float* a, int n, const int* pv, int lane) {
-  switch (n) {
-    case 1: return inv_norm1_n<1>(a, pv, lane);
-    case 2: return inv_norm1_n<2>(a, pv, lane);
-    case 3: return inv_norm1_n<3>(a, pv, lane);
-    case 4: return inv_norm1_n<4>(a, pv, lane);
-    case 5: return inv_norm1_n<5>(a, pv, lane);
-    case 6: return inv_norm1_n<6>(a, pv, lane);
-    case 7: return inv_norm1_n<7>(a, pv, lane);
-    default: return inv_norm1_n<8>(a, pv, lane);
-  }
+
+// ---- the drop rule of an FP64 block, decided in FP32 where that is certain --
+// |v| as an FP32 value from the upper bits of the FP64 one (an FP64 operation
+// or conversion takes 64 to 100 cycles on this part); false outside 2^+-55.
+__device__ __forceinline__ bool abs_f32(double v, float& f) {
+  const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  f = __int_as_float((int)(((h - (896u << 20)) << 3) | ((unsigned)__double2loint(v) >> 29)));
+  if (h - ((1023u - 55u) << 20) < (110u << 20)) return true;
+  f = 0.f;
+  return h == 0 && __double2loint(v) == 0;
+}
+// s: the FP32 sum of squares of n <= 4096 entries, ok: all were in range.
+// 1: dropped, 0: kept, -1: too near the threshold.  Truncation, the sum and the
+// threshold are off by less than (n + 8) 2^-23 together, the margin by 2^-10.
+__device__ __forceinline__ int drop_f32(float s, bool ok, int m, int n, float t) {
+  const float thr = t * (float)m * (float)n, thr2 = thr * thr;
+  if (!ok || !(thr2 == 0.f ? t == 0.f : thr2 >= 1e-30f) || !(thr2 <= 1e30f)) return -1;
+  if (s * (1.f + 0x1p-10f) < thr2) return 1;
+  if (s * (1.f - 0x1p-10f) >= thr2) return 0;
+  return -1;
 }
 
 // ---------------------------------------------------------------------------
-// Bulk asynchronous copies into shared memory, completing on an mbarrier.
-__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+// A published record is brought on chip by the warp's own asynchronous copies
+// (16 bytes a lane through L2, so that no line of L1 can be stale), which need
+// no fence between proxies: from a publication to the record in the
+// dependant's shared memory 1.2 us, against 2.3 us with a bulk copy completing
+// on an mbarrier (1.5 KB records, one warp handing on to the next).
+__device__ __forceinline__ void record_fetch(void* dst, const unsigned char* src, int bytes, int lane) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+#pragma unroll 1
+  for (int e = lane * 16; e < bytes; e += 512)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + e), "l"(src + e) : "memory");
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+// All copies but the youngest `keep` groups have arrived, for the whole warp.
+template <int KEEP>
+__device__ __forceinline__ void record_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(KEEP) : "memory");
+  __syncwarp();
 }
 
-// Orders this thread's generic-proxy view of memory with the async proxy
-// (the bulk copies): taken by a producer after writing a record and by a
-// consumer after acquiring its flag, before issuing the copy.
-__device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
-
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
+__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
 }
-
-__device__ __forceinline__ bool mbar_test(unsigned long long* bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Bounded wait for phase `parity` of bar to complete; false when limit ns
-// passed first.
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, unsigned long long limit) {
-  if (mbar_test(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
-  for (unsigned it = 1;; ++it) {
-    if (mbar_test(bar, parity)) return true;
-    if ((it & 15) == 0 && global_ns() - t0 > limit) return false;
-  }
-}
-
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
   unsigned long long v;
   asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
 
-// The published word of a row, waiting for it as wait_flag does (relaxed
-// polls with backoff, the abort word and the time budget every 16th poll,
-// one acquire fence at the end).  0 when the wait gave up.
+// The published word of a row: acquiring polls with a short backoff, the abort
+// word and the time budget looked at only every 16th poll.  0 when the wait
+// gave up.
 __device__ __forceinline__ unsigned long long wait_word(const unsigned long long* w, int* abort,
                                                         unsigned long long limit, int* st) {
-  unsigned long long v = ld_relaxed_u64(w);
+  unsigned long long v = ld_acquire_u64(w);
   if (v == 0) {
     const unsigned long long t0 = global_ns();
-    unsigned nsl = 32;
+    unsigned nsl = 16;
+#pragma unroll 1
     for (unsigned it = 1;; ++it) {
       __nanosleep(nsl);
-      if (nsl < 256) nsl <<= 1;
-      v = ld_relaxed_u64(w);
+      if (nsl < 128) nsl <<= 1;
+      v = ld_acquire_u64(w);
       if (v != 0) break;
       if ((it & 15) == 0) {
         if (*((volatile int*)abort) != 0) return 0;
@@ -689,14 +828,16 @@ __device__ __forceinline__ unsigned long long wait_word(const unsigned long long
       }
     }
   }
-  asm volatile("fence.acq_rel.gpu;" ::: "memory");
   return v;
 }
 
 // Ascending bitonic sort of a[0, n2) (n2 a power of two) by one warp.
 __device__ void warp_bitonic_sort(unsigned long long* a, int n2, int lane) {
+#pragma unroll 1
   for (int k = 2; k <= n2; k <<= 1)
+#pragma unroll 1
     for (int j = k >> 1; j > 0; j >>= 1) {
+#pragma unroll 1
       for (int x = lane; x < n2; x += 32) {
         const int y = x ^ j;
         if (y > x) {
@@ -715,23 +856,82 @@ __device__ void warp_bitonic_sort(unsigned long long* a, int n2, int lane) {
 // parameters): of the n candidate slots cand[], keep the lfil with the
 // largest norm keys, lower column first on equal keys; the others become
 // SL_DEAD and cand[] is compacted to the kept ones.  The lfil-th largest key
-// is found by radix selection, 8 bits a pass from the top (keybytes passes:
-// the keys are the bit patterns of non-negative FP64 or FP32 norms, so their
-// integer order is their value order).  Returns the number kept.
-__device__ int lfil_cut(int* cand, int n, int lfil, const long long* sf2, const int* scol, int* sstate, int* hist,
+// is found in registers when the keys are FP32 norms and n <= 256, else by
+// radix selection, 8 bits a pass from the top (keybytes passes: the keys are
+// the bit patterns of non-negative FP64 or FP32 norms, so their integer order
+// is their value order).  Returns the number kept.
+__device__ __noinline__ int lfil_cut(int* cand, int n, int lfil, const long long* sf2, const int* scol, int* sstate, int* hist,
                         int keybytes, int lane) {
   if (lfil < 0 || n <= lfil) return n;
   if (lfil == 0) {
+#pragma unroll 1
     for (int c = lane; c < n; c += 32) sstate[cand[c]] = SL_DEAD;
     __syncwarp();
     return 0;
   }
+  if (keybytes == 4 && n <= 256) {
+    // keys of 31 bits, up to 8 a lane in registers: the lfil-th largest is
+    // built bit by bit, each bit kept if lfil keys reach the value with it
+    unsigned kq[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) kq[u] = lane + 32 * u < n ? (unsigned)sf2[cand[lane + 32 * u]] + 1u : 0u;
+    unsigned thr = 0;
+#pragma unroll 1
+    for (int bit = 31; bit >= 0; --bit) {
+      const unsigned t = thr | (1u << bit);
+      int c = 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) c += kq[u] >= t;
+      if (__reduce_add_sync(0xffffffffu, c) >= lfil) thr = t;
+    }
+    int above = 0, equal = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) above += kq[u] > thr, equal += kq[u] == thr;
+    above = __reduce_add_sync(0xffffffffu, above);
+    equal = __reduce_add_sync(0xffffffffu, equal);
+    const int want = lfil - above;  // of the keys equal to thr, those with the lowest columns
+    unsigned keep = 0;
+    int q[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int c = lane + 32 * u;
+      q[u] = c < n ? cand[c] : -1;
+      bool k = kq[u] > thr;
+      if (kq[u] == thr && c < n) {
+        int rank = 0;
+        if (equal > want) {
+          const int col = scol[q[u]];
+#pragma unroll 1
+          for (int c2 = 0; c2 < n; ++c2) {
+            const int q2 = cand[c2];
+            if ((unsigned)sf2[q2] + 1u == thr && scol[q2] < col) ++rank;
+          }
+        }
+        k = rank < want;
+      }
+      if (c < n && !k) sstate[q[u]] = SL_DEAD;
+      keep |= (unsigned)k << u;
+    }
+    __syncwarp();
+    int kept = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const unsigned bk = __ballot_sync(0xffffffffu, keep >> u & 1);
+      if (keep >> u & 1) cand[kept + __popc(bk & ((1u << lane) - 1u))] = q[u];
+      kept += __popc(bk);
+    }
+    __syncwarp();
+    return kept;
+  }
   unsigned long long prefix = 0, pmask = 0;
   int want = lfil;  // keys still to take at or below the current prefix
+#pragma unroll 1
   for (int d = keybytes - 1; d >= 0; --d) {
     const int shift = 8 * d;
+#pragma unroll 1
     for (int b = lane; b < 256; b += 32) hist[b] = 0;
     __syncwarp();
+#pragma unroll 1
     for (int base = 0; base < n; base += 32) {
       const int c = base + lane;
       int bin = -1;
@@ -782,6 +982,7 @@ __device__ int lfil_cut(int* cand, int n, int lfil, const long long* sf2, const 
   // keys above prefix are kept; of the keys equal to it, the `want` with the
   // lowest columns.  Every cut slot is marked first (the tie ranks read the
   // whole list), then the list is compacted.
+#pragma unroll 1
   for (int c = lane; c < n; c += 32) {
     const int q = cand[c];
     const unsigned long long key = (unsigned long long)sf2[q];
@@ -789,6 +990,7 @@ __device__ int lfil_cut(int* cand, int n, int lfil, const long long* sf2, const 
     if (key == prefix) {
       const int col = scol[q];
       int rank = 0;
+#pragma unroll 1
       for (int c2 = 0; c2 < n; ++c2) {
         const int q2 = cand[c2];
         if ((unsigned long long)sf2[q2] == prefix && scol[q2] < col) ++rank;
@@ -799,6 +1001,7 @@ __device__ int lfil_cut(int* cand, int n, int lfil, const long long* sf2, const 
   }
   __syncwarp();
   int kept = 0;
+#pragma unroll 1
   for (int base = 0; base < n; base += 32) {
     const int c = base + lane;
     const int q = c < n ? cand[c] : -1;
@@ -813,86 +1016,240 @@ __device__ int lfil_cut(int* cand, int n, int lfil, const long long* sf2, const 
 }
 
 // The kept blocks of one part in column order: srt[p] = col << 32 | slot for
-// p < k (n2 = the next power of two, padded with ~0).  Returns n2.
-__device__ int sort_by_column(const int* cand, int k, const int* scol, unsigned long long* srt, int lane) {
+// p < k (space for the next power of two).
+__device__ __noinline__ void sort_by_column(const int* cand, int k, const int* scol, unsigned long long* srt, int lane) {
   int n2 = 1;
   while (n2 < k) n2 <<= 1;
-  if (k <= 32) {  // the keys are distinct: each goes to its rank
-    const unsigned long long key =
-        lane < k ? ((unsigned long long)(unsigned)scol[cand[lane]] << 32) | (unsigned)cand[lane] : ~0ull;
-    int rank = 0;
-    for (int j = 0; j < k; ++j) rank += __shfl_sync(0xffffffffu, key, j) < key ? 1 : 0;
-    if (lane < k)
-      srt[rank] = key;
-    else if (lane < n2)
-      srt[lane] = ~0ull;
+  if (k <= 64) {  // the keys are distinct: each goes to its rank
+    const int qa = lane < k ? cand[lane] : 0, qb = 32 + lane < k ? cand[32 + lane] : 0;
+    const unsigned ca = lane < k ? (unsigned)scol[qa] : ~0u, cb = 32 + lane < k ? (unsigned)scol[qb] : ~0u;
+    int ra = 0, rb = 0;
+#pragma unroll 4
+    for (int j = 0; j < 32; ++j) {
+      if (j >= k) break;
+      const unsigned c = __shfl_sync(0xffffffffu, ca, j);
+      ra += c < ca, rb += c < cb;
+    }
+#pragma unroll 4
+    for (int j = 32; j < 64; ++j) {
+      if (j >= k) break;
+      const unsigned c = __shfl_sync(0xffffffffu, cb, j - 32);
+      ra += c < ca, rb += c < cb;
+    }
+    if (lane < k) srt[ra] = ((unsigned long long)ca << 32) | (unsigned)qa;
+    if (32 + lane < k) srt[rb] = ((unsigned long long)cb << 32) | (unsigned)qb;
     __syncwarp();
-    return n2;
+    return;
   }
   for (int p = lane; p < n2; p += 32)
     srt[p] = p < k ? ((unsigned long long)(unsigned)scol[cand[p]] << 32) | (unsigned)cand[p] : ~0ull;
   __syncwarp();
   warp_bitonic_sort(srt, n2, lane);
-  return n2;
 }
 
-// Copy blocks to consecutive destinations, 32 blocks a round: block b of the
-// round has sz[b] values at src offset so[b] and goes to dst offset dof[b];
-// lanes walk the round's flattened values, eight loads in flight per lane.
+// Copy up to 32 blocks (lane p: sz values at src + so to dst + dof), eight
+// lanes to a block and eight loads in flight a lane.
 template <typename T>
-__device__ __forceinline__ void copy_round(IlutMisc& M, int sz, int so, long long dof, const T* __restrict__ src,
-                                           T* __restrict__ dst, int lane) {
+__device__ __noinline__ void copy_blocks(int n, int sz, int so, long long dof, const T* __restrict__ src,
+                                            T* __restrict__ dst, int lane) {
+  const int g = lane >> 3, a = lane & 7;
+#pragma unroll 1
+  for (int p0 = 0; p0 < n; p0 += 4) {
+    const int p = min(p0 + g, 31);
+    const int s = __shfl_sync(0xffffffffu, sz, p), o = __shfl_sync(0xffffffffu, so, p);
+    const long long d = __shfl_sync(0xffffffffu, dof, p);
+    const int m = p0 + g < n ? s : 0;
+#pragma unroll 1
+    for (int e0 = a; e0 < m; e0 += 64) {
+      T v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (e0 + 8 * u < m) v[u] = src[o + e0 + 8 * u];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (e0 + 8 * u < m) dst[d + e0 + 8 * u] = v[u];
+    }
+  }
+}
+
+// A factored pivot block (rows S apart) and the reciprocals of its diagonal into
+// a record.
+template <typename TL>
+__device__ __noinline__ void put_pivot(const TL* lu, int S, int n, TL* o, TL* rcp, int lane) {
+#pragma unroll 1
+  for (int e = lane; e < n * n; e += 32) {
+    const int a = e / n;
+    o[e] = lu[a * S + e - a * n];
+  }
+#pragma unroll 1
+  for (int a = lane; a < n; a += 32) {
+    TL y, z;
+    recip_rn(lu[a * (S + 1)], y, z);
+    rcp[a] = y;
+    rcp[n + a] = z;
+  }
+}
+
+// One chunk of U blocks of a step: w(:, j) -= m U_kj for the chunk's columns and
+// the rows [row0, row0 + ni) of the working row, whose multiplier is in mt.
+// qinfo[q] = {workspace offset of the target, first column, columns, 1 if the
+// target is new (its old values are zeros)}, cmap[c] = the block of column c.
+// FP32: a lane takes a column, so that a value of U and the target's address
+// serve ni rows, and the multiplier comes as broadcast 16-byte loads.
+__device__ __forceinline__ void update_columns(const int4* qinfo, const unsigned char* cmap, int cols,
+                                               const float* mt, int row0, int ni, int nk, int np, const float* U,
+                                               float* wv, int lane) {
+#pragma unroll 1
+  for (int c = lane; c < cols; c += 32) {
+    const int4 I = qinfo[cmap[c]];
+    const int jj = c - I.y, nj = I.z;
+    const float* u = U + nk * I.y + jj;
+    float* z = wv + I.x + row0 * nj + jj;
+#pragma unroll 1
+    for (int a0 = 0; a0 < ni; a0 += 8) {
+      float acc[8];
+      if (I.w) {
+#pragma unroll
+        for (int a = 0; a < 8; ++a) acc[a] = 0.f;
+      } else {
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+          if (a0 + a < ni) acc[a] = z[(a0 + a) * nj];
+      }
+      const float* m = mt + a0;
+#pragma unroll 2
+      for (int r = 0; r < nk; ++r) {
+        const float ur = u[r * nj];
+        const float4 m0 = *reinterpret_cast<const float4*>(m + r * np);
+        acc[0] = __fmaf_rn(-m0.x, ur, acc[0]);
+        acc[1] = __fmaf_rn(-m0.y, ur, acc[1]);
+        acc[2] = __fmaf_rn(-m0.z, ur, acc[2]);
+        acc[3] = __fmaf_rn(-m0.w, ur, acc[3]);
+        if (a0 + 4 < ni) {
+          const float4 m1 = *reinterpret_cast<const float4*>(m + r * np + 4);
+          acc[4] = __fmaf_rn(-m1.x, ur, acc[4]);
+          acc[5] = __fmaf_rn(-m1.y, ur, acc[5]);
+          acc[6] = __fmaf_rn(-m1.z, ur, acc[6]);
+          acc[7] = __fmaf_rn(-m1.w, ur, acc[7]);
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < 8; ++a)
+        if (a0 + a < ni) z[(a0 + a) * nj] = acc[a];
+    }
+  }
+}
+// FP64: the operations themselves are the cost (64 cycles each for any number
+// of lanes), so the elements are dealt out evenly, two a lane in flight.
+__device__ __forceinline__ void update_columns(const int4* qinfo, const unsigned char* cmap, int cols,
+                                               const double* mt, int row0, int ni, int nk, int np, const double* U,
+                                               double* wv, int lane) {
+  const int total = ni * cols;
+  const float rc = 1.f / (float)cols;
+#pragma unroll 1
+  for (int e = lane; e < total; e += 32) {
+    int a = (int)((float)e * rc);  // e / cols, corrected
+    int c = e - a * cols;
+    if (c < 0) --a, c += cols;
+    if (c >= cols) ++a, c -= cols;
+    const int4 I = qinfo[cmap[c]];
+    const int jj = c - I.y, nj = I.z;
+    const double* u = U + nk * I.y + jj;
+    double* z = wv + I.x + (row0 + a) * nj + jj;
+    double acc = I.w ? 0.0 : *z;
+    const double* m = mt + a;
+#pragma unroll 1
+    for (int r = 0; r < nk; ++r) acc = msub<double>(acc, m[r * np], u[r * nj]);
+    *z = acc;
+  }
+}
+
+// One chunk of U blocks of any sizes (lane q: block q's target offset, first
+// column and columns; missing: the target is new), the multiplier m row-major:
+// lanes over the flattened elements, four per lane in flight.  A record that
+// is not staged is read through L2.
+template <typename T>
+__device__ __noinline__ void update_general(CopyTab& tab, int nq, int off, int cst, int nj, bool missing, int ni,
+                                            int nk, const T* m, const T* rval, bool staged, T* wv, int lane) {
+  const int sz = ni * nj;
+  if (missing) {
+    T* z = wv + off;
+#pragma unroll 1
+    for (int e = 0; e < sz; ++e) z[e] = (T)0;
+  }
   int incl = sz;
   for (int o = 1; o < 32; o <<= 1) {
     const int v = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += v;
   }
   const int total = __shfl_sync(0xffffffffu, incl, 31);
-  M.qpre[lane] = incl - sz;
-  if (lane == 31) M.qpre[32] = total;
-  M.qoff[lane] = so;
-  M.wdst[lane] = dof;
+  tab.qpre[lane] = incl - sz;
+  if (lane == 31) tab.qpre[32] = total;
+  tab.qoff[lane] = off;
+  tab.quo[lane] = nk * cst;
+  tab.qnj[lane] = nj;
   __syncwarp();
-  for (int e0 = lane; e0 < total; e0 += 32 * 8) {
-    T v[8];
-    long long d8[8];
+#pragma unroll 1
+  for (int e0 = lane; e0 < total; e0 += 128) {
+    T acc[4];
+    T* dst[4];
+    int a4[4], jj4[4], nj4[4], uo4[4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < 4; ++u) {
       const int e = e0 + 32 * u;
-      d8[u] = -1;
+      dst[u] = nullptr;
       if (e < total) {
-        int lo = 0, hi = 31;  // last block with qpre <= e (empty blocks share a prefix)
+        int lo = 0, hi = nq - 1;  // block tq with qpre[tq] <= e < qpre[tq + 1]
         while (lo < hi) {
           const int mid = (lo + hi + 1) >> 1;
-          if (M.qpre[mid] <= e)
+          if (tab.qpre[mid] <= e)
             lo = mid;
           else
             hi = mid - 1;
         }
-        const int local = e - M.qpre[lo];
-        v[u] = src[M.qoff[lo] + local];
-        d8[u] = M.wdst[lo] + local;
+        const int njt = tab.qnj[lo];
+        const int local = e - tab.qpre[lo];
+        a4[u] = local / njt;
+        jj4[u] = local - a4[u] * njt;
+        nj4[u] = njt;
+        uo4[u] = tab.quo[lo];
+        dst[u] = wv + tab.qoff[lo] + local;
+        acc[u] = *dst[u];
       }
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (d8[u] >= 0) dst[d8[u]] = v[u];
+    for (int u = 0; u < 4; ++u) {
+      if (!dst[u]) continue;
+      const T* U = rval + uo4[u];
+      T av = acc[u];
+      if (staged) {
+#pragma unroll 1
+        for (int r = 0; r < nk; ++r) av = msub<T>(av, m[a4[u] * nk + r], U[r * nj4[u] + jj4[u]]);
+      } else {
+#pragma unroll 1
+        for (int r = 0; r < nk; ++r) av = msub<T>(av, m[a4[u] * nk + r], __ldcg(U + r * nj4[u] + jj4[u]));
+      }
+      *dst[u] = av;
+    }
   }
-  __syncwarp();
 }
 
-
-
 template <typename T>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, 1)
     k_ilut(VBView<T> A, IlutGeom g, Workspace ws, T* __restrict__ wvals_all, Pools P, T* __restrict__ lval,
            unsigned char* __restrict__ upool, const int64_t* __restrict__ dgoff, double* __restrict__ dg,
            float* __restrict__ dg32, int32_t* __restrict__ piv, int32_t* __restrict__ ptag, int mixed,
            double cond_thr, double t, int lfil, unsigned long long wait_limit, int* st) {
   extern __shared__ __align__(128) unsigned char ilut_sm[];
+  constexpr bool F32 = std::is_same<T, float>::value;
+  constexpr int TS = (int)sizeof(T);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
   unsigned char* const wb = ilut_sm + (size_t)warp * g.bytes;
-  IlutMisc& M = *reinterpret_cast<IlutMisc*>(wb + g.o_misc);
+  IlutMisc<T>& M = *reinterpret_cast<IlutMisc<T>*>(wb + g.o_misc);
+  CopyTab& tab = *reinterpret_cast<CopyTab*>(M.buf);
+  unsigned char* const cmap = reinterpret_cast<unsigned char*>(M.buf);
+  int4* const qinfo = reinterpret_cast<int4*>(M.buf + MCOLS / 4);
   unsigned char* const stage0 = wb + g.o_stage;
   unsigned char* const stage1 = stage0 + g.stage;
   T* const sh_vals = reinterpret_cast<T*>(wb + g.o_vals);
@@ -906,38 +1263,14 @@ __global__ void __launch_bounds__(256, 2)
   int* const lc = reinterpret_cast<int*>(wb + g.o_lc);  // pending L columns (INT_MAX when processed)
   int* const ls = reinterpret_cast<int*>(wb + g.o_ls);  // their slots
   const int64_t wid = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
-  const int VSH = g.vbytes / (int)sizeof(T);
+  const int VSH = g.vbytes / TS;
   const float tf = (float)t, condf = (float)cond_thr;
-  constexpr int TS = (int)sizeof(T);
-  volatile int* vflag = &M.flag;
-  volatile int* vns = &M.nslots;
-  volatile int* vnl = &M.nl;
   int* const gkeys = ws.keys + wid * ws.ht;
+#pragma unroll 1
   for (int k = lane; k < ws.ht; k += 32) gkeys[k] = -1;
+#pragma unroll 1
   for (int k = lane; k < g.hash; k += 32) sh_keys[k] = -1;
-  if (lane == 0) {
-    mbar_init(&M.mbar[0]);
-    mbar_init(&M.mbar[1]);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
   __syncwarp();
-  // stage buffer bookkeeping, the same in every lane: the column whose record
-  // a buffer holds (-1: free), whether its copy still has to be waited for,
-  // and the parity of its mbarrier's next phase
-  int btag0 = -1, btag1 = -1;
-  bool bpend0 = false, bpend1 = false;
-  unsigned bph0 = 0, bph1 = 0;
-  auto drain = [&]() {  // wait (bounded) for copies in flight and free both buffers
-    if (bpend0) {
-      if (mbar_wait(&M.mbar[0], bph0, wait_limit)) bph0 ^= 1;
-      bpend0 = false;
-    }
-    if (bpend1) {
-      if (mbar_wait(&M.mbar[1], bph1, wait_limit)) bph1 ^= 1;
-      bpend1 = false;
-    }
-    btag0 = btag1 = -1;
-  };
 
   for (;;) {
     long long row = 0;
@@ -951,15 +1284,14 @@ __global__ void __launch_bounds__(256, 2)
     row = __shfl_sync(0xffffffffu, row, 0);
     if (row >= A.nbr) break;
     const int64_t i = row;
-    int maxdep = 0;  // lane 0: the deepest row waited on
+    int maxdep = 0;  // the deepest row waited on
     const int ni = A.rsz[i];
     const int64_t b0 = A.bptr[i], b1 = A.bptr[i + 1];
     const int64_t v0 = A.voff[b0], nv = A.voff[b1] - v0;
     const int nb = (int)(b1 - b0);
     // The working row lives in shared memory when it leaves room for fill; a
-    // row whose fill outgrows that restarts in the warp's global workspace
-    // (nothing of it is visible before its finish, so the restart is exact).
-    bool in_sh = nb <= g.slots / 2 && nv <= VSH / 2;
+    // row whose fill outgrows that moves to the warp's global workspace.
+    bool in_sh = nb <= g.slots / 2 && nv <= VSH * 3 / 4;
     int status_local = 0;
     int* keys;
     int* hpos;
@@ -972,448 +1304,432 @@ __global__ void __launch_bounds__(256, 2)
     int smax_c;
     int64_t vmax_c;
     uint32_t hmask;
-    for (;;) {
-      if (in_sh) {
-        keys = sh_keys, hpos = sh_hpos, scol = sh_scol, soff = sh_soff, sstate = sh_sst, sf2 = sh_sf2;
-        sncl = sh_sncl;
-        wv = sh_vals;
-        smax_c = g.slots, vmax_c = VSH, hmask = (uint32_t)g.hash - 1;
-      } else {
-        keys = gkeys, hpos = ws.hpos + wid * ws.smax, scol = ws.scol + wid * ws.smax;
-        soff = ws.soff + wid * ws.smax, sstate = ws.sstate + wid * ws.smax, sf2 = ws.sf2 + wid * ws.smax;
-        sncl = ws.sncl + wid * ws.smax;
-        wv = wvals_all + wid * ws.vmax;
-        smax_c = ws.smax, vmax_c = ws.vmax, hmask = (uint32_t)ws.ht - 1;
-      }
-      if (lane == 0) {
-        M.nslots = 0;
-        M.nvals = 0;
-        M.flag = 0;
-        M.nl = 0;
-      }
-      __syncwarp();
-      // ---- load row i of A into the workspace: slot q is the row's block q
-      // and the values arrive as one contiguous copy; columns left of the
-      // diagonal enter the list of pending L columns
-      if (nb > smax_c || nv > vmax_c) {
-        if (lane == 0) {
-          *vflag = 1;
-          atomicMax(P.ctr + 5, (unsigned long long)nv);
-          atomicMax(P.ctr + 6, (unsigned long long)nb);
-        }
-      } else {
-        for (int64_t b = b0 + lane; b < b1; b += 32) {
-          const int slot = (int)(b - b0);
-          const int32_t J = A.bcol[b];
+    if (in_sh) {
+      keys = sh_keys, hpos = sh_hpos, scol = sh_scol, soff = sh_soff, sstate = sh_sst, sf2 = sh_sf2;
+      sncl = sh_sncl;
+      wv = sh_vals;
+      smax_c = g.slots, vmax_c = VSH, hmask = (uint32_t)g.hash - 1;
+    } else {
+      keys = gkeys, hpos = ws.hpos + wid * ws.smax, scol = ws.scol + wid * ws.smax;
+      soff = ws.soff + wid * ws.smax, sstate = ws.sstate + wid * ws.smax, sf2 = ws.sf2 + wid * ws.smax;
+      sncl = ws.sncl + wid * ws.smax;
+      wv = wvals_all + wid * ws.vmax;
+      smax_c = ws.smax, vmax_c = ws.vmax, hmask = (uint32_t)ws.ht - 1;
+    }
+    // the row's slots, values and pending L columns so far, and the slot of
+    // its diagonal block: the same in every lane
+    int ns = 0, nl = 0, dslot = -1;
+    long long nval = 0;
+    int ask_s = 0;  // what an overflowing row asked for
+    long long ask_v = 0;
+    // ---- load row i of A into the workspace: slot q is the row's block q
+    // and the values arrive as one contiguous copy; columns left of the
+    // diagonal enter the list of pending L columns
+    if (nb > smax_c || nv > vmax_c) {
+      status_local = DEV_OVERFLOW;
+      ask_s = nb;
+      ask_v = nv;
+    } else {
+#pragma unroll 1
+      for (int base = 0; base < nb; base += 32) {
+        const int slot = base + lane;
+        int32_t J = INT_MAX;
+        if (slot < nb) {
+          const int64_t b = b0 + slot;
+          J = A.bcol[b];
           scol[slot] = J;
           soff[slot] = (int)(A.voff[b] - v0);
           sstate[slot] = SL_LIVE;
           sncl[slot] = A.rsz[J];
           hpos[slot] = ws_place(keys, hmask, slot, J);  // the table holds 2 smax positions
-          if (J < i) {
-            const int q = atomicAdd(&M.nl, 1);
-            if (q < g.lcap) {
-              lc[q] = J;
-              ls[q] = slot;
-            }
+        }
+        const unsigned low = __ballot_sync(0xffffffffu, J < i), dia = __ballot_sync(0xffffffffu, J == i);
+        if (J < i) {
+          const int q = nl + __popc(low & lt);
+          if (q < g.lcap) {
+            lc[q] = J;
+            ls[q] = slot;
           }
         }
-        warp_copy(wv, A.val + v0, nv, lane);
-        if (lane == 0) {
-          M.nslots = nb;
-          M.nvals = (unsigned long long)nv;
-        }
+        nl += __popc(low);
+        if (dia) dslot = base + __ffs(dia) - 1;
       }
-      __syncwarp();
-      status_local = *vflag ? DEV_OVERFLOW : 0;
-      int64_t last = -1;
-      // ---- eliminate the L part in ascending column order (including fill)
-      while (status_local == 0) {
-        // the next pending L column and the one after it: from the list while
-        // it has not overflowed, else by a scan of the workspace slots
-        int c1 = INT_MAX, s1 = -1, p1 = -1, c2 = INT_MAX;
-        const int nlist = *vnl;
-        if (nlist <= g.lcap) {
-          for (int q = lane; q < nlist; q += 32) {
-            const int c = lc[q];
+      warp_copy(wv, A.val + v0, nv, lane);
+      ns = nb;
+      nval = nv;
+    }
+    __syncwarp();
+    // stage buffer bookkeeping, the same in every lane: the column whose
+    // record a buffer holds or is being copied into (-1: free)
+    int btag0 = -1, btag1 = -1;
+    int64_t last = -1;
+    // ---- eliminate the L part in ascending column order (including fill)
+    while (status_local == 0) {
+      // the next pending L column and the one after it: from the list while
+      // it has not overflowed, else by a scan of the workspace slots
+      int c1 = INT_MAX, s1 = -1, p1 = -1, c2 = INT_MAX;
+      if (nl <= g.lcap) {
+#pragma unroll 1
+        for (int q = lane; q < nl; q += 32) {
+          const int c = lc[q];
+          if (c < c1) {
+            c2 = c1;
+            c1 = c;
+            p1 = q;
+          } else if (c < c2) {
+            c2 = c;
+          }
+        }
+        if (p1 >= 0) s1 = ls[p1];
+      } else {
+#pragma unroll 1
+        for (int sidx = lane; sidx < ns; sidx += 32) {
+          const int c = scol[sidx];
+          if (sstate[sidx] == SL_LIVE && c > last && c < i) {
             if (c < c1) {
               c2 = c1;
               c1 = c;
-              s1 = ls[q];
-              p1 = q;
+              s1 = sidx;
             } else if (c < c2) {
               c2 = c;
             }
           }
-        } else {
-          const int ns = min(*vns, smax_c);
-          for (int sidx = lane; sidx < ns; sidx += 32) {
-            const int c = scol[sidx];
-            if (sstate[sidx] == SL_LIVE && c > last && c < i) {
-              if (c < c1) {
-                c2 = c1;
-                c1 = c;
-                s1 = sidx;
-              } else if (c < c2) {
-                c2 = c;
-              }
-            }
-          }
         }
-        const int kmin = warp_min_i(c1);
-        if (kmin == INT_MAX) break;
-        const unsigned who = __ballot_sync(0xffffffffu, s1 >= 0 && c1 == kmin);
-        const int owner = __ffs(who) - 1;
-        const int sk = __shfl_sync(0xffffffffu, s1, owner);
-        const int knext = warp_min_i(lane == owner ? c2 : c1);
-        if (lane == owner && p1 >= 0) lc[p1] = INT_MAX;
-        const int64_t k = kmin;
-        last = k;
-        const int nk = A.rsz[k];
-        // ---- row k's record: already fetched ahead into a stage buffer, or
-        // fetched now (a bounded wait for its word, then one bulk copy); a
-        // record too large for a buffer is read in place
-        int bi = btag0 == (int)k ? 0 : (btag1 == (int)k ? 1 : -1);
-        const unsigned char* rec = nullptr;
-        int64_t rlen = 0;
-        // the word of the next pending column is loaded now and looked at
-        // after the multiplier, so that its latency hides behind this step
-        const bool want_pf = knext != INT_MAX && btag0 != knext && btag1 != knext;
-        unsigned long long w2 = 0;
-        if (want_pf && lane == 0) w2 = ld_relaxed_u64(P.done + knext);
-        if (bi < 0) {
-          unsigned long long word = 0;
-          if (lane == 0) word = wait_word(P.done + k, P.abort, wait_limit, st);
-          word = __shfl_sync(0xffffffffu, word, 0);
-          if (word == 0 || word == kRowFailed) {
-            status_local = DEV_ETIMEOUT;
-            break;
-          }
-          rlen = (int64_t)(word & 0xFFFFFFull) * 16;
-          const unsigned char* src = upool + (int64_t)(word >> 24) * 16;
-          if (rlen <= g.stage) {
-            // a free buffer, else one holding a record fetched ahead for a
-            // later column: its copy is waited for before the buffer is reused
-            bi = btag0 < 0 ? 0 : (btag1 < 0 ? 1 : 0);
-            bool ok = true;
-            if (bi == 0 && bpend0) {
-              ok = mbar_wait(&M.mbar[0], bph0, wait_limit);
-              if (ok) bph0 ^= 1;
-              bpend0 = !ok;
-            } else if (bi == 1 && bpend1) {
-              ok = mbar_wait(&M.mbar[1], bph1, wait_limit);
-              if (ok) bph1 ^= 1;
-              bpend1 = !ok;
-            }
-            if (!__all_sync(0xffffffffu, ok)) {
-              if (lane == 0) dev_fail(st, DEV_ETIMEOUT);
-              status_local = DEV_ETIMEOUT;
-              break;
-            }
-            if (lane == 0) {
-              fence_proxy_async_all();
-              bulk_load(bi ? stage1 : stage0, src, (unsigned)rlen, &M.mbar[bi]);
-            }
-            if (bi) {
-              btag1 = (int)k;
-              bpend1 = true;
-            } else {
-              btag0 = (int)k;
-              bpend0 = true;
-            }
-          } else {
-            rec = src;
-          }
-        }
-        if (bi >= 0) {
-          bool ok = true;
-          if (bi == 0 && bpend0) {
-            ok = mbar_wait(&M.mbar[0], bph0, wait_limit);
-            if (ok) bph0 ^= 1;
-            bpend0 = !ok;
-          } else if (bi == 1 && bpend1) {
-            ok = mbar_wait(&M.mbar[1], bph1, wait_limit);
-            if (ok) bph1 ^= 1;
-            bpend1 = !ok;
-          }
-          if (!__all_sync(0xffffffffu, ok)) {
-            if (lane == 0) dev_fail(st, DEV_ETIMEOUT);
-            status_local = DEV_ETIMEOUT;
-            break;
-          }
-          rec = bi ? stage1 : stage0;
-        }
-        const bool staged = bi >= 0;
-        if (P.depth && lane == 0) maxdep = max(maxdep, ld_relaxed_gpu(P.depth + k));
-        // header: U blocks, pivot size, pivot precision, U values
-        int hv = 0;
-        if (lane < 4) hv = staged ? reinterpret_cast<const int*>(rec)[lane] : __ldcg(reinterpret_cast<const int*>(rec) + lane);
-        const int ucnt = __shfl_sync(0xffffffffu, hv, 0);
-        const int hnk = __shfl_sync(0xffffffffu, hv, 1);
-        const int lu64 = __shfl_sync(0xffffffffu, hv, 2);
-        const int uval_n = __shfl_sync(0xffffffffu, hv, 3);
-        const RecLayout RL = rec_layout(ucnt, nk, lu64, uval_n, TS);
-        if (hnk != nk || ucnt < 0 || uval_n < 0 || (!staged && RL.bytes > rlen && rlen) ||
-            (staged && RL.bytes > g.stage)) {
-          status_local = DEV_INTERNAL;  // never true for a published row: record and skip
+      }
+      const int kmin = __reduce_min_sync(0xffffffffu, c1);
+      if (kmin == INT_MAX) break;
+      const int owner = __ffs(__ballot_sync(0xffffffffu, c1 == kmin)) - 1;
+      const int sk = __shfl_sync(0xffffffffu, s1, owner);
+      const int knext = __reduce_min_sync(0xffffffffu, lane == owner ? c2 : c1);
+      if (lane == owner && p1 >= 0) lc[p1] = INT_MAX;
+      const int64_t k = kmin;
+      last = k;
+      const int nk = A.rsz[k];
+      // ---- row k's record: already fetched ahead into a stage buffer, or
+      // fetched now (a bounded wait for its word, then the copies); a record
+      // too large for a buffer is read in place.  The word of the next pending
+      // column is looked at meanwhile, and its record fetched into the other
+      // buffer when its row is already published: beside the copies of this
+      // one, or, when this one was fetched ahead, after the multiplier.
+      // (bi: the buffer, 2: both as one, for a record larger than one.)
+      int bi = btag0 == (int)k ? 0 : (btag1 == (int)k ? 1 : -1);
+      const unsigned char* rec = nullptr;
+      int64_t rlen = 0;
+      const bool want_pf = knext != INT_MAX && btag0 != knext && btag1 != knext;
+      unsigned long long w2 = 0;
+      bool fetched = false;  // the next record is being fetched
+      if (bi < 0) {
+        unsigned long long word = 0;
+        if (lane == 0) word = wait_word(P.done + k, P.abort, wait_limit, st);
+        word = __shfl_sync(0xffffffffu, word, 0);
+        if (word == 0 || word == kRowFailed) {
+          status_local = DEV_ETIMEOUT;
           break;
         }
-        const int* rpiv = reinterpret_cast<const int*>(rec + RL.piv);
-        const int* rcol = reinterpret_cast<const int*>(rec + RL.ucol);
-        const int* rrel = reinterpret_cast<const int*>(rec + RL.urel);
-        const int* rnj = reinterpret_cast<const int*>(rec + RL.unj);
-        const T* rval = reinterpret_cast<const T*>(rec + RL.val);
-        T* m = wv + soff[sk];
-        // the multiplier m = a_ik (P^T L U)_k^{-1}, in place, one lane per row;
-        // an FP32 multiplier of at most 64 values is also kept in M.mbuf, where
-        // the drop test and the update read it
-        bool mb = false;
-        if constexpr (std::is_same<T, float>::value) mb = staged && !lu64 && nk <= 8 && ni * nk <= 64;
-        const T* msrc = m;
-        if constexpr (std::is_same<T, float>::value)
-          if (mb) msrc = M.mbuf;
+        rlen = (int64_t)(word & 0xFFFFFFull) * 16;
+        const unsigned char* src = upool + (int64_t)(word >> 24) * 16;
+        if (rlen <= g.stage) {
+          // a free buffer, else one holding a record fetched ahead for a
+          // later column, whose copies have to arrive before it is reused
+          bi = btag0 < 0 ? 0 : (btag1 < 0 ? 1 : 0);
+          if (btag0 >= 0 && btag1 >= 0) record_wait<0>();
+          record_fetch(bi ? stage1 : stage0, src, (int)rlen, lane);
+          (bi ? btag1 : btag0) = (int)k;
+          if (want_pf && (bi ? btag0 : btag1) < 0) {
+            if (lane == 0) w2 = ld_acquire_u64(P.done + knext);
+            w2 = __shfl_sync(0xffffffffu, w2, 0);
+            if (w2 != 0 && w2 != kRowFailed && (int64_t)(w2 & 0xFFFFFFull) * 16 <= g.stage) {
+              record_fetch(bi ? stage0 : stage1, upool + (int64_t)(w2 >> 24) * 16, (int)((w2 & 0xFFFFFFull) * 16),
+                           lane);
+              (bi ? btag0 : btag1) = knext;
+              fetched = true;
+            }
+          }
+          if (fetched)
+            record_wait<1>();
+          else
+            record_wait<0>();
+        } else if (rlen <= 2LL * g.stage) {
+          record_wait<0>();
+          record_fetch(stage0, src, (int)rlen, lane);
+          bi = 2;
+          btag0 = btag1 = (int)k;
+          record_wait<0>();
+        } else {
+          rec = src;
+        }
+      } else {
+        if (want_pf && lane == 0) w2 = ld_relaxed_u64(P.done + knext);
+        record_wait<0>();
+      }
+      const bool staged = bi >= 0;
+      if (staged) rec = bi == 1 ? stage1 : stage0;
+      // header: U blocks, pivot size, pivot precision and depth, U columns
+      const int4 hd = staged ? *reinterpret_cast<const int4*>(rec) : __ldcg(reinterpret_cast<const int4*>(rec));
+      const int ucnt = hd.x, lu64 = hd.z & 1, ncol = hd.w;
+      maxdep = max(maxdep, hd.z >> 1);
+      const RecLayout<int> RL = rec_layout<int>(ucnt, nk, lu64, ncol, TS);
+      if (hd.y != nk || ucnt < 0 || ncol < 0 || (!staged && RL.bytes > rlen) ||
+          (staged && RL.bytes > (bi == 2 ? 2 : 1) * g.stage)) {
+        status_local = DEV_INTERNAL;  // never true for a published row: record and skip
+        break;
+      }
+      const int* rperm = reinterpret_cast<const int*>(rec + RL.perm);
+      const int* rcol = reinterpret_cast<const int*>(rec + RL.ucol);
+      const int* rcst = reinterpret_cast<const int*>(rec + RL.ucst);
+      const int* rnj = reinterpret_cast<const int*>(rec + RL.unj);
+      const T* rval = reinterpret_cast<const T*>(rec + RL.val);
+      const unsigned char* const rs = bi == 1 ? stage1 : stage0;  // a staged record
+      T* m = wv + soff[sk];
+      // the multiplier m = a_ik (P^T L U)_k^{-1}, in place, one lane per row.
+      // With a staged record whose pivot block is not too large (mb), np rows at
+      // a time are also held transposed in M.mt, where the column update reads
+      // them; when that is the whole multiplier (mall) the drop test does too.
+      constexpr int CAP = 1024 / TS;
+      const int np = ni > 8 && nk * 16 <= CAP ? 16 : 8;
+      const bool mb = staged && nk * 8 <= CAP && !(F32 && lu64);
+      const bool mall = mb && ni <= np;
+      const int S = lu_stride(nk, lu64, TS);
+      if (mb) {
+        const T* lu = reinterpret_cast<const T*>(rs + RL.lu);
+        const T* ry = reinterpret_cast<const T*>(rs + RL.rcp);
+        const int* pm = reinterpret_cast<const int*>(rs + RL.perm);
+        bool small = false;
+        if constexpr (F32) {
+          small = nk <= NSMALL;
+          if (small) {
+#pragma unroll 1
+            for (int a = lane; a < ni; a += 32)
+              mult_row_small(lu, ry, ry + nk, pm, nk, m + a * nk, m + a * nk, mall ? M.mt + a : nullptr, np);
+          }
+        }
+        if (!small) {
+#pragma unroll 1
+          for (int a = lane; a < ni && lane < np; a += np)
+            mult_row_loop<T>(lu, ry, ry + nk, pm, nk, reinterpret_cast<T*>(M.buf) + lane, np, m + a * nk,
+                             mall ? M.mt + a : nullptr, np);
+        }
+        if (mall && lane >= ni && lane < np) {  // the padding rows of the transposed multiplier
+#pragma unroll 1
+          for (int r = 0; r < nk; ++r) M.mt[r * np + lane] = (T)0;
+        }
+      } else {
+#pragma unroll 1
         for (int a = lane; a < ni; a += 32) {
           if (staged) {
             if (lu64)
-              ainv_right_row_sh<T, double, double>(reinterpret_cast<const double*>(rec + RL.lu), rpiv, nk, m + a * nk);
-            else {
-              bool small = false;
-              if constexpr (std::is_same<T, float>::value)
-                small = ainv_right_row_small(reinterpret_cast<const float*>(rec + RL.lu), rpiv, nk, m + a * nk,
-                                             mb ? M.mbuf + a * nk : nullptr);
-              if (!small)
-                ainv_right_row_sh<T, float, T>(reinterpret_cast<const T*>(rec + RL.lu), rpiv, nk, m + a * nk);
-            }
+              ainv_right_row_sh<T, double, double>(reinterpret_cast<const double*>(rec + RL.lu), S, rperm, nk,
+                                                   m + a * nk);
+            else
+              ainv_right_row_sh<T, float, T>(reinterpret_cast<const T*>(rec + RL.lu), S, rperm, nk, m + a * nk);
           } else {
             if (lu64)
-              ainv_right_row<T, double>(reinterpret_cast<const double*>(rec + RL.lu), rpiv, nk, m + a * nk);
+              ainv_right_row<T, double>(reinterpret_cast<const double*>(rec + RL.lu), S, rperm, nk, m + a * nk);
             else
-              ainv_right_row<T, T>(reinterpret_cast<const T*>(rec + RL.lu), rpiv, nk, m + a * nk);
+              ainv_right_row<T, T>(reinterpret_cast<const T*>(rec + RL.lu), S, rperm, nk, m + a * nk);
           }
         }
-        __syncwarp();
-        long long key = 0;
-        bool dropped;
-        if (sizeof(T) == sizeof(double)) {  // the oracle's summation order
+      }
+      __syncwarp();
+      // the drop rule.  The norm of a kept FP32 multiplier is its lfil key; an
+      // FP64 one's is formed after the row is published, if lfil asks for it.
+      const int sz_m = ni * nk;
+      const unsigned kinv = (65536u + (unsigned)nk - 1u) / (unsigned)nk;  // e / nk for e < 256, nk <= 32
+      bool dropped;
+      long long key = 0;
+      if constexpr (F32) {  // FP32 squares, summed by a warp reduction
+        float sf = 0.f;
+#pragma unroll 1
+        for (int e = lane; e < sz_m; e += 32) {
+          float x;
+          if (mall) {
+            const int a = (int)((unsigned)e * kinv >> 16);
+            x = (float)M.mt[(e - a * nk) * np + a];
+          } else {
+            x = (float)m[e];
+          }
+          sf = __fmaf_rn(x, x, sf);
+        }
+        for (int o = 16; o > 0; o >>= 1) sf += __shfl_xor_sync(0xffffffffu, sf, o);
+        dropped = drop_rule_f(sf, ni, nk, tf);
+        key = norm_key(sf);
+      } else {
+        float sf = 0.f;
+        bool in = true;
+#pragma unroll 1
+        for (int e = lane; e < sz_m; e += 32) {
+          float x;
+          in = abs_f32((double)m[e], x) && in;
+          sf = __fmaf_rn(x, x, sf);
+        }
+        for (int o = 16; o > 0; o >>= 1) sf += __shfl_xor_sync(0xffffffffu, sf, o);
+        int d = drop_f32(sf, __all_sync(0xffffffffu, in) && sz_m <= 4096, ni, nk, tf);
+        if (d < 0) {  // too near the threshold: the oracle's summation order
           double f2 = 0.0;
-          if (lane == 0) f2 = fro2_seq(m, ni * nk);
+          if (lane == 0) f2 = fro2_batched(m, sz_m);
           f2 = __shfl_sync(0xffffffffu, f2, 0);
-          dropped = drop_rule(f2, ni, nk, t);
-          key = norm_key(f2);
-        } else {  // mixed factor: FP32 squares summed by a warp reduction
-          float sf = 0.f;
-          for (int e = lane; e < ni * nk; e += 32) {
-            const float x = (float)msrc[e];
-            sf = __fmaf_rn(x, x, sf);
-          }
-          for (int o = 16; o > 0; o >>= 1) sf += __shfl_xor_sync(0xffffffffu, sf, o);
-          dropped = drop_rule_f(sf, ni, nk, tf);
-          key = norm_key(sf);
+          d = drop_rule(f2, ni, nk, t);
         }
-        // the next pending column's record, fetched ahead while the update
-        // computes, when its row was already published at the start of the
-        // step, no buffer holds it yet and a buffer is free (the current
-        // step's buffer holds k)
-        if (want_pf) {
-          const int ob = btag0 < 0 ? 0 : (btag1 < 0 ? 1 : -1);
-          int go = 0;
-          if (ob >= 0 && lane == 0 && w2 != 0 && w2 != kRowFailed && (int64_t)(w2 & 0xFFFFFFull) * 16 <= g.stage) {
-            asm volatile("fence.acq_rel.gpu;" ::: "memory");
-            fence_proxy_async_all();
-            bulk_load(ob ? stage1 : stage0, upool + (int64_t)(w2 >> 24) * 16, (unsigned)((w2 & 0xFFFFFFull) * 16),
-                      &M.mbar[ob]);
-            go = 1;
-          }
-          go = __shfl_sync(0xffffffffu, go, 0);
-          if (go) {
-            if (ob) {
-              btag1 = knext;
-              bpend1 = true;
-            } else {
-              btag0 = knext;
-              bpend0 = true;
-            }
-          }
+        dropped = d != 0;
+      }
+      // this record came ahead of its step: the next one's, if its row was
+      // published at the start of the step and a buffer is free
+      if (want_pf && !fetched) {
+        const int ob = btag0 < 0 ? 0 : (btag1 < 0 ? 1 : -1);
+        w2 = __shfl_sync(0xffffffffu, w2, 0);
+        if (ob >= 0 && w2 != 0 && w2 != kRowFailed && (int64_t)(w2 & 0xFFFFFFull) * 16 <= g.stage) {
+          asm volatile("fence.acq_rel.gpu;" ::: "memory");
+          record_fetch(ob ? stage1 : stage0, upool + (int64_t)(w2 >> 24) * 16, (int)((w2 & 0xFFFFFFull) * 16), lane);
+          (ob ? btag1 : btag0) = knext;
         }
-        if (dropped) {
-          if (lane == 0) sstate[sk] = SL_DEAD;
-          __syncwarp();
-          if (bi == 0) btag0 = -1;
-          if (bi == 1) btag1 = -1;
-          continue;
-        }
-        if (lane == 0) {
-          sstate[sk] = SL_LKEPT;
-          sf2[sk] = key;
-        }
+      }
+      if (dropped) {
+        if (lane == 0) sstate[sk] = SL_DEAD;
         __syncwarp();
-        // U row k in chunks of 32 blocks: look up or create the target blocks
-        // (probe, then place, separated by __syncwarp), then update all
-        // elements of the chunk with lanes spread over the flattened elements.
-        for (int q0 = 0; q0 < ucnt && status_local == 0; q0 += 32) {
-          const int q = q0 + lane;
-          int32_t j = -1;
-          int slot = -1;
-          int uo = 0, njq = 0;
-          bool missing = false;
-          if (q < ucnt) {
-            j = staged ? rcol[q] : __ldcg(rcol + q);
-            uo = staged ? rrel[q] : __ldcg(rrel + q);
-            njq = staged ? rnj[q] : __ldcg(rnj + q);
-            if (j <= k || j >= A.nbr || uo < 0 || njq <= 0 || (int64_t)uo + (int64_t)nk * njq > uval_n) {
-              *vflag = 4;  // a published U block lies right of k inside its record
-              j = -1;
-            } else {
-              slot = ws_lookup(keys, scol, hmask, j);
-              missing = slot < 0;
-            }
+        if (bi != 1) btag0 = -1;
+        if (bi != 0) btag1 = -1;
+        continue;
+      }
+      if (lane == 0) {
+        sstate[sk] = SL_LKEPT;
+        if (F32) sf2[sk] = key;
+      }
+      __syncwarp();
+      // U row k in chunks of 32 blocks: look up or create the target blocks
+      // (probe, then place, separated by __syncwarp), then update.
+#pragma unroll 1
+      for (int q0 = 0; q0 < ucnt && status_local == 0; q0 += 32) {
+        const int q = q0 + lane;
+        const int nq = min(32, ucnt - q0);
+        int32_t j = -1;
+        int slot = -1;
+        int cst = 0, nj = 0;
+        bool missing = false, bad = false;
+        if (q < ucnt) {
+          j = staged ? rcol[q] : __ldcg(rcol + q);
+          cst = staged ? rcst[q] : __ldcg(rcst + q);
+          nj = staged ? rnj[q] : __ldcg(rnj + q);
+          // a published U block lies right of k inside its record
+          bad = j <= k || j >= A.nbr || cst < 0 || nj <= 0 || (int64_t)cst + nj > ncol;
+          if (!bad) {
+            slot = ws_lookup(keys, scol, hmask, j);
+            missing = slot < 0;
           }
-          __syncwarp();
-          // A shared working row that this chunk's new blocks would overflow
-          // moves to the warp's global workspace first: slot numbers (so the
-          // pending L columns and the lookups above), value offsets and the
-          // multiplier's values stay as they are; the global hash is rebuilt.
-          // (When the global workspace is too small as well, the creation
-          // below fails and the row takes the overflow path.)
-          if (in_sh) {
-            const unsigned mm = __ballot_sync(0xffffffffu, missing);
-            if (mm) {
-              const int add_s = __popc(mm);
-              const int add_v = warp_sum_i(missing ? ni * njq : 0);
-              const int ns0 = *vns;
-              const long long nv0 = (long long)M.nvals;
-              if ((ns0 + add_s > smax_c || nv0 + add_v > vmax_c) && ns0 + add_s <= ws.smax &&
-                  nv0 + add_v <= ws.vmax) {
-                int* const gh = ws.hpos + wid * ws.smax;
-                int* const gc = ws.scol + wid * ws.smax;
-                int* const go = ws.soff + wid * ws.smax;
-                int* const gs = ws.sstate + wid * ws.smax;
-                long long* const gf = ws.sf2 + wid * ws.smax;
-                int* const gn = ws.sncl + wid * ws.smax;
-                T* const gv = wvals_all + wid * ws.vmax;
-                for (int q = lane; q < ns0; q += 32) {
-                  gc[q] = scol[q];
-                  go[q] = soff[q];
-                  gs[q] = sstate[q];
-                  gf[q] = sf2[q];
-                  gn[q] = sncl[q];
-                }
-                for (long long e = lane; e < nv0; e += 32) gv[e] = wv[e];
-                __syncwarp();
-                const uint32_t gmask = (uint32_t)ws.ht - 1;
-                for (int q = lane; q < ns0; q += 32) gh[q] = ws_place(gkeys, gmask, q, gc[q]);
-                for (int q = lane; q < g.hash; q += 32) sh_keys[q] = -1;
-                __syncwarp();
-                keys = gkeys, hpos = gh, scol = gc, soff = go, sstate = gs, sf2 = gf, sncl = gn;
-                wv = gv;
-                smax_c = ws.smax, vmax_c = ws.vmax, hmask = gmask;
-                in_sh = false;
-                m = wv + soff[sk];
-                if (!mb) msrc = m;
-              }
-            }
-          }
-          if (missing) {
-            const int sz = ni * njq;
-            slot = ws_new_slot(smax_c, vmax_c, keys, hpos, scol, soff, sstate, sncl, &M.nslots, &M.nvals, hmask, j,
-                               njq, sz);
-            if (slot < 0) {
-              *vflag = 1;
-            } else {
-              T* z = wv + soff[slot];
-#pragma unroll 4
-              for (int e = 0; e < sz; ++e) z[e] = (T)0;
-              if (j < i) {  // fill in the L part: pending for a later step
-                const int pq = atomicAdd(&M.nl, 1);
-                if (pq < g.lcap) {
-                  lc[pq] = j;
-                  ls[pq] = slot;
-                }
-              }
-            }
-          }
-          __syncwarp();
-          if (*vflag == 1) {
-            status_local = DEV_OVERFLOW;
-            break;
-          }
-          if (*vflag == 4) {
-            status_local = DEV_INTERNAL;
-            break;
-          }
-          const int nj = j >= 0 ? njq : 0;
-          const int sz = ni * nj;
-          int incl = sz;
+        }
+        if (__any_sync(0xffffffffu, bad)) {
+          status_local = DEV_INTERNAL;
+          break;
+        }
+        const unsigned mm = __ballot_sync(0xffffffffu, missing);
+        int off = 0;
+        if (mm) {  // new blocks: slots and values in the order of the columns
+          int incl = missing ? ni * nj : 0;
           for (int o = 1; o < 32; o <<= 1) {
             const int v = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += v;
           }
-          const int total = __shfl_sync(0xffffffffu, incl, 31);
-          M.qpre[lane] = incl - sz;
-          if (lane == 31) M.qpre[32] = total;
-          M.qoff[lane] = slot >= 0 ? soff[slot] : 0;
-          M.quo[lane] = uo;
-          M.qnj[lane] = nj;
-          __syncwarp();
-          const int nq = min(32, ucnt - q0);
-          // four elements per lane in flight
-          for (int e0 = lane; e0 < total; e0 += 128) {
-            T acc[4];
-            T* dst[4];
-            int a4[4], jj4[4], nj4[4], uo4[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int e = e0 + 32 * u;
-              dst[u] = nullptr;
-              if (e < total) {
-                int lo = 0, hi = nq - 1;  // block tq with qpre[tq] <= e < qpre[tq + 1]
-                while (lo < hi) {
-                  const int mid = (lo + hi + 1) >> 1;
-                  if (M.qpre[mid] <= e)
-                    lo = mid;
-                  else
-                    hi = mid - 1;
-                }
-                const int njt = M.qnj[lo];
-                const int local = e - M.qpre[lo];
-                a4[u] = local / njt;
-                jj4[u] = local - a4[u] * njt;
-                nj4[u] = njt;
-                uo4[u] = M.quo[lo];
-                dst[u] = wv + M.qoff[lo] + local;
-                acc[u] = *dst[u];
-              }
+          const int add_v = __shfl_sync(0xffffffffu, incl, 31), add_s = __popc(mm);
+          // A shared working row that the new blocks would overflow moves to
+          // the warp's global workspace first: slot numbers (so the pending L
+          // columns and the lookups above), value offsets and the multiplier's
+          // values stay as they are; the global hash is rebuilt.
+          if (in_sh && (ns + add_s > smax_c || nval + add_v > vmax_c) && ns + add_s <= ws.smax &&
+              nval + add_v <= ws.vmax) {
+            int* const gh = ws.hpos + wid * ws.smax;
+            int* const gc = ws.scol + wid * ws.smax;
+            int* const go = ws.soff + wid * ws.smax;
+            int* const gs = ws.sstate + wid * ws.smax;
+            long long* const gf = ws.sf2 + wid * ws.smax;
+            int* const gn = ws.sncl + wid * ws.smax;
+            T* const gv = wvals_all + wid * ws.vmax;
+#pragma unroll 1
+            for (int x = lane; x < ns; x += 32) {
+              gc[x] = scol[x];
+              go[x] = soff[x];
+              gs[x] = sstate[x];
+              gf[x] = sf2[x];
+              gn[x] = sncl[x];
             }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              if (!dst[u]) continue;
-              const T* U = rval + uo4[u];
-              T av = acc[u];
-              if (staged) {
-                for (int r = 0; r < nk; ++r) av = msub<T>(av, msrc[a4[u] * nk + r], U[r * nj4[u] + jj4[u]]);
-              } else {
-                for (int r = 0; r < nk; ++r) av = msub<T>(av, msrc[a4[u] * nk + r], __ldcg(U + r * nj4[u] + jj4[u]));
-              }
-              *dst[u] = av;
+            warp_copy(gv, (const T*)wv, nval, lane);
+            __syncwarp();
+            const uint32_t gmask = (uint32_t)ws.ht - 1;
+#pragma unroll 1
+            for (int x = lane; x < ns; x += 32) gh[x] = ws_place(gkeys, gmask, x, gc[x]);
+#pragma unroll 1
+            for (int x = lane; x < g.hash; x += 32) sh_keys[x] = -1;
+            __syncwarp();
+            keys = gkeys, hpos = gh, scol = gc, soff = go, sstate = gs, sf2 = gf, sncl = gn;
+            wv = gv;
+            smax_c = ws.smax, vmax_c = ws.vmax, hmask = gmask;
+            in_sh = false;
+            m = wv + soff[sk];
+          }
+          if (ns + add_s > smax_c || nval + add_v > vmax_c) {
+            status_local = DEV_OVERFLOW;
+            ask_s = ns + add_s;
+            ask_v = nval + add_v;
+            break;
+          }
+          if (missing) {
+            slot = ns + __popc(mm & lt);
+            off = (int)nval + incl - ni * nj;
+            scol[slot] = j;
+            soff[slot] = off;
+            sstate[slot] = SL_LIVE;
+            sncl[slot] = nj;
+            hpos[slot] = ws_place(keys, hmask, slot, j);
+          }
+          // fill in the L part: pending for a later step
+          const unsigned low = __ballot_sync(0xffffffffu, missing && j < i);
+          if (missing && j < i) {
+            const int pq = nl + __popc(low & lt);
+            if (pq < g.lcap) {
+              lc[pq] = j;
+              ls[pq] = slot;
             }
           }
-          __syncwarp();
+          const unsigned dia = __ballot_sync(0xffffffffu, missing && j == i);
+          if (dia) dslot = __shfl_sync(0xffffffffu, slot, __ffs(dia) - 1);
+          nl += __popc(low);
+          ns += add_s;
+          nval += add_v;
         }
-        if (bi == 0) btag0 = -1;
-        if (bi == 1) btag1 = -1;
-      }
-      if (status_local == DEV_OVERFLOW && in_sh) {
-        // the fill outgrew the shared workspace: start the row again in the
-        // global one (records fetched ahead stay valid)
-        for (int q = lane; q < g.hash; q += 32) sh_keys[q] = -1;
+        if (slot >= 0 && !missing) off = soff[slot];
+        const int cst0 = __shfl_sync(0xffffffffu, cst, 0);
+        const int cols = __shfl_sync(0xffffffffu, cst + nj, nq - 1) - cst0;
+        if (mb && cols <= MCOLS) {
+          if (lane < nq) {
+            qinfo[lane] = make_int4(off, cst - cst0, nj, missing ? 1 : 0);
+#pragma unroll 1
+            for (int c = 0; c < nj; ++c) cmap[cst - cst0 + c] = (unsigned char)lane;
+          }
+          __syncwarp();
+          const T* U = reinterpret_cast<const T*>(rs + RL.val) + nk * cst0;
+          if (mall) {
+            update_columns(qinfo, cmap, cols, M.mt, 0, ni, nk, np, U, wv, lane);
+          } else {
+#pragma unroll 1
+            for (int a0 = 0; a0 < ni; a0 += np) {
+              const int na = min(np, ni - a0);
+#pragma unroll 1
+              for (int e = lane; e < nk * np; e += 32) {
+                const int r = e >> (np == 16 ? 4 : 3), a = e & (np - 1);
+                M.mt[e] = a < na ? m[(a0 + a) * nk + r] : (T)0;
+              }
+              __syncwarp();
+              update_columns(qinfo, cmap, cols, M.mt, a0, na, nk, np, U, wv, lane);
+              __syncwarp();
+            }
+          }
+        } else {
+          update_general<T>(tab, nq, off, cst, nj, missing, ni, nk, m, rval, staged, wv, lane);
+        }
         __syncwarp();
-        in_sh = false;
-        continue;
       }
-      break;
+      if (bi != 1) btag0 = -1;
+      if (bi != 0) btag1 = -1;
     }
-    drain();  // every record fetched ahead has been used, unless the row failed
-    const int ns = min(*vns, smax_c);
+    record_wait<0>();  // every record fetched ahead has been used, unless the row failed
     // A row that ends in the global workspace has its slot metadata copied
     // to the shared working-row region (unused by such a row) when it fits,
     // so that the scans of the finish read on-chip data; its values stay in
@@ -1428,6 +1744,7 @@ __global__ void __launch_bounds__(256, 2)
         int* mst = mcol + ns;
         int* mncl = mst + ns;
         int* moff = mncl + ns;
+#pragma unroll 1
         for (int q = lane; q < ns; q += 32) {
           mf2[q] = sf2[q];
           mcol[q] = scol[q];
@@ -1439,248 +1756,343 @@ __global__ void __launch_bounds__(256, 2)
         sf2 = mf2, scol = mcol, sstate = mst, sncl = mncl, soff = moff;
       }
     }
-    // ---- finish the row.
-    int dslot = -1;
+    // ---- finish the row: what its dependants read first (the U part, the
+    // pivot block, the record), then publish, then the L part.
+    if (status_local == 0 && dslot < 0) status_local = DEV_ESINGULAR;
+    // candidate list of the blocks right of the diagonal, in the stage buffers
+    // when it fits beside its sorted form, else in the warp's global space
+    int nU = 0;
+    int* candU = nullptr;
+    unsigned long long* srtU = nullptr;
+    int gb_at = 0;  // first free byte of the stage buffers
     if (status_local == 0) {
-      for (int q = lane; q < ns; q += 32)
-        if (scol[q] == i && sstate[q] == SL_LIVE) dslot = q;
-      dslot = warp_max_i(dslot);
-      if (dslot < 0) status_local = DEV_ESINGULAR;
+      int p2u = 1;
+      while (p2u < ns) p2u <<= 1;
+      const int64_t need = ((4LL * ns + 15) & ~15LL) + 8LL * p2u;
+      if (need <= 2LL * g.stage) {
+        candU = reinterpret_cast<int*>(stage0);
+        srtU = reinterpret_cast<unsigned long long*>(stage0 + ((4LL * ns + 15) & ~15LL));
+        gb_at = (int)((need + 15) & ~15LL);
+      } else {
+        candU = ws.fin + wid * 2 * ws.smax;
+        srtU = ws.srt + wid * 4 * ws.smax;
+      }
+#pragma unroll 1
+      for (int q0 = 0; q0 < ns; q0 += 32) {
+        const int q = q0 + lane;
+        const bool isU = q < ns && sstate[q] == SL_LIVE && scol[q] > i;
+        const unsigned bU = __ballot_sync(0xffffffffu, isU);
+        if (isU) candU[nU + __popc(bU & lt)] = q;
+        nU += __popc(bU);
+      }
+      __syncwarp();
+      // threshold (in FP32: the norms are the lfil keys; in FP64 the keys are
+      // formed when lfil has to choose), survivors compacted
+      int kept = 0;
+#pragma unroll 1
+      for (int c0 = 0; c0 < nU; c0 += 32) {
+        const int c = c0 + lane;
+        const int q = c < nU ? candU[c] : -1;
+        bool keep = false;
+        if (q >= 0) {
+          const int nc = sncl[q], n = ni * nc;
+          const T* v = wv + soff[q];
+          if constexpr (F32) {
+            const float f2 = fro2_f32(v, n);
+            keep = !drop_rule_f(f2, ni, nc, tf);
+            sf2[q] = norm_key(f2);
+          } else {
+            float sf = 0.f;
+            bool in = n <= 4096;
+#pragma unroll 4
+            for (int e = 0; e < n; ++e) {
+              float x;
+              in = abs_f32((double)v[e], x) && in;
+              sf = __fmaf_rn(x, x, sf);
+            }
+            const int d = drop_f32(sf, in, ni, nc, tf);
+            keep = !(d < 0 ? drop_rule(fro2_batched(v, n), ni, nc, t) : d != 0);
+          }
+          if (!keep) sstate[q] = SL_DEAD;
+        }
+        const unsigned bk = __ballot_sync(0xffffffffu, keep);
+        if (keep) candU[kept + __popc(bk & lt)] = q;
+        kept += __popc(bk);
+        __syncwarp();
+      }
+      nU = kept;
+      if (lfil >= 0 && nU > lfil) {
+        if (!F32) {
+#pragma unroll 1
+          for (int c = lane; c < nU; c += 32) {
+            const int q = candU[c];
+            sf2[q] = norm_key(fro2_batched(wv + soff[q], ni * sncl[q]));
+          }
+          __syncwarp();
+        }
+        nU = lfil_cut(candU, nU, lfil, sf2, scol, sstate, M.buf, TS, lane);
+      }
+      sort_by_column(candU, nU, scol, srtU, lane);
     }
-    // GEPP of the diagonal block, in shared memory when it fits (the stage
-    // buffers are free now).  FP64 factor: FP64 in the oracle's operation
-    // order.  Mixed factor: FP32 GEPP and 1-norm condition estimate (explicit
-    // inverse columns); a block above the threshold, larger than 32, or
-    // singular in FP32 is factored again in FP64 and tagged.
-    bool tag64 = sizeof(T) == sizeof(double);
-    bool lu_sm = false;  // the FP32 pivot LU is in M.lu32
+    // the record's size and, while the pivot block is factored, its space
+    // (with an FP64 pivot LU when the factor's type or a large block asks for
+    // one; a small FP32 block that turns out to need one takes a second space)
+    int ucols = 0;
+    unsigned long long roff16 = 0;
+    int64_t rbytes = 0;
+    int lu64r = F32 && ni <= 32 ? 0 : 1;
+    if (status_local == 0) {
+#pragma unroll 1
+      for (int p = lane; p < nU; p += 32) ucols += sncl[(int)(srtU[p] & 0xffffffffu)];
+      ucols = __reduce_add_sync(0xffffffffu, ucols);
+      rbytes = rec_layout<int64_t>(nU, ni, lu64r, ucols, TS).bytes;
+      if (lane == 0) roff16 = atomicAdd(P.ctr + 2, (unsigned long long)(rbytes / 16));
+    }
+    // GEPP of the diagonal block, in registers, in shared memory when it fits
+    // (the stage buffers' free part), else in place.  FP64 factor: FP64 in the
+    // oracle's operation order.  Mixed factor: FP32 GEPP and 1-norm condition
+    // estimate (explicit inverse columns); a block above the threshold, larger
+    // than 32, or singular in FP32 is factored again in FP64 and tagged.
+    bool tag64 = !F32;
+    bool lu_sm = false;  // the pivot LU and its reciprocals are in M
+    const T* lu_g = nullptr;  // else: the FP32 pivot LU, rows lu_str apart
+    int lu_str = ni;
+    const double* lu_g64 = nullptr;
     if (status_local == 0) {
       const T* srcd = wv + soff[dslot];
-      unsigned char* gb = stage0;
-      const int gcap = 2 * g.stage;
-      const bool gs32 = ni * ni * 4 <= gcap, gs64 = ni * ni * 8 <= gcap;
+      unsigned char* gb = stage0 + gb_at;
+      const int gcap = 2 * g.stage - gb_at;
       int* pvs = ni <= PVMAX ? M.pv : nullptr;
       int32_t* gpiv = piv + A.roff[i];
       bool ok = true;
-      if (sizeof(T) == sizeof(float)) {
+      if constexpr (F32) {
         tag64 = true;
-        float* a = gs32 ? reinterpret_cast<float*>(gb) : dg32 + dgoff[i];
-        for (int e = lane; e < ni * ni; e += 32) a[e] = (float)srcd[e];
-        __syncwarp();
         float norm1 = 0.f;
+#pragma unroll 1
         for (int jj = lane; jj < ni; jj += 32) {
           float sum = 0.f;
-          for (int ii = 0; ii < ni; ++ii) sum += fabsf(a[ii * ni + jj]);
+#pragma unroll 1
+          for (int ii = 0; ii < ni; ++ii) sum += fabsf(srcd[ii * ni + jj]);
           norm1 = fmaxf(norm1, sum);
         }
         for (int o = 16; o > 0; o >>= 1) norm1 = fmaxf(norm1, __shfl_xor_sync(0xffffffffu, norm1, o));
-        __syncwarp();
-        const bool small = ni <= 8 && pvs;  // registers; M.pv holds the interchanges
-        if (small ? gepp_small(a, ni, pvs, gpiv, lane) : (ni <= 32 && gepp_warp<float>(a, ni, pvs, gpiv, lane))) {
-          const float kappa = norm1 * (small ? inv_norm1_small(a, ni, pvs, lane)
-                                             : inv_norm1_f32(a, ni, pvs ? pvs : gpiv, lane));
-          tag64 = !(kappa <= condf);
-          if (!tag64) {
-            lu_sm = small;
-            for (int e = lane; e < ni * ni; e += 32) {
-              if (gs32) dg32[dgoff[i] + e] = a[e];
-              dg[dgoff[i] + e] = (double)a[e];
-              if (small) M.lu32[e] = a[e];
-            }
+        float inv1 = 0.f;
+        if (ni <= NSMALL) {
+          if (gepp_cond<NSMALL>(srcd, ni, M.lu, M.ry, M.rz, M.pv, M.perm, gpiv, lane, &inv1)) {
+            tag64 = !(norm1 * inv1 <= condf);
+            lu_sm = !tag64;
+          }
+        } else if (ni <= NPIV && (ni <= 16 ? 1024 : 4096) <= gcap) {
+          float* a = reinterpret_cast<float*>(gb);
+          lu_str = ni <= 16 ? 16 : 32;
+          if (ni <= 16 ? gepp_cond<16>(srcd, ni, a, M.ry, M.rz, M.pv, M.perm, gpiv, lane, &inv1)
+                       : gepp_cond<32>(srcd, ni, a, M.ry, M.rz, M.pv, M.perm, gpiv, lane, &inv1)) {
+            tag64 = !(norm1 * inv1 <= condf);
+            lu_g = a;
+          }
+        } else if (ni <= 32) {
+          float* a = dg32 + dgoff[i];
+          lu_str = ni;
+#pragma unroll 1
+          for (int e = lane; e < ni * ni; e += 32) a[e] = srcd[e];
+          __syncwarp();
+          if (gepp_warp<float>(a, ni, pvs, gpiv, lane)) {
+            tag64 = !(norm1 * inv_norm1_f32(a, ni, pvs, lane) <= condf);
+            lu_g = a;
           }
         }
         __syncwarp();
       }
       if (tag64) {
-        double* a = gs64 ? reinterpret_cast<double*>(gb) : dg + dgoff[i];
+        double* a = ni * ni * 8 <= gcap ? reinterpret_cast<double*>(gb) : dg + dgoff[i];
+#pragma unroll 1
         for (int e = lane; e < ni * ni; e += 32) a[e] = (double)srcd[e];
         __syncwarp();
         ok = gepp_warp<double>(a, ni, pvs, gpiv, lane);
-        if (ok)
-          for (int e = lane; e < ni * ni; e += 32) {
-            if (gs64) dg[dgoff[i] + e] = a[e];
-            if (mixed) dg32[dgoff[i] + e] = (float)a[e];
-          }
+        lu_g64 = a;
       }
       __syncwarp();
       if (!ok)
         status_local = DEV_ESINGULAR;
-      else if (mixed && lane == 0)
-        ptag[i] = tag64 ? 1 : 0;
+      else if ((tag64 || lu_str == ni) && !lu_sm && ni <= PVMAX)
+        perm_of(M.pv, ni, M.perm, lane);
     }
-    // U part: threshold on the blocks right of the diagonal (norm keys kept
-    // for lfil)
+    // the space, with what the pivot block turned out to need
     if (status_local == 0) {
-      for (int q = lane; q < ns; q += 32) {
-        const int c = scol[q];
-        if (sstate[q] == SL_LIVE && c > i) {
-          const int nc = sncl[q];
-          bool drop;
-          long long kq;
-          if (sizeof(T) == sizeof(double)) {
-            const double f2 = fro2_batched(wv + soff[q], ni * nc);
-            drop = drop_rule(f2, ni, nc, t);
-            kq = norm_key(f2);
-          } else {
-            const float f2 = fro2_f32(wv + soff[q], ni * nc);
-            drop = drop_rule_f(f2, ni, nc, tf);
-            kq = norm_key(f2);
-          }
-          sf2[q] = kq;
-          if (drop) sstate[q] = SL_DEAD;
-        }
+      if (F32 && tag64 && !lu64r) {
+        lu64r = 1;
+        rbytes = rec_layout<int64_t>(nU, ni, lu64r, ucols, TS).bytes;
+        if (lane == 0) roff16 = atomicAdd(P.ctr + 2, (unsigned long long)(rbytes / 16));
       }
-      __syncwarp();
-    }
-    // candidate lists of the kept L blocks and the surviving U blocks, the
-    // lfil cut of each, then each part sorted by column; in the stage buffers
-    // when they fit, else in the warp's global finish space
-    int nL = 0, nU = 0, n2L = 0, n2U = 0;
-    int* candL = nullptr;
-    int* candU = nullptr;
-    unsigned long long* srtL = nullptr;
-    unsigned long long* srtU = nullptr;
-    if (status_local == 0) {
-      int cl = 0, cu = 0;
-      for (int q = lane; q < ns; q += 32) {
-        const int s = sstate[q];
-        cl += s == SL_LKEPT;
-        cu += s == SL_LIVE && scol[q] > i;
-      }
-      cl = warp_sum_i(cl);
-      cu = warp_sum_i(cu);
-      int p2l = 1, p2u = 1;
-      while (p2l < cl) p2l <<= 1;
-      while (p2u < cu) p2u <<= 1;
-      const int64_t need = 4LL * (cl + cu) + 8LL * (p2l + p2u) + 16;
-      if (need <= 2LL * g.stage) {
-        candL = reinterpret_cast<int*>(stage0);
-        candU = candL + cl;
-        srtL = reinterpret_cast<unsigned long long*>(stage0 + ((4LL * (cl + cu) + 15) & ~15LL));
-        srtU = srtL + p2l;
-      } else {
-        candL = ws.fin + wid * 2 * ws.smax;
-        candU = candL + ws.smax;
-        srtL = ws.srt + wid * 4 * ws.smax;
-        srtU = srtL + 2 * ws.smax;
-      }
-      for (int base = 0; base < ns; base += 32) {
-        const int q = base + lane;
-        bool isL = false, isU = false;
-        if (q < ns) {
-          const int s = sstate[q];
-          isL = s == SL_LKEPT;
-          isU = s == SL_LIVE && scol[q] > i;
-        }
-        const unsigned bL = __ballot_sync(0xffffffffu, isL), bU = __ballot_sync(0xffffffffu, isU);
-        const unsigned lt = (1u << lane) - 1u;
-        if (isL) candL[nL + __popc(bL & lt)] = q;
-        if (isU) candU[nU + __popc(bU & lt)] = q;
-        nL += __popc(bL);
-        nU += __popc(bU);
-      }
-      __syncwarp();
-      // lfil: keep the lfil largest of the L part and of the U part
-      nL = lfil_cut(candL, nL, lfil, sf2, scol, sstate, M.hist, TS, lane);
-      nU = lfil_cut(candU, nU, lfil, sf2, scol, sstate, M.hist, TS, lane);
-      n2L = sort_by_column(candL, nL, scol, srtL, lane);
-      n2U = sort_by_column(candU, nU, scol, srtU, lane);
-    }
-    // sizes, then the pool space: the U record and the L blocks
-    long long vl = 0, vu = 0;
-    unsigned long long lb = 0, lvv = 0, roff16 = 0;
-    int64_t rbytes = 0;
-    int lu64r = 0;
-    if (status_local == 0) {
-      for (int p = lane; p < nL; p += 32) vl += (long long)ni * sncl[(int)(srtL[p] & 0xffffffffu)];
-      for (int p = lane; p < nU; p += 32) vu += (long long)ni * sncl[(int)(srtU[p] & 0xffffffffu)];
-      vl = warp_sum_ll(vl);
-      vu = warp_sum_ll(vu);
-      lu64r = (sizeof(T) == sizeof(double) || tag64) ? 1 : 0;
-      const RecLayout RL = rec_layout(nU, ni, lu64r, vu, TS);
-      rbytes = RL.bytes;
-      if (lane == 0) {
-        lb = atomicAdd(P.ctr + 0, (unsigned long long)nL);
-        lvv = atomicAdd(P.ctr + 1, (unsigned long long)vl);
-        roff16 = atomicAdd(P.ctr + 2, (unsigned long long)(rbytes / 16));
-      }
-      lb = __shfl_sync(0xffffffffu, lb, 0);
-      lvv = __shfl_sync(0xffffffffu, lvv, 0);
       roff16 = __shfl_sync(0xffffffffu, roff16, 0);
-      const bool fits = (int64_t)(lb + nL) <= P.lbcap && (int64_t)(lvv + vl) <= P.lvcap &&
-                        (int64_t)roff16 + rbytes / 16 <= P.ucap16 && rbytes / 16 <= kRecMaxUnits &&
-                        vu <= INT_MAX;
-      if (!fits) status_local = DEV_OVERFLOW;
+      if ((int64_t)roff16 + rbytes / 16 > P.ucap16 || rbytes / 16 > kRecMaxUnits) status_local = DEV_OVERFLOW;
     }
-    // the U record: header, pivots, pivot LU, columns, value offsets, values
+    // the record
     if (status_local == 0) {
-      const RecLayout RL = rec_layout(nU, ni, lu64r, vu, TS);
+      const RecLayout<int> RL = rec_layout<int>(nU, ni, lu64r, ucols, TS);
       unsigned char* r = upool + (int64_t)roff16 * 16;
-      if (lane == 0) {
-        int* h = reinterpret_cast<int*>(r);
-        h[0] = nU;
-        h[1] = ni;
-        h[2] = lu64r;
-        h[3] = (int)vu;
+      if (lane == 0) *reinterpret_cast<int4*>(r) = make_int4(nU, ni, 2 * (maxdep + 1) + lu64r, ucols);
+      int* rp = reinterpret_cast<int*>(r + RL.perm);
+      if (ni <= PVMAX) {
+#pragma unroll 1
+        for (int a = lane; a < ni; a += 32) rp[a] = M.perm[a];
+      } else if (lane == 0) {  // a block of more than PVMAX rows: in place
+        const int32_t* gpiv = piv + A.roff[i];
+#pragma unroll 1
+        for (int a = 0; a < ni; ++a) rp[a] = a;
+#pragma unroll 1
+        for (int a = 0; a < ni; ++a) {
+          const int q = gpiv[a], v = rp[a];
+          rp[a] = rp[q];
+          rp[q] = v;
+        }
       }
-      const int32_t* gpiv = piv + A.roff[i];
-      for (int a = lane; a < ni; a += 32) reinterpret_cast<int*>(r + RL.piv)[a] = ni <= PVMAX ? M.pv[a] : gpiv[a];
-      for (int e = lane; e < ni * ni; e += 32) {
-        if (lu64r)
-          reinterpret_cast<double*>(r + RL.lu)[e] = dg[dgoff[i] + e];
-        else
-          reinterpret_cast<float*>(r + RL.lu)[e] = lu_sm ? M.lu32[e] : dg32[dgoff[i] + e];
+      if (lu_sm) {
+        T* o = reinterpret_cast<T*>(r + RL.lu);
+#pragma unroll 1
+        for (int e = lane; e < ni * NSMALL; e += 32) o[e] = M.lu[e];
+        T* y = reinterpret_cast<T*>(r + RL.rcp);
+        if (lane < ni) {
+          y[lane] = M.ry[lane];
+          y[ni + lane] = M.rz[lane];
+        }
+      } else if (lu64r) {
+        put_pivot(lu_g64, ni, ni, reinterpret_cast<double*>(r + RL.lu), reinterpret_cast<double*>(r + RL.rcp), lane);
+      } else {
+        put_pivot(lu_g, lu_str, ni, reinterpret_cast<T*>(r + RL.lu), reinterpret_cast<T*>(r + RL.rcp), lane);
       }
       int* rcol = reinterpret_cast<int*>(r + RL.ucol);
-      int* rrel = reinterpret_cast<int*>(r + RL.urel);
+      int* rcst = reinterpret_cast<int*>(r + RL.ucst);
       int* rnjw = reinterpret_cast<int*>(r + RL.unj);
       T* rv = reinterpret_cast<T*>(r + RL.val);
       int carry = 0;
+#pragma unroll 1
       for (int p0 = 0; p0 < nU; p0 += 32) {
         const int p = p0 + lane;
-        int sz = 0, so = 0;
+        int nc = 0, so = 0;
         if (p < nU) {
           const int c = (int)(srtU[p] >> 32), q = (int)(srtU[p] & 0xffffffffu);
-          const int nc = sncl[q];
-          sz = ni * nc;
+          nc = sncl[q];
           so = soff[q];
           rcol[p] = c;
           rnjw[p] = nc;
         }
-        int incl = sz;
+        int incl = nc;
         for (int o = 1; o < 32; o <<= 1) {
           const int v = __shfl_up_sync(0xffffffffu, incl, o);
           if (lane >= o) incl += v;
         }
-        const int rel = carry + incl - sz;
-        if (p < nU) rrel[p] = rel;
-        copy_round<T>(M, sz, so, rel, wv, rv, lane);
+        const int cst = carry + incl - nc;
+        if (p < nU) rcst[p] = cst;
+        copy_blocks<T>(min(32, nU - p0), ni * nc, so, (long long)ni * cst, wv, rv, lane);
         carry += __shfl_sync(0xffffffffu, incl, 31);
       }
     }
     if (status_local != 0 && lane == 0) {
       dev_fail(st, status_local);
       atomicExch(P.abort, 1);
-      P.lcnt[i] = 0;
-      P.lstart[i] = 0;
     }
-    if (lane == 0) {  // what the row asked for, to size a retry
-      atomicMax(P.ctr + 5, M.nvals);
-      atomicMax(P.ctr + 6, (unsigned long long)M.nslots);
-    }
-    if (P.depth && lane == 0) P.depth[i] = maxdep + 1;
-    // publish the row: every lane's writes are made visible device-wide (and
-    // to the bulk copies of the readers) before lane 0 sets the word
-    fence_proxy_async_all();
+    // publish the row: every lane's writes are made visible device-wide
+    // before lane 0 sets the word
     __threadfence();
     __syncwarp();
-    if (lane == 0)
-      atomicExch(P.done + i, status_local == 0 ? ((unsigned long long)roff16 << 24) | (unsigned long long)(rbytes / 16)
-                                               : kRowFailed);
-    // the L part is read by no other row: written after publishing, in
-    // column order
+    if (lane == 0) {
+      const unsigned long long w = status_local == 0
+                                       ? ((unsigned long long)roff16 << 24) | (unsigned long long)(rbytes / 16)
+                                       : kRowFailed;
+      asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(P.done + i), "l"(w) : "memory");
+      if (ask_s) {  // to size a retry
+        atomicMax(P.ctr + 5, (unsigned long long)ask_v);
+        atomicMax(P.ctr + 6, (unsigned long long)ask_s);
+      }
+      if (P.depth) P.depth[i] = maxdep + 1;
+    }
+    // ---- what no other row reads: the pivot block as the solve takes it, then
+    // the L part
+    if (status_local == 0) {
+#pragma unroll 1
+      for (int e = lane; e < ni * ni; e += 32) {
+        if (lu_sm) {
+          const int a = e / ni;
+          const float v = (float)M.lu[a * NSMALL + e - a * ni];
+          dg32[dgoff[i] + e] = v;
+          dg[dgoff[i] + e] = (double)v;
+        } else if (tag64) {
+          const double v = lu_g64[e];
+          dg[dgoff[i] + e] = v;
+          if (mixed) dg32[dgoff[i] + e] = (float)v;
+        } else {
+          const int a = e / ni;
+          const float v = (float)lu_g[a * lu_str + e - a * ni];
+          dg32[dgoff[i] + e] = v;
+          dg[dgoff[i] + e] = (double)v;
+        }
+      }
+      if (mixed && lane == 0) ptag[i] = tag64 ? 1 : 0;
+      __syncwarp();  // the stage buffers are free now
+    }
+    int nL = 0;
+    int* candL = nullptr;
+    unsigned long long* srtL = nullptr;
+    unsigned long long lb = 0, lvv = 0;
+    if (status_local == 0) {
+      int cl = 0;
+#pragma unroll 1
+      for (int q0 = 0; q0 < ns; q0 += 32) {
+        const int q = q0 + lane;
+        cl += __popc(__ballot_sync(0xffffffffu, q < ns && sstate[q] == SL_LKEPT));
+      }
+      int p2l = 1;
+      while (p2l < cl) p2l <<= 1;
+      if (((4LL * cl + 15) & ~15LL) + 8LL * p2l <= 2LL * g.stage) {
+        candL = reinterpret_cast<int*>(stage0);
+        srtL = reinterpret_cast<unsigned long long*>(stage0 + ((4LL * cl + 15) & ~15LL));
+      } else {
+        candL = ws.fin + wid * 2 * ws.smax;
+        srtL = ws.srt + wid * 4 * ws.smax;
+      }
+#pragma unroll 1
+      for (int q0 = 0; q0 < ns; q0 += 32) {
+        const int q = q0 + lane;
+        const bool isL = q < ns && sstate[q] == SL_LKEPT;
+        const unsigned bL = __ballot_sync(0xffffffffu, isL);
+        if (isL) candL[nL + __popc(bL & lt)] = q;
+        nL += __popc(bL);
+      }
+      __syncwarp();
+      if (lfil >= 0 && nL > lfil) {
+        if (!F32) {
+#pragma unroll 1
+          for (int c = lane; c < nL; c += 32) {
+            const int q = candL[c];
+            sf2[q] = norm_key(fro2_batched(wv + soff[q], ni * sncl[q]));
+          }
+          __syncwarp();
+        }
+        nL = lfil_cut(candL, nL, lfil, sf2, scol, sstate, M.buf, TS, lane);
+      }
+      sort_by_column(candL, nL, scol, srtL, lane);
+      long long vl = 0;
+#pragma unroll 1
+      for (int p = lane; p < nL; p += 32) vl += (long long)ni * sncl[(int)(srtL[p] & 0xffffffffu)];
+      vl = warp_sum_ll(vl);
+      if (lane == 0) {
+        lb = atomicAdd(P.ctr + 0, (unsigned long long)nL);
+        lvv = atomicAdd(P.ctr + 1, (unsigned long long)vl);
+      }
+      lb = __shfl_sync(0xffffffffu, lb, 0);
+      lvv = __shfl_sync(0xffffffffu, lvv, 0);
+      if ((int64_t)(lb + nL) > P.lbcap || (int64_t)(lvv + vl) > P.lvcap) {
+        status_local = DEV_OVERFLOW;
+        if (lane == 0) {
+          dev_fail(st, status_local);
+          atomicExch(P.abort, 1);
+        }
+      }
+    }
     if (status_local == 0) {
       long long carry = 0;
+#pragma unroll 1
       for (int p0 = 0; p0 < nL; p0 += 32) {
         const int p = p0 + lane;
         int sz = 0, so = 0;
@@ -1697,28 +2109,27 @@ __global__ void __launch_bounds__(256, 2)
         }
         const long long dof = (long long)lvv + carry + incl - sz;
         if (p < nL) P.lvo[lb + p] = dof;
-        copy_round<T>(M, sz, so, dof, wv, lval, lane);
+        copy_blocks<T>(min(32, nL - p0), sz, so, dof, wv, lval, lane);
         carry += __shfl_sync(0xffffffffu, incl, 31);
       }
-      if (lane == 0) {
-        P.lstart[i] = (int64_t)lb;
-        P.lcnt[i] = nL;
-      }
     }
-    (void)n2L;
-    (void)n2U;
+    if (lane == 0) {
+      P.lstart[i] = status_local == 0 ? (int64_t)lb : 0;
+      P.lcnt[i] = status_local == 0 ? nL : 0;
+    }
     // clear the hash positions this row used (and the shared hash when the
     // finish staged metadata over it)
     if (in_sh || meta_sh) {
+#pragma unroll 1
       for (int q = lane; q < g.hash; q += 32) sh_keys[q] = -1;
     }
     if (!in_sh) {
+#pragma unroll 1
       for (int q = lane; q < ns; q += 32)
         if (hpos[q] >= 0) keys[hpos[q]] = -1;
     }
     __syncwarp();
   }
-  drain();
 }
 
 // Gather the pooled L rows into VBCSR (warp per row).
@@ -1762,14 +2173,15 @@ __global__ void k_rec_to_vb(int64_t nbr, int pass, const unsigned long long* __r
       if (lane == 0) cnt[i] = ucnt;
       continue;
     }
-    const RecLayout RL = rec_layout(ucnt, h[1], h[2], h[3], (int)sizeof(T));
+    const RecLayout<int> RL = rec_layout<int>(ucnt, h[1], h[2] & 1, h[3], (int)sizeof(T));
     if (pass == 1) {
       for (int q = lane; q < ucnt; q += 32) bcol[bptr[i] + q] = reinterpret_cast<const int*>(r + RL.ucol)[q];
       continue;
     }
     const T* src = reinterpret_cast<const T*>(r + RL.val);
     T* dst = val + voff[bptr[i]];
-    for (int e = lane; e < h[3]; e += 32) dst[e] = src[e];
+    const int64_t n = (int64_t)h[3] * h[1];
+    for (int64_t e = lane; e < n; e += 32) dst[e] = src[e];
   }
 }
 
@@ -1814,6 +2226,7 @@ __global__ void k_row_stats(int64_t nbr, const int64_t* __restrict__ bptr, unsig
 
 // Shared workspace of one warp: slots, value bytes, stage-buffer bytes and
 // pending-column capacity, every part 16-byte aligned.
+template <typename T>
 static IlutGeom make_geom(int slots, int vbytes, int stage, int lcap) {
   IlutGeom G{};
   G.slots = slots;
@@ -1825,7 +2238,7 @@ static IlutGeom make_geom(int slots, int vbytes, int stage, int lcap) {
   auto up = [](int v, int a) { return (v + a - 1) / a * a; };
   int o = 0;
   G.o_misc = o;
-  o = up(o + (int)sizeof(IlutMisc), 128);
+  o = up(o + (int)sizeof(IlutMisc<T>), 128);
   G.o_stage = o;
   o += 2 * stage;
   G.o_vals = o;
@@ -1919,11 +2332,17 @@ void ilut_last(LastDev<T>& X, double t, int lfil, bool mixed, double cond_thr, u
   // the candidates below on a prefix of this matrix's own tickets (every
   // prefix of the ticket order is factored exactly on its own), the fastest
   // kept per device, precision and class of row sizes for the rest of the
-  // process; small matrices take the measured default.  The candidates span
-  // what the configured workloads were measured to prefer: 64 or 128 slots,
-  // 2 to 8 KB of values, 16 down to 6 warps per SM.  The prefix is 1/64 of
-  // the tickets (2 048 to 16 384), so the two or three timings add at most about
-  // 5 % to the first factorization of a class.
+  // process; small matrices take the first.  What counts is that records and
+  // working rows stay on chip; the rows in flight then matter little (3.0
+  // million unknowns FP32, the whole factorization, slots / value bytes / stage
+  // bytes: 64 / 6 144 / 3 072, 8 warps an SM, 709 ms; 128 / 8 192 / 4 096, 8
+  // warps, 671; 128 / 12 288 / 4 096, 7 warps, 644; 128 / 16 384 / 6 144, 5
+  // warps, 677).  FP64 rows hold twice the bytes (360 000 unknowns: 128 / 8 192
+  // / 6 144, 7 warps, 382 ms; 128 / 16 384 / 6 144, 5 warps, 339); rows of many
+  // small blocks need slots (48 000 unknowns at tau 0.9: 512 / 8 192 / 4 096
+  // 527 ms; 512 / 16 384 487; 768 / 16 384, 3 warps, 454).  The prefix is 1/64
+  // of the tickets (2 048 to 16 384), so the timings add at most about 5 % to
+  // the first factorization of a class.
   DBuf<unsigned long long> rstat(2, s);
   rstat.zero();
   launch(k_row_stats, grid_for(p, 256), 256, 0, s, p, A.bptr.p, rstat.p);
@@ -1932,13 +2351,9 @@ void ilut_last(LastDev<T>& X, double t, int lfil, bool mixed, double cond_thr, u
   const bool wide = rs[0] * 4 > (unsigned long long)p;
   const bool f64 = sizeof(T) == sizeof(double);
   std::vector<IlutGeom> cands;
-  cands.push_back((wide && f64) ? make_geom(128, 8192, 2048, 256) : make_geom(64, 2048, 2048, wide ? 256 : 128));
-  cands.push_back(make_geom(64, 4096, 2048, 128));
-  // Fewer warps per SM means fewer rows in flight; a prefix under-weights
-  // that window, which a matrix of narrow rows depends on (on the 3M-unknown
-  // workload the prefix preferred 12 warps per SM, which ran the whole matrix
-  // 12 % slower than 16), so only wide rows also time the 128-slot shape.
-  if (wide) cands.push_back(make_geom(128, f64 ? 8192 : 4096, 2048, 256));
+  if (wide) cands.push_back(make_geom<T>(768, 16384, 4096, 512));
+  cands.push_back(make_geom<T>(128, f64 ? 16384 : 12288, f64 ? 6144 : 4096, wide ? 256 : 128));
+  if (!wide) cands.push_back(make_geom<T>(128, 8192, f64 ? 6144 : 4096, 128));
   const int reserve = 1024;  // shared memory the system keeps per block
   // warps per block and blocks per SM of a geometry: the most warps per SM
   // (at most 16)
@@ -1947,7 +2362,7 @@ void ilut_last(LastDev<T>& X, double t, int lfil, bool mixed, double cond_thr, u
     for (int w = 8; w >= 1; --w) {
       if (w * G.bytes > smem_block) continue;
       int b = smem_sm / (w * G.bytes + reserve);
-      while (w * b > 16) --b;
+      while (w * b > 8) --b;
       if (b >= 1 && w * b > wpb * bps) wpb = w, bps = b;
     }
     return wpb >= 1;
@@ -1956,7 +2371,7 @@ void ilut_last(LastDev<T>& X, double t, int lfil, bool mixed, double cond_thr, u
   // about half of the last-level matrix on the configured workloads; the
   // pools start at its full size and grow on overflow (retry)
   int64_t lbcap = std::max<int64_t>(A.nnzb, 1024), lvcap = std::max<int64_t>(A.nval, 1 << 16);
-  int64_t ucap16 = (A.nval * (int64_t)sizeof(T) + X.Dg.nval * 8 + 8 * A.nnzb + 64 * p) / 16 + 4096;
+  int64_t ucap16 = (A.nval * (int64_t)sizeof(T) + X.Dg.nval * 8 + 8 * A.nnzb + 16 * n + 96 * p) / 16 + 4096;
   int smax = 1024;
   int64_t vmax = 32768;
   // buffers of one launch
