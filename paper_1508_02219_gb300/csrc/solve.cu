@@ -1154,7 +1154,7 @@ void sweep_last(const PrecDev<T>& P, const SolveBufs& B, const double* g, double
   launch(k_tri<T, false, R>, nb, TRI_W * 32, smem, s, last.L.view(), nullptr, nullptr, nullptr, nullptr, nullptr, g,
          last.r.p, (R*)B.recf, B.yy, B.yy, last.lorder.p, B.tick, B.abort, (unsigned long long)P.wait_limit,
          P.status.p, nullptr, nullptr);
-  if (B.recb == B.recf) VB_CUDA(cudaMemsetAsync(B.recb, 0xff, rec_words<R>(n, p) * sizeof(R), s));
+  if (B.recb == B.recf) VB_CUDA(cudaMemsetAsync(B.recb, 0xff, B.clear_bytes, s));
   launch(k_tri<T, true, R>, nb, TRI_W * 32, smem, s, last.U.view(), last.Dg.voff.p, last.Dg.val.p,
          sizeof(T) == sizeof(float) ? last.Dg32.val.p : nullptr, last.ptag.p, last.piv.p, B.yy, last.c.p, (R*)B.recb,
          B.xx, z, last.uorder.p, B.tick + 1, B.abort, (unsigned long long)P.wait_limit, P.status.p, fixed, fixv);
@@ -1353,7 +1353,7 @@ void PrecDev<T>::solve_scratch(const double* x, double* y, unsigned char* scratc
   SolveBufs B{};
   // FP64 records, shared by the two sweeps: no more scratch than their flags took
   B.recf = B.recb = B.clear = scratch + sp.rec;
-  B.clear_bytes = rec_words<double>(nl_last, last.A.nbr) * 8;
+  B.clear_bytes = (size_t)(nl_last + last.A.nbr) * 8;  // exactly: y follows
   B.yy = wp;
   wp += nl_last;
   for (int l = 0; l < nl; ++l) {

@@ -105,3 +105,15 @@ def test_sweeps_zero_and_tiny_right_hand_sides():
     for e in (-60, 60):
         assert np.array_equal(_apply(V, P32, np.ldexp(x, e)), np.ldexp(y32, e))
     assert not _apply(V, P, 0.0 * x).any() and not _apply(V, P32, 0.0 * x).any()
+
+
+@pytest.mark.parametrize("nb", [1, 2, 31, 32, 33, 64, 257])
+def test_level_orders_of_few_rows(nb):
+    """The order that the sweeps take their rows in is computed 32 rows to a
+    warp: whole and partial groups, chains inside one group."""
+    V = vb()
+    m = _matrix(1, 3, nb, 2, seed=nb)
+    P = V.vbarms_factor(V.vbarms_vbsr_from_blocks(*m), 0, 0.0, -1)
+    x = np.random.default_rng(nb).standard_normal(int(m[0].sum()))
+    yo = oracle.Prec(oracle.VBMat(m[0], m[0], *m[1:]), 0, 0.0, -1).apply(x)
+    assert np.linalg.norm(_apply(V, P, x) - yo) <= 1e-12 * np.linalg.norm(yo)
