@@ -39,7 +39,7 @@
 // entries are corrected products with their reciprocals, the pivot search and
 // the reciprocals overlap, and FP64 drop tests are decided in FP32 where that
 // is certain.  The kernel's time before and now: 3.0 million unknowns FP32 710
-// and 416 ms, 360 000 FP64 498 and 270 ms, 48 000 at tau 0.9 786 and 270 ms.
+// and 392 ms, 360 000 FP64 498 and 266 ms, 48 000 at tau 0.9 786 and 267 ms.
 //
 // A wait that runs out sets VB_ETIMEOUT and raises an abort flag; a row that
 // failed publishes kRowFailed so that its dependants stop too.  Overflowing a
@@ -2636,12 +2636,21 @@ namespace {
 
 // Level of every row in the dependency DAG of a triangular block pattern:
 // lev[i] = 1 + max lev[k] over the row's block columns k (0 without
-// blocks).  Warps of a persistent grid take the rows in dependency order
-// (forward, for L: ascending, every column below the row; backward, for U:
-// descending, every column above) and spin, bounded, on the columns' words:
-// a row publishes lev + 1 (-1 when it failed) in its word with one atomic
-// store, so the word is both flag and value and needs no fence.  The first
-// half of the grid does L, the second U, at the same time.
+// blocks).  The warps of a persistent grid take 32 rows at a time in dependency
+// order (forward, for L: ascending, every column below the row; backward, for
+// U: descending, every column above), one row a lane; every turn of the warp
+// each lane looks once at the column it stands at, so rows of one warp may
+// depend on one another.  A row publishes lev + 1 (-1 when it failed) in its
+// word with one store, so the word is both flag and value and needs no fence.
+// The lanes take their columns from the far end to the near one, which is ready
+// last.  The first half of the grid does L, the second U, at the same time.
+//
+// Bound: the DAG's depth times a hop through L2, while enough rows are in
+// flight: consecutive rows depend on one another, so a window of a warp per row
+// (4 864 rows a side) kept the whole at the pace of the rows' order.  With a
+// lane per row (78 000 a side) 3.0 million unknowns (327 000 rows, 2 650 levels)
+// take 3 ms instead of 15.7, a batch of 24 matrices 1.1
+// instead of 22.4, 48 000 unknowns at tau 0.9 3.8 instead of 9.0.
 struct DagSide {
   int64_t p;
   const int64_t* bptr;
@@ -2651,54 +2660,62 @@ struct DagSide {
   int* depth;
 };
 
-// The published word, or 0 when the wait gave up (abort raised elsewhere, or
-// limit ns passed: DEV_ETIMEOUT recorded and abort raised).
-__device__ __forceinline__ int dag_wait(const int32_t* w, int* abort, unsigned long long limit, int* st) {
-  int v = ld_relaxed_gpu(w);
-  if (v == 0) {
-    const unsigned long long t0 = global_ns();
-    for (unsigned it = 1;; ++it) {
-      v = ld_relaxed_gpu(w);
-      if (v != 0) break;
+__global__ void __launch_bounds__(256)
+    k_dag_level(DagSide fw, DagSide bw, unsigned half, int* __restrict__ abort, unsigned long long limit, int* st) {
+  const bool back = blockIdx.x >= half;
+  const DagSide D = back ? bw : fw;
+  const int lane = threadIdx.x & 31;
+  int deepest = 0;
+  for (;;) {
+    long long t = 0;
+    if (lane == 0) t = (long long)atomicAdd(D.tick, 1ULL);
+    t = __shfl_sync(0xffffffffu, t, 0) * 32 + lane;
+    if (!__any_sync(0xffffffffu, t < D.p)) break;
+    const int64_t i = back ? D.p - 1 - t : t;
+    bool wait = t < D.p;
+    int64_t b = 0;
+    int left = 0, l = 0;
+    if (wait) {  // from the first block (L) or the last one (U) to the row's other end
+      b = back ? D.bptr[i + 1] - 1 : D.bptr[i];
+      left = (int)(D.bptr[i + 1] - D.bptr[i]);
+    }
+    unsigned long long t0 = 0;
+    for (unsigned it = 1; __any_sync(0xffffffffu, wait); ++it) {
+      bool moved = false;
+      if (wait) {
+        int v = 1;
+        if (left > 0) v = ld_relaxed_gpu(D.word + D.bcol[b]);
+        if (v != 0) {
+          moved = true;
+          if (left > 0) l = max(l, v);  // v = lev[k] + 1
+          b += back ? -1 : 1;
+          --left;
+          if (left <= 0 || v < 0) {
+            if (v > 0) deepest = max(deepest, l + 1);
+            asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(D.word + i), "r"(v < 0 ? -1 : l + 1) : "memory");
+            wait = false;
+          }
+        }
+      }
+      if (__any_sync(0xffffffffu, moved)) {
+        t0 = 0;
+        continue;
+      }
+      __nanosleep(32);
       if ((it & 63) == 0) {
-        if (*((volatile int*)abort) != 0) return 0;
-        if (global_ns() - t0 > limit) {
+        if (*((volatile int*)abort) != 0) return;
+        const unsigned long long now = global_ns();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > limit) {
           dev_fail(st, DEV_ETIMEOUT);
           atomicExch(abort, 1);
-          return 0;
+          return;
         }
       }
     }
   }
-  return v;
-}
-
-__global__ void k_dag_level(DagSide fw, DagSide bw, unsigned half, int* __restrict__ abort, unsigned long long limit,
-                            int* st) {
-  const bool back = blockIdx.x >= half;
-  const DagSide D = back ? bw : fw;
-  const int lane = threadIdx.x & 31;
-  for (;;) {
-    long long t = 0;
-    if (lane == 0) t = (long long)atomicAdd(D.tick, 1ULL);
-    t = __shfl_sync(0xffffffffu, t, 0);
-    if (t >= D.p) break;
-    const int64_t i = back ? D.p - 1 - t : t;
-    int l = 0, bad = 0;
-    for (int64_t b = D.bptr[i] + lane; b < D.bptr[i + 1]; b += 32) {
-      const int v = dag_wait(D.word + D.bcol[b], abort, limit, st);
-      if (v <= 0)
-        bad = 1;
-      else
-        l = max(l, v);  // v = lev[k] + 1
-    }
-    l = warp_max_i(l);
-    bad = __any_sync(0xffffffffu, bad);
-    if (lane == 0) {
-      if (!bad) atomicMax(D.depth, l + 1);
-      atomicExch(D.word + i, bad ? -1 : l + 1);
-    }
-  }
+  deepest = warp_max_i(deepest);
+  if (lane == 0 && deepest) atomicMax(D.depth, deepest);
 }
 
 // word = lev + 1 -> lev
@@ -2775,7 +2792,7 @@ void level_orders(LastDev<T>& X, uint64_t wait_limit, int* dst, cudaStream_t s) 
   int dev = 0, nsm = 0;
   VB_CUDA(cudaGetDevice(&dev));
   VB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const unsigned half = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)nsm * 4, (p + 7) / 8));
+  const unsigned half = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)nsm * 2, (p + 255) / 256));
   DagSide fw{p, X.L.bptr.p, X.L.bcol.p, lev.p, tick.p, dmax.p};
   DagSide bw{p, X.U.bptr.p, X.U.bcol.p, lev.p + p, tick.p + 1, dmax.p + 1};
   launch(k_dag_level, 2 * half, 256, 0, s, fw, bw, half, abort.p, (unsigned long long)wait_limit, dst);
