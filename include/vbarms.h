@@ -32,8 +32,10 @@
  *  - Vectors given to vbarms_apply / fgmres_solve are caller-owned device
  *    arrays of doubles in the ORIGINAL (unpermuted) numbering.
  *
- * Internal scratch and factors live in device memory obtained with
- * cudaMallocAsync on the handle's stream.
+ * Internal scratch and factors live in device memory taken, in stream order on
+ * the handle's stream, from a memory pool of the library's own (one per
+ * device).  A pool keeps at most an eighth of its device's memory unused while
+ * any handle lives, and a 256th after the last one is destroyed.
  */
 #ifndef VBARMS_H
 #define VBARMS_H

@@ -11,6 +11,7 @@
 using namespace vb;
 
 struct vbarms_vbsr_st {
+  PoolUser pool;  // first member: released after the buffers
   cudaStream_t s = nullptr;
   int dev = 0;  // the device current when the handle was created
   Compressed C;
@@ -896,8 +897,11 @@ void vbarms_vbsr_destroy(vbarms_vbsr A) {
   if (!A) return;
   try {
     DeviceScope ds(A->dev);
-    cudaStreamSynchronize(A->s);
+    const int dev = A->dev;
+    const cudaStream_t s = A->s;
+    cudaStreamSynchronize(s);
     delete A;
+    pool_idle(dev, s);
   } catch (const Error&) {
     delete A;
   }
@@ -911,8 +915,11 @@ void vbarms_prec_destroy(vbarms_prec M) {
   }
   try {
     DeviceScope ds(M->impl->dev);
-    cudaStreamSynchronize(M->impl->s);
+    const int dev = M->impl->dev;
+    const cudaStream_t s = M->impl->s;
+    cudaStreamSynchronize(s);
     delete M;
+    pool_idle(dev, s);
   } catch (const Error&) {
     delete M;
   }

@@ -226,6 +226,7 @@ void scatter_dev(double* y, const double* x, const int32_t* idx, int64_t n, cuda
 // factorization (then its rows are [off, off + len) of the batch's original
 // numbering and impl is shared by the batch).
 struct vbarms_prec_st {
+  vb::PoolUser pool;  // first member: released after the buffers
   std::shared_ptr<vb::PrecBase> impl;
   int64_t off = 0;
   int64_t len = -1;  // -1: the whole factorization

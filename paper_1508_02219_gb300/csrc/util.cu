@@ -1,4 +1,6 @@
 // Host/device plumbing: status word readback, prefix sums, partitions.
+#include <mutex>
+
 #include "common.cuh"
 
 namespace vb {
@@ -14,6 +16,77 @@ int current_device() {
   int d = 0;
   VB_CUDA(cudaGetDevice(&d));
   return d;
+}
+
+// --------------------------------------------------------------------------
+// The device memory pools, one per device, made on first use.  cudaMemPool_t
+// is safe with any number of threads and streams.
+namespace {
+constexpr int kPoolDevices = 64;
+std::mutex g_pool_mu;
+struct DevPool {
+  cudaMemPool_t pool = nullptr;
+  size_t idle = 0;  // bytes it may keep when no handle lives
+} g_pool[kPoolDevices];
+std::atomic<long long> g_pool_users{0};
+
+cudaError_t pool_of(int dev, cudaMemPool_t* out) {
+  if (dev < 0 || dev >= kPoolDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  DevPool& D = g_pool[dev];
+  if (!D.pool) {
+    size_t avail = 0, total = 0;
+    cudaError_t e = cudaMemGetInfo(&avail, &total);
+    if (e != cudaSuccess) return e;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    e = cudaMemPoolCreate(&p, &props);
+    if (e != cudaSuccess) return e;
+    uint64_t keep = total / 8;
+    e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e != cudaSuccess) {
+      cudaMemPoolDestroy(p);
+      return e;
+    }
+    D.pool = p;
+    D.idle = total / 256;
+  }
+  *out = D.pool;
+  return cudaSuccess;
+}
+}  // namespace
+
+cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
+  int dev = 0;
+  cudaMemPool_t pool = nullptr;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = pool_of(dev, &pool);
+  if (e != cudaSuccess) return e;
+  e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  if (e == cudaErrorMemoryAllocation) {  // what the pool holds unused may be in pieces: give it back and try again
+    (void)cudaGetLastError();
+    (void)cudaStreamSynchronize(s);
+    (void)cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(p, bytes, pool, s);
+  }
+  return e;
+}
+
+PoolUser::PoolUser() { g_pool_users.fetch_add(1); }
+PoolUser::~PoolUser() { g_pool_users.fetch_sub(1); }
+
+void pool_idle(int dev, cudaStream_t s) {
+  if (dev < 0 || dev >= kPoolDevices || g_pool_users.load() != 0) return;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  const DevPool& D = g_pool[dev];
+  uint64_t held = 0;
+  if (D.pool && cudaMemPoolGetAttribute(D.pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+      held > D.idle && cudaStreamSynchronize(s) == cudaSuccess)
+    (void)cudaMemPoolTrimTo(D.pool, D.idle);
+  (void)cudaGetLastError();
 }
 
 void check_status(int* dst, cudaStream_t s, const char* where) {
