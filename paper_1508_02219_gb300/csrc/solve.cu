@@ -36,6 +36,116 @@ __global__ void k_scatter_scale(int64_t n, const int32_t* __restrict__ sp, const
   }
 }
 
+// (double)v by integer operations (normal values; the conversion instruction
+// takes the FP64 unit).
+__device__ __forceinline__ double tri_widen(float v) {
+  const unsigned u = (unsigned)__float_as_int(v);
+  if ((u & 0x7f800000u) - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+  return (double)v;
+}
+__device__ __forceinline__ double tri_widen(double v) { return v; }
+
+// a / b correctly rounded from y = RN(1/b) and z, the rest of 1/b (tri_recip):
+// q0 = a y + a z is within one ulp of a / b, a - b q0 is exact, and the
+// correction by it rounds to RN(a / b) (Markstein's theorem; exact remainder
+// and correctly rounded reciprocal).  Four operations instead of a division's
+// 84 (FP32) or 560 (FP64) cycles.  Operands outside the range where no
+// intermediate can underflow or overflow (y = 0 marks such a b) are divided.
+__device__ __forceinline__ void tri_recip(float b, float& y, float& z) {
+  y = 0.f, z = 0.f;
+  if (fabsf(b) >= 0x1p-40f && fabsf(b) <= 0x1p40f) {
+    y = __frcp_rn(b);
+    z = __fmul_rn(__fmaf_rn(-b, y, 1.f), y);
+  }
+}
+__device__ __forceinline__ void tri_recip(double b, double& y, double& z) {
+  y = 0.0, z = 0.0;
+  if (fabs(b) >= 0x1p-300 && fabs(b) <= 0x1p300) {
+    y = __drcp_rn(b);
+    z = __dmul_rn(__fma_rn(-b, y, 1.0), y);
+  }
+}
+__device__ __forceinline__ double tri_div(double a, double b, double y, double z) {
+  const unsigned e = ((unsigned)__double2hiint(a) >> 20) & 0x7ff;  // |a| in [2^-300, 2^300): integer compares
+  if (__double2hiint(y) != 0 && e >= 1023 - 300 && e < 1023 + 300) {
+    const double q = __fma_rn(a, y, __dmul_rn(a, z));
+    return __fma_rn(__fma_rn(-b, q, a), y, q);
+  }
+  return __ddiv_rn(a, b);
+}
+
+// The reduction levels' pivot blocks of at most PIV_R rows are solved in a
+// thread's registers, every load before the chain of operations; larger ones by
+// the warp together.  One thread's walk through the largest block, one global
+// load after another, was what each launch waited for (720 000 unknowns, up to
+// 20 rows, eight launches in an application: 60 us each, 19 forward and 45
+// backward now, where an FP64 division still costs 256 cycles a row).
+constexpr int PIV_R = 8;
+
+template <typename TL>
+__device__ __forceinline__ void pivot_forward_reg(const TL* __restrict__ lu, const int32_t* __restrict__ pv, int m,
+                                                  double* __restrict__ u) {
+  double x[PIV_R];
+  int p[PIV_R];
+  TL l[PIV_R * PIV_R];
+#pragma unroll
+  for (int k = 0; k < PIV_R; ++k)
+    if (k < m) x[k] = u[k], p[k] = pv[k];
+#pragma unroll
+  for (int i = 1; i < PIV_R; ++i)
+#pragma unroll
+    for (int k = 0; k < i; ++k)
+      if (i < m) l[i * PIV_R + k] = lu[i * m + k];
+#pragma unroll
+  for (int k = 0; k < PIV_R; ++k)
+    if (k < m) {
+#pragma unroll
+      for (int q = k + 1; q < PIV_R; ++q)
+        if (q < m && q == p[k]) {
+          const double t = x[k];
+          x[k] = x[q];
+          x[q] = t;
+        }
+    }
+#pragma unroll
+  for (int i = 1; i < PIV_R; ++i)
+    if (i < m) {
+#pragma unroll
+      for (int k = 0; k < i; ++k) x[i] = __dsub_rn(x[i], __dmul_rn(tri_widen(l[i * PIV_R + k]), x[k]));
+    }
+#pragma unroll
+  for (int k = 0; k < PIV_R; ++k)
+    if (k < m) u[k] = x[k];
+}
+
+// x <- U^{-1} u
+template <typename TL>
+__device__ __forceinline__ void pivot_backward_reg(const TL* __restrict__ lu, int m, const double* __restrict__ u,
+                                                   double* __restrict__ x) {
+  double s[PIV_R];
+  TL l[PIV_R * PIV_R];
+#pragma unroll
+  for (int k = 0; k < PIV_R; ++k)
+    if (k < m) s[k] = u[k];
+#pragma unroll
+  for (int i = 0; i < PIV_R; ++i)
+#pragma unroll
+    for (int k = i; k < PIV_R; ++k)
+      if (k < m) l[i * PIV_R + k] = lu[i * m + k];
+#pragma unroll
+  for (int i = PIV_R - 1; i >= 0; --i)
+    if (i < m) {
+#pragma unroll
+      for (int k = i + 1; k < PIV_R; ++k)
+        if (k < m) s[i] = __dsub_rn(s[i], __dmul_rn(tri_widen(l[i * PIV_R + k]), s[k]));
+      s[i] = __ddiv_rn(s[i], tri_widen(l[i * PIV_R + i]));
+    }
+#pragma unroll
+  for (int k = 0; k < PIV_R; ++k)
+    if (k < m) x[k] = s[k];
+}
+
 // u <- L^{-1} P u per pivot block (one thread per block).
 template <typename TL>
 __device__ void pivot_forward(const TL* lu, const int32_t* pv, int m, double* u) {
@@ -58,31 +168,151 @@ __device__ void pivot_backward(const TL* lu, int m, double* u) {
   }
 }
 
-__global__ void k_pivot_fwd(int64_t nD, const int32_t* __restrict__ sz, const int64_t* __restrict__ roff,
-                            const int64_t* __restrict__ voff, const double* __restrict__ lu64,
-                            const float* __restrict__ lu32, const int32_t* __restrict__ ptag,
-                            const int32_t* __restrict__ piv, double* __restrict__ u) {
-  for (int64_t y = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; y < nD; y += (int64_t)gridDim.x * blockDim.x) {
-    if (lu32 && !ptag[y])
-      pivot_forward<float>(lu32 + voff[y], piv + roff[y], sz[y], u + roff[y]);
-    else
-      pivot_forward<double>(lu64 + voff[y], piv + roff[y], sz[y], u + roff[y]);
+// Blocks of more than PIV_R and at most 32 rows: the whole warp, lane a with
+// row a.  L column by column over all rows at once; in U the products with the
+// newest unknown are formed for all rows at once (in S, the staged block, rows
+// m | 1 apart), so that only the subtractions of one row stay serial.
+template <typename TL>
+__device__ __forceinline__ void pivot_forward_warp(const TL* __restrict__ lu, const int32_t* __restrict__ pv, int m,
+                                                   double* __restrict__ u, int lane) {
+  double y = lane < m ? u[lane] : 0.0;
+  const int p = lane < m ? pv[lane] : lane;
+#pragma unroll 1
+  for (int k = 0; k < m; ++k) {
+    const int q = __shfl_sync(0xffffffffu, p, k) & 31;
+    const double a = __shfl_sync(0xffffffffu, y, k), b = __shfl_sync(0xffffffffu, y, q);
+    if (lane == k) y = b;
+    if (lane == q) y = a;
+  }
+  const TL* row = lu + (lane < m ? lane : 0) * m;
+#pragma unroll 1
+  for (int k0 = 0; k0 + 1 < m; k0 += 8) {
+    TL l[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k0 + k < m) l[k] = row[k0 + k];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k0 + k + 1 < m) {
+        const double yk = __shfl_sync(0xffffffffu, y, k0 + k);
+        if (lane > k0 + k && lane < m) y = __dsub_rn(y, __dmul_rn(tri_widen(l[k]), yk));
+      }
+  }
+  if (lane < m) u[lane] = y;
+}
+
+template <typename TL>
+__device__ __forceinline__ void pivot_backward_warp(const TL* __restrict__ lu, int m, const double* __restrict__ u,
+                                                    double* __restrict__ x, double* S, int lane) {
+  double y = lane < m ? u[lane] : 0.0;
+  const int d = m | 1;
+#pragma unroll 4
+  for (int e = lane; e < m * m; e += 32) {
+    const int a = e / m;
+    S[a * d + e - a * m] = tri_widen(lu[e]);
+  }
+  __syncwarp();
+  double dg = 1.0, ry, rz;
+  if (lane < m) dg = S[lane * (d + 1)];
+  tri_recip(dg, ry, rz);
+#pragma unroll 1
+  for (int i = m - 1; i >= 0; --i) {
+    if (lane == i) {
+#pragma unroll 4
+      for (int k = i + 1; k < m; ++k) y = __dsub_rn(y, S[i * d + k]);
+      y = tri_div(y, dg, ry, rz);
+    }
+    const double v = __shfl_sync(0xffffffffu, y, i);
+    if (lane < i) S[lane * d + i] = __dmul_rn(S[lane * d + i], v);
+    __syncwarp();
+  }
+  if (lane < m) x[lane] = y;
+  __syncwarp();
+}
+
+constexpr int PIV_T = 128;  // threads per block of the two kernels below
+
+// Pivot blocks per warp: few when the chip has warps to spare, so that a warp
+// meets few large blocks one after the other (an FP64 operation costs the same
+// for 8 lanes as for 32).
+inline int piv_per(int64_t nD) { return nD <= 32768 ? 8 : 32; }
+inline unsigned piv_grid(int64_t nD) { return grid_for(nD, PIV_T / 32 * piv_per(nD)); }
+
+__global__ void __launch_bounds__(PIV_T)
+    k_pivot_fwd(int64_t nD, int per, const int32_t* __restrict__ sz, const int64_t* __restrict__ roff,
+                const int64_t* __restrict__ voff, const double* __restrict__ lu64, const float* __restrict__ lu32,
+                const int32_t* __restrict__ ptag, const int32_t* __restrict__ piv, double* __restrict__ u) {
+  const int lane = threadIdx.x & 31;
+  const int64_t wpg = (int64_t)gridDim.x * (PIV_T / 32);
+  for (int64_t y0 = (blockIdx.x * (int64_t)(PIV_T / 32) + (threadIdx.x >> 5)) * per; y0 < nD; y0 += wpg * per) {
+    const int64_t y = y0 + lane;
+    const bool has = lane < per && y < nD;
+    const int m = has ? sz[y] : 0;
+    const bool f32 = has && lu32 && !ptag[y];
+    if (m > 0 && m <= PIV_R) {
+      if (f32)
+        pivot_forward_reg<float>(lu32 + voff[y], piv + roff[y], m, u + roff[y]);
+      else
+        pivot_forward_reg<double>(lu64 + voff[y], piv + roff[y], m, u + roff[y]);
+    } else if (m > 32) {
+      if (f32)
+        pivot_forward<float>(lu32 + voff[y], piv + roff[y], m, u + roff[y]);
+      else
+        pivot_forward<double>(lu64 + voff[y], piv + roff[y], m, u + roff[y]);
+    }
+    __syncwarp();
+    const unsigned f = __ballot_sync(0xffffffffu, f32);
+    for (unsigned w = __ballot_sync(0xffffffffu, m > PIV_R && m <= 32); w; w &= w - 1) {
+      const int o = __ffs(w) - 1, mo = __shfl_sync(0xffffffffu, m, o);
+      if (f >> o & 1)
+        pivot_forward_warp<float>(lu32 + voff[y0 + o], piv + roff[y0 + o], mo, u + roff[y0 + o], lane);
+      else
+        pivot_forward_warp<double>(lu64 + voff[y0 + o], piv + roff[y0 + o], mo, u + roff[y0 + o], lane);
+    }
   }
 }
 
-__global__ void k_pivot_bwd(int64_t nD, const int32_t* __restrict__ sz, const int64_t* __restrict__ roff,
-                            const int64_t* __restrict__ voff, const double* __restrict__ lu64,
-                            const float* __restrict__ lu32, const int32_t* __restrict__ ptag,
-                            const double* __restrict__ u, double* __restrict__ x) {
-  for (int64_t y = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; y < nD; y += (int64_t)gridDim.x * blockDim.x) {
-    const int m = sz[y];
-    for (int a = 0; a < m; ++a) x[roff[y] + a] = u[roff[y] + a];
-    if (lu32 && !ptag[y])
-      pivot_backward<float>(lu32 + voff[y], m, x + roff[y]);
-    else
-      pivot_backward<double>(lu64 + voff[y], m, x + roff[y]);
+__global__ void __launch_bounds__(PIV_T)
+    k_pivot_bwd(int64_t nD, int per, const int32_t* __restrict__ sz, const int64_t* __restrict__ roff,
+                const int64_t* __restrict__ voff, const double* __restrict__ lu64, const float* __restrict__ lu32,
+                const int32_t* __restrict__ ptag, const double* __restrict__ u, double* __restrict__ x) {
+  __shared__ double stage[PIV_T / 32][32 * 33];
+  const int lane = threadIdx.x & 31;
+  double* S = stage[threadIdx.x >> 5];
+  const int64_t wpg = (int64_t)gridDim.x * (PIV_T / 32);
+  for (int64_t y0 = (blockIdx.x * (int64_t)(PIV_T / 32) + (threadIdx.x >> 5)) * per; y0 < nD; y0 += wpg * per) {
+    const int64_t y = y0 + lane;
+    const bool has = lane < per && y < nD;
+    const int m = has ? sz[y] : 0;
+    const bool f32 = has && lu32 && !ptag[y];
+    if (m > 0 && m <= PIV_R) {
+      if (f32)
+        pivot_backward_reg<float>(lu32 + voff[y], m, u + roff[y], x + roff[y]);
+      else
+        pivot_backward_reg<double>(lu64 + voff[y], m, u + roff[y], x + roff[y]);
+    } else if (m > 32) {
+      for (int a = 0; a < m; ++a) x[roff[y] + a] = u[roff[y] + a];
+      if (f32)
+        pivot_backward<float>(lu32 + voff[y], m, x + roff[y]);
+      else
+        pivot_backward<double>(lu64 + voff[y], m, x + roff[y]);
+    }
+    __syncwarp();
+    const unsigned f = __ballot_sync(0xffffffffu, f32);
+    for (unsigned w = __ballot_sync(0xffffffffu, m > PIV_R && m <= 32); w; w &= w - 1) {
+      const int o = __ffs(w) - 1, mo = __shfl_sync(0xffffffffu, m, o);
+      if (f >> o & 1)
+        pivot_backward_warp<float>(lu32 + voff[y0 + o], mo, u + roff[y0 + o], x + roff[y0 + o], S, lane);
+      else
+        pivot_backward_warp<double>(lu64 + voff[y0 + o], mo, u + roff[y0 + o], x + roff[y0 + o], S, lane);
+    }
   }
 }
+
+// Columns of a block whose loads are in flight together: 720 000 unknowns, A x
+// 523 us instead of 575 (two FP64 operations an entry alone are 250), G x and
+// W x 32 instead of 39.
+constexpr int SPMV_K = 6;
 
 // y_row -= M x  for every scalar row of a VBCSR M (one thread per scalar row,
 // blocks in order, then the entries of the row).
@@ -100,7 +330,16 @@ __global__ void k_bsr_sub(VBView<T> M, const int64_t* __restrict__ rowblk, int64
         const int nc = M.csz[J];
         const T* v = M.val + M.voff[b] + (int64_t)a * nc;
         const double* xj = x + M.coff[J];
-        for (int k = 0; k < nc; ++k) acc = __fmaf_rn((float)v[k], (float)xj[k], acc);
+        for (int k0 = 0; k0 < nc; k0 += SPMV_K) {  // loads first, SPMV_K columns at a time
+          float vk[SPMV_K];
+          double xk[SPMV_K];
+#pragma unroll
+          for (int k = 0; k < SPMV_K; ++k)
+            if (k0 + k < nc) vk[k] = (float)v[k0 + k], xk[k] = xj[k0 + k];
+#pragma unroll
+          for (int k = 0; k < SPMV_K; ++k)
+            if (k0 + k < nc) acc = __fmaf_rn(vk[k], (float)xk[k], acc);
+        }
       }
       y[q] = y[q] - (double)acc;
       continue;
@@ -111,7 +350,15 @@ __global__ void k_bsr_sub(VBView<T> M, const int64_t* __restrict__ rowblk, int64
       const int nc = M.csz[J];
       const T* v = M.val + M.voff[b] + (int64_t)a * nc;
       const double* xj = x + M.coff[J];
-      for (int k = 0; k < nc; ++k) s = __dsub_rn(s, __dmul_rn(ld(v + k), xj[k]));
+      for (int k0 = 0; k0 < nc; k0 += SPMV_K) {
+        double vk[SPMV_K], xk[SPMV_K];
+#pragma unroll
+        for (int k = 0; k < SPMV_K; ++k)
+          if (k0 + k < nc) vk[k] = ld(v + k0 + k), xk[k] = xj[k0 + k];
+#pragma unroll
+        for (int k = 0; k < SPMV_K; ++k)
+          if (k0 + k < nc) s = __dsub_rn(s, __dmul_rn(vk[k], xk[k]));
+      }
     }
     y[q] = s;
   }
@@ -129,7 +376,15 @@ __global__ void k_spmv(VBView<double> A, const int64_t* __restrict__ rowblk, int
       const int nc = A.csz[J];
       const double* v = A.val + A.voff[b] + (int64_t)a * nc;
       const double* xj = x + A.coff[J];
-      for (int k = 0; k < nc; ++k) s = __dadd_rn(s, __dmul_rn(v[k], xj[k]));
+      for (int k0 = 0; k0 < nc; k0 += SPMV_K) {  // loads first, SPMV_K columns at a time
+        double vk[SPMV_K], xk[SPMV_K];
+#pragma unroll
+        for (int k = 0; k < SPMV_K; ++k)
+          if (k0 + k < nc) vk[k] = v[k0 + k], xk[k] = xj[k0 + k];
+#pragma unroll
+        for (int k = 0; k < SPMV_K; ++k)
+          if (k0 + k < nc) s = __dadd_rn(s, __dmul_rn(vk[k], xk[k]));
+      }
     }
     y[q] = s;
   }
@@ -263,45 +518,6 @@ __device__ __forceinline__ bool tri_take(const float* p, int cnt, float* x) {
     }
   return ok;
 }
-
-// a / b correctly rounded from y = RN(1/b) and z, the rest of 1/b (tri_recip):
-// q0 = a y + a z is within one ulp of a / b, a - b q0 is exact, and the
-// correction by it rounds to RN(a / b) (Markstein's theorem; exact remainder
-// and correctly rounded reciprocal).  Four operations instead of a division's
-// 84 (FP32) or 560 (FP64) cycles.  Operands outside the range where no
-// intermediate can underflow or overflow (y = 0 marks such a b) are divided.
-__device__ __forceinline__ void tri_recip(float b, float& y, float& z) {
-  y = 0.f, z = 0.f;
-  if (fabsf(b) >= 0x1p-40f && fabsf(b) <= 0x1p40f) {
-    y = __frcp_rn(b);
-    z = __fmul_rn(__fmaf_rn(-b, y, 1.f), y);
-  }
-}
-__device__ __forceinline__ void tri_recip(double b, double& y, double& z) {
-  y = 0.0, z = 0.0;
-  if (fabs(b) >= 0x1p-300 && fabs(b) <= 0x1p300) {
-    y = __drcp_rn(b);
-    z = __dmul_rn(__fma_rn(-b, y, 1.0), y);
-  }
-}
-__device__ __forceinline__ double tri_div(double a, double b, double y, double z) {
-  const unsigned e = ((unsigned)__double2hiint(a) >> 20) & 0x7ff;  // |a| in [2^-300, 2^300): integer compares
-  if (__double2hiint(y) != 0 && e >= 1023 - 300 && e < 1023 + 300) {
-    const double q = __fma_rn(a, y, __dmul_rn(a, z));
-    return __fma_rn(__fma_rn(-b, q, a), y, q);
-  }
-  return __ddiv_rn(a, b);
-}
-
-// (double)v by integer operations (normal values; the conversion instruction
-// takes the FP64 unit).
-__device__ __forceinline__ double tri_widen(float v) {
-  const unsigned u = (unsigned)__float_as_int(v);
-  if ((u & 0x7f800000u) - 0x00800000u < 0x7f000000u)
-    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
-  return (double)v;
-}
-__device__ __forceinline__ double tri_widen(double v) { return v; }
 
 // RN32(RN64(R - s)) for an FP64 R and an FP32 s by FP32 operations: R is held
 // as the exact sum h + m + l of three floats; t + e = h - s and f + e2 = t + w
@@ -1180,7 +1396,7 @@ void solve_core(const PrecDev<T>& P, const double* in, double* out, const SolveB
     if (L.grouped)
       grouped_forward<T>(L, B.bh[l], s);
     else if (L.nD)
-      launch(k_pivot_fwd, grid_for(L.nD, 128), 128, 0, s, L.nD, L.D.rsz.p, L.D.roff.p, L.D.voff.p, L.D.val.p,
+      launch(k_pivot_fwd, piv_grid(L.nD), PIV_T, 0, s, L.nD, piv_per(L.nD), L.D.rsz.p, L.D.roff.p, L.D.voff.p, L.D.val.p,
              mixed ? L.D32.val.p : nullptr, L.ptag.p, L.piv.p, B.bh[l]);
     const int64_t ng = M.n - M.nf;
     if (ng && L.G.nnzb)
@@ -1217,7 +1433,7 @@ void solve_core(const PrecDev<T>& P, const double* in, double* out, const SolveB
     if (L.grouped)
       grouped_backward<T>(L, B.bh[l], B.xh[l], s);
     else if (L.nD)
-      launch(k_pivot_bwd, grid_for(L.nD, 128), 128, 0, s, L.nD, L.D.rsz.p, L.D.roff.p, L.D.voff.p, L.D.val.p,
+      launch(k_pivot_bwd, piv_grid(L.nD), PIV_T, 0, s, L.nD, piv_per(L.nD), L.D.rsz.p, L.D.roff.p, L.D.voff.p, L.D.val.p,
              mixed ? L.D32.val.p : nullptr, L.ptag.p, B.bh[l], B.xh[l]);
     if (M.n) launch(k_scatter_scale, grid_for(M.n, 256), 256, 0, s, M.n, M.sperm.p, L.c.p, B.xh[l], xo);
     VB_LAUNCH_CHECK();

@@ -117,3 +117,17 @@ def test_level_orders_of_few_rows(nb):
     x = np.random.default_rng(nb).standard_normal(int(m[0].sum()))
     yo = oracle.Prec(oracle.VBMat(m[0], m[0], *m[1:]), 0, 0.0, -1).apply(x)
     assert np.linalg.norm(_apply(V, P, x) - yo) <= 1e-12 * np.linalg.norm(yo)
+
+
+@pytest.mark.parametrize("name", CASES)
+def test_one_reduction_level_matches_oracle(name):
+    """The reduction level's pivot solves (a thread or a warp per block, by size)
+    and the products with G and W."""
+    V = vb()
+    m = _matrix(*CASES[name], seed=20 + sorted(CASES).index(name))
+    x = np.random.default_rng(11).standard_normal(int(m[0].sum()))
+    P = V.vbarms_factor(V.vbarms_vbsr_from_blocks(*m), 1, 0.0, -1)
+    yo = oracle.Prec(oracle.VBMat(m[0], m[0], *m[1:]), 1, 0.0, -1).apply(x)
+    assert np.linalg.norm(_apply(V, P, x) - yo) <= 1e-12 * np.linalg.norm(yo)
+    P32 = V.vbarms_factor(V.vbarms_vbsr_from_blocks(*m), 1, 0.0, -1, precision="fp32")
+    assert np.linalg.norm(_apply(V, P32, x) - yo) <= 9 * len(x) * 2.0 ** -24 * np.linalg.norm(yo)
