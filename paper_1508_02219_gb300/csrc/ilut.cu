@@ -39,7 +39,7 @@
 // entries are corrected products with their reciprocals, the pivot search and
 // the reciprocals overlap, and FP64 drop tests are decided in FP32 where that
 // is certain.  The kernel's time before and now: 3.0 million unknowns FP32 710
-// and 392 ms, 360 000 FP64 498 and 266 ms, 48 000 at tau 0.9 786 and 267 ms.
+// and 376 ms, 360 000 FP64 498 and 261 ms, 48 000 at tau 0.9 786 and 253 ms.
 //
 // A wait that runs out sets VB_ETIMEOUT and raises an abort flag; a row that
 // failed publishes kRowFailed so that its dependants stop too.  Overflowing a
@@ -327,6 +327,15 @@ __device__ __noinline__ double fro2_batched(const T* __restrict__ v, int n) {
 template <typename T>
 __device__ __forceinline__ float fro2_f32(const T* __restrict__ v, int n) {
   float s = 0.f;
+  if (n <= 4) {
+    float x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = u < n ? (float)v[u] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (u < n) s = __fmaf_rn(x[u], x[u], s);
+    return s;
+  }
 #pragma unroll 1
   for (int e0 = 0; e0 < n; e0 += 16) {  // sixteen loads in flight, summed in element order
     float x[16];
@@ -365,6 +374,12 @@ __device__ __noinline__ void ainv_right_row_sh(const TS* lu, int S, const int* p
 __device__ __forceinline__ long long abs_key(double x) { return __double_as_longlong(x) & 0x7fffffffffffffffLL; }
 __device__ __forceinline__ long long abs_key(float x) { return (long long)(__float_as_int(x) & 0x7fffffff); }
 
+// The largest of the lanes' non-negative values, NaN counting as 0 (as a chain
+// of fmaxf from 0 has it).
+__device__ __forceinline__ float warp_max_f(float v) {
+  return __int_as_float((int)__reduce_max_sync(0xffffffffu, v == v ? (unsigned)__float_as_int(v) : 0u));
+}
+
 template <typename TL>
 __device__ __forceinline__ TL div_rn(TL a, TL b);
 template <>
@@ -386,25 +401,23 @@ template <typename TL>
 __device__ __noinline__ bool gepp_warp(TL* a, int n, int* pvs, int32_t* gpiv, int lane) {
 #pragma unroll 1
   for (int kk = 0; kk < n; ++kk) {
-    long long key = -1;
+    // the largest |a_ik|, its upper word first, the lowest row on ties
+    unsigned long long key = 0;  // |a| + 1, 0: no row
     int idx = 0x7fffffff;
 #pragma unroll 1
     for (int ii = kk + lane; ii < n; ii += 32) {
-      const long long v = abs_key(a[ii * n + kk]);
+      const unsigned long long v = (unsigned long long)abs_key(a[ii * n + kk]) + 1ull;
       if (v > key) {
         key = v;
         idx = ii;
       }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      const long long ok = __shfl_xor_sync(0xffffffffu, key, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-      if (ok > key || (ok == key && oi < idx)) {
-        key = ok;
-        idx = oi;
-      }
-    }
-    if (key <= 0) return false;
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(key >> 32));
+    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(key >> 32) == hi ? (unsigned)key : 0u);
+    const unsigned long long most = ((unsigned long long)hi << 32) | lo;
+    idx = __reduce_min_sync(0xffffffffu, key == most ? idx : 0x7fffffff);
+    key = most - 1;
+    if (key == 0) return false;
     const int pr = idx;
     if (lane == 0) {
       gpiv[kk] = pr;
@@ -420,6 +433,7 @@ __device__ __noinline__ bool gepp_warp(TL* a, int n, int* pvs, int32_t* gpiv, in
     __syncwarp();
     const TL d = a[kk * n + kk];
     const int w = n - kk - 1;
+    const float rw = __fdividef(1.f, (float)max(w, 1));
 #pragma unroll 1
     for (int r = lane; r < w; r += 32) {
       TL* l = a + (kk + 1 + r) * n + kk;
@@ -428,7 +442,9 @@ __device__ __noinline__ bool gepp_warp(TL* a, int n, int* pvs, int32_t* gpiv, in
     __syncwarp();
 #pragma unroll 1
     for (int e = lane; e < w * w; e += 32) {
-      const int r = e / w, c = e - r * w;
+      int r = (int)((float)e * rw), c = e - r * w;  // e / w, corrected
+      if (c < 0) --r, c += w;
+      if (c >= w) ++r, c -= w;
       const int ii = kk + 1 + r, jj = kk + 1 + c;
       a[ii * n + jj] = msub<TL>(a[ii * n + jj], a[ii * n + kk], a[kk * n + jj]);
     }
@@ -513,28 +529,41 @@ __device__ __forceinline__ bool div_range(double a, double y) {
 }
 
 // ---- FP32 pivot blocks held in registers -----------------------------------
-// The block's entries are read up front by broadcast 16-byte loads (rows N
-// floats apart), so that only the chain of operations itself is left; a size n
-// below N costs a uniform branch per row.  Each routine gives every element the
+// The block's entries are read up front by broadcast 16-byte loads (rows 8
+// floats apart for N <= 8, else N), so that only the chain of operations itself
+// is left; a size n below N costs a uniform branch per row.  Small blocks are
+// taken by the class 2, 4, 6 or 8 that holds them, since a class for 8 alone
+// spends a row's and a column's instructions on every size below (that and the
+// cheaper reductions and copies of a finish: 392 to 376 ms at 3.0 million unknowns,
+// 267 to 253 at tau 0.9).  Each routine gives every element the
 // operations of its generic counterpart (ainv_right_row_sh, gepp_warp,
 // inv_norm1_f32) in the same order, so the results are identical bit for bit.
 // A 6 x 6 block, one warp alone: multiplier 1 900 cycles with the entries read
 // where they are used, factorization with condition estimate 6 200.
 
 template <int N>
+__device__ __forceinline__ constexpr int lu_rows() {  // distance of the rows
+  return N <= 8 ? 8 : N;
+}
+template <int N>
 __device__ __forceinline__ void load_lu(const float* lu, float* L) {
 #pragma unroll
-  for (int e = 0; e < N * N; e += 4) {
-    const float4 v = *reinterpret_cast<const float4*>(lu + e);
-    L[e] = v.x, L[e + 1] = v.y, L[e + 2] = v.z, L[e + 3] = v.w;
-  }
+  for (int a = 0; a < N; ++a)
+#pragma unroll
+    for (int c = 0; c < N; c += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(lu + a * lu_rows<N>() + c);
+      L[a * N + c] = v.x;
+      if (c + 1 < N) L[a * N + c + 1] = v.y;
+      if (c + 2 < N) L[a * N + c + 2] = v.z;
+      if (c + 3 < N) L[a * N + c + 3] = v.w;
+    }
 }
 
-// r <- r (P^T L U)^{-1} for one row x[0, n), n <= 8; the result goes, permuted,
-// to the row m and (unless NULL) to mt with stride np.
-__device__ __forceinline__ void mult_row_small(const float* lu, const float* ry, const float* rz, const int* perm,
-                                               int n, const float* x, float* m, float* mt, int np) {
-  constexpr int N = NSMALL;
+// r <- r (P^T L U)^{-1} for one row x[0, n), n <= N <= 8; the result goes,
+// permuted, to the row m and (unless NULL) to mt with stride np.
+template <int N>
+__device__ __forceinline__ void mult_row_n(const float* lu, const float* ry, const float* rz, const int* perm, int n,
+                                           const float* x, float* m, float* mt, int np) {
   float L[N * N], r[N], y[N], z[N];
   int c[N];
 #pragma unroll
@@ -580,6 +609,18 @@ __device__ __forceinline__ void mult_row_small(const float* lu, const float* ry,
     }
 }
 
+__device__ __forceinline__ void mult_row_small(const float* lu, const float* ry, const float* rz, const int* perm,
+                                               int n, const float* x, float* m, float* mt, int np) {
+  if (n <= 2)
+    mult_row_n<2>(lu, ry, rz, perm, n, x, m, mt, np);
+  else if (n <= 4)
+    mult_row_n<4>(lu, ry, rz, perm, n, x, m, mt, np);
+  else if (n <= 6)
+    mult_row_n<6>(lu, ry, rz, perm, n, x, m, mt, np);
+  else
+    mult_row_n<8>(lu, ry, rz, perm, n, x, m, mt, np);
+}
+
 // GEPP of the n x n row-major FP32 block at src (n <= N), row i in lane i's
 // registers: the pivot is the largest |a_ik| (the lowest position on ties)
 // found by a warp max-reduction of the keys and a ballot, while every lane
@@ -592,6 +633,7 @@ __device__ __forceinline__ void mult_row_small(const float* lu, const float* ry,
 template <int N>
 __device__ __noinline__ bool gepp_cond(const float* src, int n, float* lu, float* ry, float* rz, int* pvs, int* perm,
                                        int32_t* gpiv, int lane, float* inv1) {
+  constexpr int S = lu_rows<N>();
   float r[N];
 #pragma unroll
   for (int j = 0; j < N; ++j) r[j] = lane < n && j < n ? src[lane * n + j] : 0.f;
@@ -640,7 +682,7 @@ __device__ __noinline__ bool gepp_cond(const float* src, int n, float* lu, float
     ry[pos] = yd;
     rz[pos] = zd;
 #pragma unroll
-    for (int j = 0; j < N; ++j) lu[pos * N + j] = r[j];
+    for (int j = 0; j < N; ++j) lu[pos * S + j] = r[j];
   }
   __syncwarp();
   // x = P e_c: one at the place that row c was brought to (lanes without a
@@ -676,7 +718,7 @@ __device__ __noinline__ bool gepp_cond(const float* src, int n, float* lu, float
       if (i < n) {
 #pragma unroll
         for (int k4 = 0; k4 < i; k4 += 4) {
-          const float4 v = *reinterpret_cast<const float4*>(lu + i * N + k4);
+          const float4 v = *reinterpret_cast<const float4*>(lu + i * S + k4);
           const float l[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
           for (int k = k4; k < i && k < k4 + 4; ++k) x[i] = __fmaf_rn(-l[k - k4], x[k], x[i]);
@@ -687,23 +729,31 @@ __device__ __noinline__ bool gepp_cond(const float* src, int n, float* lu, float
       if (i < n) {
 #pragma unroll
         for (int k4 = (i + 1) & ~3; k4 < N; k4 += 4) {
-          const float4 v = *reinterpret_cast<const float4*>(lu + i * N + k4);
+          const float4 v = *reinterpret_cast<const float4*>(lu + i * S + k4);
           const float l[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
           for (int k = k4; k < N && k < k4 + 4; ++k)
             if (k > i && k < n) x[i] = __fmaf_rn(-l[k - k4], x[k], x[i]);
         }
-        x[i] = div_range(x[i], ry[i]) ? div_recip(x[i], lu[i * (N + 1)], ry[i], rz[i])
-                                      : __fdiv_rn(x[i], lu[i * (N + 1)]);
+        x[i] = div_range(x[i], ry[i]) ? div_recip(x[i], lu[i * (S + 1)], ry[i], rz[i])
+                                      : __fdiv_rn(x[i], lu[i * (S + 1)]);
       }
   }
 #pragma unroll
   for (int i = 0; i < N; ++i)
     if (i < n) cs += fabsf(x[i]);
   if (lane >= n) cs = 0.f;
-  for (int o = 16; o > 0; o >>= 1) cs = fmaxf(cs, __shfl_xor_sync(0xffffffffu, cs, o));
-  *inv1 = cs;
+  // (NaN in every lane, which takes 32 columns, stays NaN)
+  *inv1 = N == 32 && __all_sync(0xffffffffu, cs != cs) ? cs : warp_max_f(cs);
   return true;
+}
+
+__device__ __forceinline__ bool gepp_cond_small(const float* src, int n, float* lu, float* ry, float* rz, int* pvs,
+                                                int* perm, int32_t* gpiv, int lane, float* inv1) {
+  return n <= 2   ? gepp_cond<2>(src, n, lu, ry, rz, pvs, perm, gpiv, lane, inv1)
+         : n <= 4 ? gepp_cond<4>(src, n, lu, ry, rz, pvs, perm, gpiv, lane, inv1)
+         : n <= 6 ? gepp_cond<6>(src, n, lu, ry, rz, pvs, perm, gpiv, lane, inv1)
+                  : gepp_cond<8>(src, n, lu, ry, rz, pvs, perm, gpiv, lane, inv1);
 }
 
 // The same for any n and either type, in loops, the row held in shared memory
@@ -871,18 +921,25 @@ __device__ __noinline__ int lfil_cut(int* cand, int n, int lfil, const long long
   }
   if (keybytes == 4 && n <= 256) {
     // keys of 31 bits, up to 8 a lane in registers: the lfil-th largest is
-    // built bit by bit, each bit kept if lfil keys reach the value with it
+    // built from the top, bits kept if lfil keys reach the value with them
     unsigned kq[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) kq[u] = lane + 32 * u < n ? (unsigned)sf2[cand[lane + 32 * u]] + 1u : 0u;
     unsigned thr = 0;
 #pragma unroll 1
-    for (int bit = 31; bit >= 0; --bit) {
-      const unsigned t = thr | (1u << bit);
-      int c = 0;
+    for (int bit = 30; bit >= 0; bit -= 2) {  // two bits at a time, three counts of at most 256 in one sum
+      const unsigned t1 = thr | (1u << bit), t2 = thr | (2u << bit), t3 = thr | (3u << bit);
+      unsigned c = 0;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) c += kq[u] >= t;
-      if (__reduce_add_sync(0xffffffffu, c) >= lfil) thr = t;
+      for (int u = 0; u < 8; ++u)
+        c += (kq[u] >= t1 ? 1u : 0u) + (kq[u] >= t2 ? 1u << 10 : 0u) + (kq[u] >= t3 ? 1u << 20 : 0u);
+      c = __reduce_add_sync(0xffffffffu, c);
+      if ((int)(c >> 20) >= lfil)
+        thr = t3;
+      else if ((int)(c >> 10 & 1023) >= lfil)
+        thr = t2;
+      else if ((int)(c & 1023) >= lfil)
+        thr = t1;
     }
     int above = 0, equal = 0;
 #pragma unroll
@@ -1052,6 +1109,16 @@ __device__ __noinline__ void sort_by_column(const int* cand, int k, const int* s
 template <typename T>
 __device__ __noinline__ void copy_blocks(int n, int sz, int so, long long dof, const T* __restrict__ src,
                                             T* __restrict__ dst, int lane) {
+  if (__reduce_max_sync(0xffffffffu, lane < n ? sz : 0) <= 4) {  // a lane a block
+    T v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (lane < n && u < sz) v[u] = src[so + u];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (lane < n && u < sz) dst[dof + u] = v[u];
+    return;
+  }
   const int g = lane >> 3, a = lane & 7;
 #pragma unroll 1
   for (int p0 = 0; p0 < n; p0 += 4) {
@@ -1875,10 +1942,10 @@ __global__ void __launch_bounds__(256, 1)
           for (int ii = 0; ii < ni; ++ii) sum += fabsf(srcd[ii * ni + jj]);
           norm1 = fmaxf(norm1, sum);
         }
-        for (int o = 16; o > 0; o >>= 1) norm1 = fmaxf(norm1, __shfl_xor_sync(0xffffffffu, norm1, o));
+        norm1 = warp_max_f(norm1);
         float inv1 = 0.f;
         if (ni <= NSMALL) {
-          if (gepp_cond<NSMALL>(srcd, ni, M.lu, M.ry, M.rz, M.pv, M.perm, gpiv, lane, &inv1)) {
+          if (gepp_cond_small(srcd, ni, M.lu, M.ry, M.rz, M.pv, M.perm, gpiv, lane, &inv1)) {
             tag64 = !(norm1 * inv1 <= condf);
             lu_sm = !tag64;
           }
@@ -2334,8 +2401,8 @@ void ilut_last(LastDev<T>& X, double t, int lfil, bool mixed, double cond_thr, u
   // kept per device, precision and class of row sizes for the rest of the
   // process; small matrices take the first.  What counts is that records and
   // working rows stay on chip; the rows in flight then matter little (3.0
-  // million unknowns FP32, the whole factorization, slots / value bytes / stage
-  // bytes: 64 / 6 144 / 3 072, 8 warps an SM, 709 ms; 128 / 8 192 / 4 096, 8
+  // million unknowns FP32, the whole factorization when the chosen shape read 644
+  // ms, which is 474 now; slots / value bytes / stage bytes: 64 / 6 144 / 3 072, 8 warps an SM, 709 ms; 128 / 8 192 / 4 096, 8
   // warps, 671; 128 / 12 288 / 4 096, 7 warps, 644; 128 / 16 384 / 6 144, 5
   // warps, 677).  FP64 rows hold twice the bytes (360 000 unknowns: 128 / 8 192
   // / 6 144, 7 warps, 382 ms; 128 / 16 384 / 6 144, 5 warps, 339); rows of many

@@ -39,6 +39,17 @@ def test_mixed_factors_close(name):
     assert np.array_equal(P.vector(0, "piv"), Po.vec(0, "piv"))
 
 
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 6, 7, 8, 9])
+def test_mixed_factors_of_one_block_size(n):
+    m = _matrix(n, n, 30, 6, seed=90 + n)
+    V, P, Po = _factors(m, 0.0, -1, "fp32")
+    # the bound of the test above
+    for w in ("L", "U", "D"):
+        g, o = P.export(0, w), Po.mat(0, w)
+        assert np.linalg.norm(g["val"] - o.val) <= 3 * 30 * n * 2.0 ** -24 * np.linalg.norm(o.val), w
+    assert np.array_equal(P.vector(0, "piv"), Po.vec(0, "piv"))
+
+
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("nb,band,lfil", [(420, 190, 12), (700, 340, 9)])
 def test_lfil_cuts_of_many_candidates(nb, band, lfil, precision):
