@@ -117,3 +117,17 @@ def test_invalid_group_size():
         with pytest.raises(V.VbarmsError) as e:
             V.vbarms_factor(A, 2, 1e-3, -1, group_size=gs)
         assert e.value.status == V.VB_EINVAL
+
+
+@pytest.mark.parametrize("nb,band,gs", [(31, 5, 4), (33, 9, 3), (160, 75, 64), (700, 40, 64), (1025, 6, 7)])
+def test_groups_of_long_adjacency_lists(nb, band, gs):
+    """Lists longer than a warp takes at once, groups of more members than its
+    lanes, orders that end inside a warp's 32 candidates."""
+    from test_gpu_sweeps import _matrix
+
+    m = _matrix(1, 2, nb, band, seed=nb)
+    P = vb().vbarms_factor(vb().vbarms_vbsr_from_blocks(*m), 1, 1e-3, 6, group_size=gs)
+    Po = oracle.Prec(oracle.VBMat(m[0], m[0], *m[1:]), 1, 1e-3, 6, gs=gs)
+    assert Po.levels == 1 and np.diff(Po.gptr(0)).max() > 1
+    assert np.array_equal(P.vector(0, "gptr"), Po.gptr(0))
+    compare_factor(P, Po)
