@@ -363,7 +363,7 @@ vb_status vbarms_prec_kernel_stats(vbarms_prec M, int kernel, int* launches, dou
 /* The per-warp workspace the last-level ILUT of M ran with ("tile shape"
  * of its kernel): slots (blocks of a working row held in shared memory),
  * value_bytes (their values), warps_per_sm; source = 0 default (last level
- * under 16384 block rows), 1 chosen by timing the candidate shapes on a
+ * under 65536 block rows), 1 chosen by timing the candidate shapes on a
  * prefix of this factorization's own rows (tune_s seconds of timing), 2
  * taken from an earlier timing of a matrix of the same device, precision and
  * class of row sizes in this process.  A prefix of the ILUT's row order is

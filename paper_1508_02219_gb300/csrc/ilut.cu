@@ -2423,7 +2423,7 @@ void ilut_last(LastDev<T>& X, double t, int lfil, bool mixed, double cond_thr, u
   if (!wide) cands.push_back(make_geom<T>(128, 8192, f64 ? 6144 : 4096, 128));
   const int reserve = 1024;  // shared memory the system keeps per block
   // warps per block and blocks per SM of a geometry: the most warps per SM
-  // (at most 16)
+  // (at most 8: their registers)
   auto shape = [&](const IlutGeom& G, int& wpb, int& bps) {
     wpb = 0, bps = 0;
     for (int w = 8; w >= 1; --w) {
