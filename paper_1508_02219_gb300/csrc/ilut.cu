@@ -1427,7 +1427,9 @@ __global__ void __launch_bounds__(256, 1)
     }
     __syncwarp();
     // stage buffer bookkeeping, the same in every lane: the column whose
-    // record a buffer holds or is being copied into (-1: free)
+    // record a buffer holds or is being copied into (-1: free, and no copy into
+    // it in flight: a step frees only the buffers of its own record, so that
+    // one fetched ahead stays known across a step that reads its record in place)
     int btag0 = -1, btag1 = -1;
     int64_t last = -1;
     // ---- eliminate the L part in ascending column order (including fill)
@@ -1653,8 +1655,8 @@ __global__ void __launch_bounds__(256, 1)
       if (dropped) {
         if (lane == 0) sstate[sk] = SL_DEAD;
         __syncwarp();
-        if (bi != 1) btag0 = -1;
-        if (bi != 0) btag1 = -1;
+        if (btag0 == (int)k) btag0 = -1;
+        if (btag1 == (int)k) btag1 = -1;
         continue;
       }
       if (lane == 0) {
@@ -1793,8 +1795,8 @@ __global__ void __launch_bounds__(256, 1)
         }
         __syncwarp();
       }
-      if (bi != 1) btag0 = -1;
-      if (bi != 0) btag1 = -1;
+      if (btag0 == (int)k) btag0 = -1;
+      if (btag1 == (int)k) btag1 = -1;
     }
     record_wait<0>();  // every record fetched ahead has been used, unless the row failed
     // A row that ends in the global workspace has its slot metadata copied
