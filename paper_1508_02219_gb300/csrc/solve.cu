@@ -1099,6 +1099,7 @@ __global__ void __launch_bounds__(TRI_W * 32, TRI_B)
       if (lane < ni) publish(i, r0, lane, u, sc);
     } else {  // pivot blocks of more than TRI_MP rows: one lane
       double* sv = reinterpret_cast<double*>(sm.part);
+      __syncwarp();  // a large row's values may reach into part: every lane has read them
 #pragma unroll
       for (int t = 0; t < TRI_R; ++t)
         if (lane + 32 * t < ni) sv[lane + 32 * t] = ni <= TRI_MR ? u : s[t];

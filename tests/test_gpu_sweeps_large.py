@@ -1,0 +1,44 @@
+"""The last level's triangular sweeps on block rows of more than 16 scalars whose
+1 025 to 1 536 values take the whole on-chip space of a warp: pivot blocks of more
+than 32 rows, and FP64 pivot blocks of 17 to 32 rows in a mixed factor."""
+import numpy as np
+import pytest
+
+import oracle
+from gpu_helpers import cuda_ok, vb
+from test_gpu_sweeps import _apply, _matrix
+
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not cuda_ok(), reason="needs a CUDA GPU")]
+
+
+def _check(lo, hi, nb, band, seed, precision, **opt):
+    m = _matrix(lo, hi, nb, band, seed=seed)
+    V = vb()
+    P = V.vbarms_factor(V.vbarms_vbsr_from_blocks(*m), 0, 0.0, -1, precision=precision, **opt)
+    for w in ("L", "U"):
+        o = P.export(0, w)
+        nv = np.diff(o["voff"][o["bptr"]])
+        assert ((nv > 1024) & (nv <= 1536)).sum() >= nb // 2, w
+    n = int(m[0].sum())
+    x = np.random.default_rng(seed).standard_normal(n)
+    yo = oracle.Prec(oracle.VBMat(m[0], m[0], *m[1:]), 0, 0.0, -1).apply(x)
+    y = _apply(V, P, x)
+    # FP64: the solve's parity bound.  FP32 factor and solve: 3 n u |L||U| each
+    # way, |A^-1||L||U| <= 3 on these dominant matrices, u = 2^-24
+    tol = 1e-12 if precision == "fp64" else 9 * n * 2.0 ** -24
+    assert np.linalg.norm(y - yo) <= tol * np.linalg.norm(yo)
+    return P
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("lo,hi", [(33, 33), (33, 38), (38, 39)])
+def test_pivot_blocks_of_more_than_32_rows(lo, hi, precision):
+    for seed in range(4):
+        _check(lo, hi, 24, 1, seed, precision)
+
+
+@pytest.mark.parametrize("lo,hi,band", [(17, 18, 4), (20, 21, 3), (24, 27, 2)])
+def test_fp64_pivot_blocks_of_17_to_32_rows_in_a_mixed_factor(lo, hi, band):
+    for seed in range(4):
+        P = _check(lo, hi, 40, band, seed, "fp32", fp64_pivot_cond=1.0)
+        assert P.vector(0, "ptag").all()
