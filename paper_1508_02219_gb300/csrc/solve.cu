@@ -458,13 +458,15 @@ constexpr int TRI_B = 2;
 // Shared memory of one warp.
 template <typename T>
 struct alignas(16) TriSmem {
-  T stage[TRI_STAGE];           // the row's block values (a row of more than TRI_MR
-  T part[32 * TRI_MR];          //   scalars: up to the end of part); part: per block
-                                //   of the row (modulo 32), its product
+  // the row's block values: TRI_STAGE of them, all of val when the row has more
+  // than TRI_MR scalars; behind TRI_STAGE, per block of the row (modulo 32), its
+  // product, or a large pivot block's unknowns
+  T val[TRI_STAGE + 32 * TRI_MR];
   // the factored pivot block and the reciprocals of its diagonal (tri_recip):
   // up to TRI_MP rows of T, or up to TRI_MP / 2 rows of a tagged FP64 block
   T lu[TRI_MP * (TRI_MP + 1)];
   T ry[TRI_MP], rz[TRI_MP];
+  __device__ __forceinline__ T* part() { return val + TRI_STAGE; }
 };
 
 // The wait of one warp between two polls: a short sleep, the abort word and
@@ -1021,12 +1023,12 @@ __global__ void __launch_bounds__(TRI_W * 32, TRI_B)
     }
     const int64_t v0 = M.voff[b0];
     const int64_t nv = M.voff[b1] - v0;
-    const bool staged = nv <= TRI_STAGE + (ni > TRI_MR ? 32 * TRI_MR : 0);
+    const bool staged = nv <= (ni > TRI_MR ? TRI_STAGE + 32 * TRI_MR : TRI_STAGE);
     if (staged) {
 #pragma unroll 4
-      for (int64_t e = lane; e < nv; e += 32) sm.stage[e] = M.val[v0 + e];
+      for (int64_t e = lane; e < nv; e += 32) sm.val[e] = M.val[v0 + e];
     }
-    const T* sval = staged ? sm.stage : M.val + v0;
+    const T* sval = staged ? sm.val : M.val + v0;
     const TriRow<T> row{M.bcol + b0, M.voff + b0, M.csz, M.coff, v0, nb, ni};
     double u = 0.0, sc = 0.0;  // lane a: row a's unknown, its scale
     if (lane < ni) {
@@ -1044,8 +1046,8 @@ __global__ void __launch_bounds__(TRI_W * 32, TRI_B)
       // ones in FP64; the row's result is formed in FP64
       T sa;
       const bool ok = ni <= 8 && staged
-                          ? tri_row<8>(row, sm.stage, rec, sm.part, abort, wait_limit, st, lane, &sa)
-                          : tri_row16<T, R>(row, sval, rec, sm.part, abort, wait_limit, st, lane, &sa);
+                          ? tri_row<8>(row, sm.val, rec, sm.part(), abort, wait_limit, st, lane, &sa)
+                          : tri_row16<T, R>(row, sval, rec, sm.part(), abort, wait_limit, st, lane, &sa);
       if (!ok) return;
       if constexpr (narrow) uf = tri_sub32(u, us, sa, lane < ni);
       if (!narrow || (BWD && !f32p)) u = lane < ni ? u - (double)sa : 0.0;
@@ -1098,8 +1100,8 @@ __global__ void __launch_bounds__(TRI_W * 32, TRI_B)
       }
       if (lane < ni) publish(i, r0, lane, u, sc);
     } else {  // pivot blocks of more than TRI_MP rows: one lane
-      double* sv = reinterpret_cast<double*>(sm.part);
-      __syncwarp();  // a large row's values may reach into part: every lane has read them
+      double* sv = reinterpret_cast<double*>(sm.part());
+      __syncwarp();  // a large row's values may reach behind TRI_STAGE: every lane has read them
 #pragma unroll
       for (int t = 0; t < TRI_R; ++t)
         if (lane + 32 * t < ni) sv[lane + 32 * t] = ni <= TRI_MR ? u : s[t];

@@ -42,3 +42,10 @@ def test_fp64_pivot_blocks_of_17_to_32_rows_in_a_mixed_factor(lo, hi, band):
     for seed in range(4):
         P = _check(lo, hi, 40, band, seed, "fp32", fp64_pivot_cond=1.0)
         assert P.vector(0, "ptag").all()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("lo,hi,band", [(17, 18, 4), (20, 21, 3), (24, 27, 2)])
+def test_rows_of_17_to_32_scalars(lo, hi, band, precision):
+    """The pivot block's own space lies right behind the values."""
+    _check(lo, hi, 40, band, 7, precision)
