@@ -1491,6 +1491,7 @@ __global__ void __launch_bounds__(256, 1)
         unsigned long long word = 0;
         if (lane == 0) word = wait_word(P.done + k, P.abort, wait_limit, st);
         word = __shfl_sync(0xffffffffu, word, 0);
+        __syncwarp();  // every lane's reads of the record come after lane 0's acquire (a shuffle orders no memory)
         if (word == 0 || word == kRowFailed) {
           status_local = DEV_ETIMEOUT;
           break;
@@ -1507,6 +1508,7 @@ __global__ void __launch_bounds__(256, 1)
           if (want_pf && (bi ? btag0 : btag1) < 0) {
             if (lane == 0) w2 = ld_acquire_u64(P.done + knext);
             w2 = __shfl_sync(0xffffffffu, w2, 0);
+            __syncwarp();
             if (w2 != 0 && w2 != kRowFailed && (int64_t)(w2 & 0xFFFFFFull) * 16 <= g.stage) {
               record_fetch(bi ? stage0 : stage1, upool + (int64_t)(w2 >> 24) * 16, (int)((w2 & 0xFFFFFFull) * 16),
                            lane);
@@ -1648,6 +1650,7 @@ __global__ void __launch_bounds__(256, 1)
         w2 = __shfl_sync(0xffffffffu, w2, 0);
         if (ob >= 0 && w2 != 0 && w2 != kRowFailed && (int64_t)(w2 & 0xFFFFFFull) * 16 <= g.stage) {
           asm volatile("fence.acq_rel.gpu;" ::: "memory");
+          __syncwarp();
           record_fetch(ob ? stage1 : stage0, upool + (int64_t)(w2 >> 24) * 16, (int)((w2 & 0xFFFFFFull) * 16), lane);
           (ob ? btag1 : btag0) = knext;
         }
