@@ -755,6 +755,7 @@ __device__ __noinline__ bool tri_large(TriRow<T> row, const T* sval, const doubl
         if (!__all_sync(0xffffffffu, go)) return false;
         continue;
       }
+      __syncwarp();  // the loads below come after the polls that saw the values (a ballot orders no memory)
       for (; b < cnt && (arrived >> b & 1); ++b) {
         const int bk = __shfl_sync(0xffffffffu, nk, b), bv = __shfl_sync(0xffffffffu, vo, b);
         const double* bx = (const double*)__shfl_sync(0xffffffffu, (unsigned long long)xk, b);

@@ -49,3 +49,19 @@ def test_fp64_pivot_blocks_of_17_to_32_rows_in_a_mixed_factor(lo, hi, band):
 def test_rows_of_17_to_32_scalars(lo, hi, band, precision):
     """The pivot block's own space lies right behind the values."""
     _check(lo, hi, 40, band, 7, precision)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_columns_that_every_lane_loads_again(precision):
+    """Dependencies of more than 8 unknowns: the first 8 come from the lane that
+    polled them, the others from each lane's own loads."""
+    V = vb()
+    m = _matrix(17, 40, 30, 5, seed=2)
+    P = V.vbarms_factor(V.vbarms_vbsr_from_blocks(*m), 0, 0.0, -1, precision=precision)
+    n = int(m[0].sum())
+    Po = oracle.Prec(oracle.VBMat(m[0], m[0], *m[1:]), 0, 0.0, -1)
+    for k in range(8):
+        x = np.random.default_rng(k).standard_normal(n)
+        yo = Po.apply(x)
+        tol = 1e-12 if precision == "fp64" else 9 * n * 2.0 ** -24
+        assert np.linalg.norm(_apply(V, P, x) - yo) <= tol * np.linalg.norm(yo)
