@@ -811,12 +811,13 @@ __device__ __forceinline__ bool abs_f32(double v, float& f) {
   f = 0.f;
   return h == 0 && __double2loint(v) == 0;
 }
-// s: the FP32 sum of squares of n <= 4096 entries, ok: all were in range.
+// s: the FP32 sum of squares of n <= 4096 entries, ok: all were in range; none:
+// the FP64 tolerance is zero (its FP32 value t also is when it is below 2^-150).
 // 1: dropped, 0: kept, -1: too near the threshold.  Truncation, the sum and the
 // threshold are off by less than (n + 8) 2^-23 together, the margin by 2^-10.
-__device__ __forceinline__ int drop_f32(float s, bool ok, int m, int n, float t) {
+__device__ __forceinline__ int drop_f32(float s, bool ok, int m, int n, float t, bool none) {
   const float thr = t * (float)m * (float)n, thr2 = thr * thr;
-  if (!ok || !(thr2 == 0.f ? t == 0.f : thr2 >= 1e-30f) || !(thr2 <= 1e30f)) return -1;
+  if (!ok || !(thr2 == 0.f ? none : thr2 >= 1e-30f) || !(thr2 <= 1e30f)) return -1;
   if (s * (1.f + 0x1p-10f) < thr2) return 1;
   if (s * (1.f - 0x1p-10f) >= thr2) return 0;
   return -1;
@@ -1634,7 +1635,7 @@ __global__ void __launch_bounds__(256, 1)
           sf = __fmaf_rn(x, x, sf);
         }
         for (int o = 16; o > 0; o >>= 1) sf += __shfl_xor_sync(0xffffffffu, sf, o);
-        int d = drop_f32(sf, __all_sync(0xffffffffu, in) && sz_m <= 4096, ni, nk, tf);
+        int d = drop_f32(sf, __all_sync(0xffffffffu, in) && sz_m <= 4096, ni, nk, tf, t == 0.0);
         if (d < 0) {  // too near the threshold: the oracle's summation order
           double f2 = 0.0;
           if (lane == 0) f2 = fro2_batched(m, sz_m);
@@ -1882,7 +1883,7 @@ __global__ void __launch_bounds__(256, 1)
               in = abs_f32((double)v[e], x) && in;
               sf = __fmaf_rn(x, x, sf);
             }
-            const int d = drop_f32(sf, in, ni, nc, tf);
+            const int d = drop_f32(sf, in, ni, nc, tf, t == 0.0);
             keep = !(d < 0 ? drop_rule(fro2_batched(v, n), ni, nc, t) : d != 0);
           }
           if (!keep) sstate[q] = SL_DEAD;
