@@ -470,7 +470,9 @@ struct alignas(16) TriSmem {
 };
 
 // The wait of one warp between two polls: a short sleep, the abort word and
-// the time budget every 16th poll.  False when the wait gave up.
+// the time budget every 16th poll.  it = 0 starts it anew: the budget is that of
+// one wait, from arrival to arrival, not of all the waits of a row.  False when
+// the wait gave up.
 struct TriWait {
   unsigned it = 0;
   unsigned long long t0 = 0;
@@ -627,6 +629,7 @@ __device__ __forceinline__ bool tri_row(const TriRow<T>& row, const T* sval, con
       if (!__all_sync(0xffffffffu, go)) return false;
       continue;
     }
+    w.it = 0;
     for (unsigned left = arrived; left;) {
       unsigned mine = left;  // the group's owner: the g-th lowest lane left
 #pragma unroll
@@ -755,6 +758,7 @@ __device__ __noinline__ bool tri_large(TriRow<T> row, const T* sval, const doubl
         if (!__all_sync(0xffffffffu, go)) return false;
         continue;
       }
+      w.it = 0;
       __syncwarp();  // the loads below come after the polls that saw the values (a ballot orders no memory)
       for (; b < cnt && (arrived >> b & 1); ++b) {
         const int bk = __shfl_sync(0xffffffffu, nk, b), bv = __shfl_sync(0xffffffffu, vo, b);
