@@ -199,15 +199,18 @@ __global__ void __launch_bounds__(64)
   __syncthreads();
   if (warp > 0) {
     // reads the next 32 candidates' lists and those of their neighbours into
-    // L1: nothing depends on this warp or on what it reads
+    // L1: no result depends on what it reads.  Its wait is bounded; lane 0 looks
+    // where the greedy is, so that the warp goes on or waits as one.
     volatile long long* vp = &prog;
     volatile const uint32_t* vm = mark;
     auto open = [&](int v) { return !(vm[v >> 5] >> (v & 31) & 1u); };
     for (int64_t base = 32; base < p; base += 32) {
-      long long now = *vp;
-      for (int spin = 0; now + 32 < base && spin < (1 << 22); ++spin) {
+      long long now = 0;
+      for (int spin = 0;; ++spin) {
+        if (lane == 0) now = *vp;
+        now = __shfl_sync(0xffffffffu, now, 0);
+        if (now + 32 >= base || spin >= (1 << 22)) break;
         __nanosleep(40);
-        now = *vp;
       }
       if (now >= base) continue;  // overtaken
       const int64_t i = base + lane;
