@@ -35,7 +35,8 @@
  * Internal scratch and factors live in device memory taken, in stream order on
  * the handle's stream, from a memory pool of the library's own (one per
  * device).  A pool keeps at most an eighth of its device's memory unused while
- * any handle lives, and a 256th after the last one is destroyed.
+ * any handle lives on the device, and a 256th after the last one there has been
+ * destroyed, or dropped by a call that failed.
  */
 #ifndef VBARMS_H
 #define VBARMS_H

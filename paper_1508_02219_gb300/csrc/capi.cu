@@ -235,6 +235,7 @@ vb_status compress_entry(const char* who, int64_t n, const int64_t* rowptr, cons
     cudaStream_t s = (cudaStream_t)stream;
     h->s = s;
     h->dev = current_device();
+    h->pool.attach(h->dev, s);
     h->status.alloc(1, s);
     h->status.zero();
     const int64_t* d_rowptr = rowptr;
@@ -322,6 +323,7 @@ vb_status vbarms_vbsr_from_blocks(int64_t nblk, const int32_t* bsz, const int64_
     cudaStream_t s = (cudaStream_t)stream;
     h->s = s;
     h->dev = current_device();
+    h->pool.attach(h->dev, s);
     h->status.alloc(1, s);
     h->status.zero();
     int64_t n = 0;
@@ -405,6 +407,7 @@ vb_status vbarms_factor(vbarms_vbsr A, int nlev, double droptol, int lfil, const
                opt->wait_limit ? opt->wait_limit : (uint64_t)kDefaultWaitNs, opt->schur_drop_all != 0,
                opt->keep_factors != 0, opt->group_size};
   auto h = std::make_unique<vbarms_prec_st>();
+  h->pool.attach(A->dev, A->s);
   vb_status st = guarded([&] {
     DeviceScope ds(A->dev);
     if (o.precision == VB_FP64)
@@ -470,6 +473,7 @@ vb_status vbarms_factor_batched(int nmat, const vbarms_vbsr* A, const int* nlev,
       int64_t off = 0;
       for (int m : members) {
         res[m] = std::make_unique<vbarms_prec_st>();
+        res[m]->pool.attach(U.dev, s);
         res[m]->impl = P;
         res[m]->off = off;
         res[m]->len = A[m]->C.n;
@@ -498,6 +502,7 @@ vb_status vbarms_dd_factor(vbarms_vbsr A, int nparts, int overlap, int restricte
                opt->wait_limit ? opt->wait_limit : (uint64_t)kDefaultWaitNs, opt->schur_drop_all != 0,
                opt->keep_factors != 0, opt->group_size};
   auto h = std::make_unique<vbarms_prec_st>();
+  h->pool.attach(A->dev, A->s);
   vb_status st = guarded([&] {
     DeviceScope ds(A->dev);
     cudaStream_t s = A->s;
@@ -551,6 +556,7 @@ vb_status vbarms_dd_schur_factor(vbarms_vbsr A, int nparts, int msteps, int nlev
                opt->wait_limit ? opt->wait_limit : (uint64_t)kDefaultWaitNs, opt->schur_drop_all != 0,
                opt->keep_factors != 0, opt->group_size};
   auto h = std::make_unique<vbarms_prec_st>();
+  h->pool.attach(A->dev, A->s);
   vb_status st = guarded([&] {
     DeviceScope ds(A->dev);
     cudaStream_t s = A->s;
@@ -897,11 +903,8 @@ void vbarms_vbsr_destroy(vbarms_vbsr A) {
   if (!A) return;
   try {
     DeviceScope ds(A->dev);
-    const int dev = A->dev;
-    const cudaStream_t s = A->s;
-    cudaStreamSynchronize(s);
+    cudaStreamSynchronize(A->s);
     delete A;
-    pool_idle(dev, s);
   } catch (const Error&) {
     delete A;
   }
@@ -915,11 +918,8 @@ void vbarms_prec_destroy(vbarms_prec M) {
   }
   try {
     DeviceScope ds(M->impl->dev);
-    const int dev = M->impl->dev;
-    const cudaStream_t s = M->impl->s;
-    cudaStreamSynchronize(s);
+    cudaStreamSynchronize(M->impl->s);
     delete M;
-    pool_idle(dev, s);
   } catch (const Error&) {
     delete M;
   }

@@ -109,16 +109,21 @@ __device__ __forceinline__ int ld_relaxed_gpu(const int32_t* p) {
 // 27 of 148; 16 subdomains of 360 000 unknowns, set up and solved: 19 of 88).
 cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s);
 
-// One per handle.  A pool keeps at most an eighth of its device's memory unused
-// while a handle lives, and a 256th after the last one (pool_idle, called with
-// the stream on which that one's buffers were freed).
+// One per handle, its first member (destroyed after the buffers), attached to
+// the handle's device and stream.  A device's pool keeps at most an eighth of its
+// memory unused while a handle lives on it; the last one to go, destroyed or
+// dropped by a call that failed, gives back all but a 256th.
 struct PoolUser {
-  PoolUser();
+  PoolUser() = default;
+  void attach(int device, cudaStream_t stream);
   ~PoolUser();
   PoolUser(const PoolUser&) = delete;
   PoolUser& operator=(const PoolUser&) = delete;
+
+ private:
+  int dev = -1;  // -1: not attached
+  cudaStream_t s = nullptr;
 };
-void pool_idle(int dev, cudaStream_t s);
 
 // Stream-ordered device buffer (pool_alloc / cudaFreeAsync).
 template <typename T>

@@ -26,9 +26,9 @@ constexpr int kPoolDevices = 64;
 std::mutex g_pool_mu;
 struct DevPool {
   cudaMemPool_t pool = nullptr;
-  size_t idle = 0;  // bytes it may keep when no handle lives
+  size_t idle = 0;                    // bytes it may keep when no handle lives on the device
+  std::atomic<long long> users{0};    // handles that do
 } g_pool[kPoolDevices];
-std::atomic<long long> g_pool_users{0};
 
 cudaError_t pool_of(int dev, cudaMemPool_t* out) {
   if (dev < 0 || dev >= kPoolDevices) return cudaErrorInvalidDevice;
@@ -75,17 +75,30 @@ cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
   return e;
 }
 
-PoolUser::PoolUser() { g_pool_users.fetch_add(1); }
-PoolUser::~PoolUser() { g_pool_users.fetch_sub(1); }
+void PoolUser::attach(int device, cudaStream_t stream) {
+  if (dev >= 0 || device < 0 || device >= kPoolDevices) return;
+  dev = device;
+  s = stream;
+  g_pool[dev].users.fetch_add(1);
+}
 
-void pool_idle(int dev, cudaStream_t s) {
-  if (dev < 0 || dev >= kPoolDevices || g_pool_users.load() != 0) return;
-  std::lock_guard<std::mutex> lk(g_pool_mu);
-  const DevPool& D = g_pool[dev];
+PoolUser::~PoolUser() {
+  if (dev < 0 || g_pool[dev].users.fetch_sub(1) != 1) return;
+  cudaMemPool_t pool = nullptr;
+  size_t idle = 0;
+  {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    pool = g_pool[dev].pool;
+    idle = g_pool[dev].idle;
+  }
   uint64_t held = 0;
-  if (D.pool && cudaMemPoolGetAttribute(D.pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
-      held > D.idle && cudaStreamSynchronize(s) == cudaSuccess)
-    (void)cudaMemPoolTrimTo(D.pool, D.idle);
+  int cur = -1;
+  if (pool && cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess && held > idle &&
+      cudaGetDevice(&cur) == cudaSuccess && (cur == dev || cudaSetDevice(dev) == cudaSuccess)) {
+    // the buffers were freed in the stream's order
+    if (cudaStreamSynchronize(s) == cudaSuccess) (void)cudaMemPoolTrimTo(pool, idle);
+    if (cur != dev) (void)cudaSetDevice(cur);
+  }
   (void)cudaGetLastError();
 }
 
