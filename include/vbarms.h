@@ -36,7 +36,7 @@
  * the handle's stream, from a memory pool of the library's own (one per
  * device).  A pool keeps at most an eighth of its device's memory unused while
  * any handle lives on the device, and a 256th after the last one there has been
- * destroyed, or dropped by a call that failed.
+ * destroyed, or dropped by a call that failed; vbarms_memory_trim empties it.
  */
 #ifndef VBARMS_H
 #define VBARMS_H
@@ -397,6 +397,13 @@ vb_status vbarms_prec_pivot_tiles(vbarms_prec M, int lev, int* counts, int* mode
  * threads, all handles); read it before and after a call to count the
  * launches of that call.                                                   */
 uint64_t vbarms_launch_count(void);
+
+/* Gives back the memory that the library's pool of the current device holds
+ * unused, all but keep_bytes, once the device's work so far is done (it waits
+ * for it): for programs whose other allocations need that memory while handles
+ * of the library live.  Later calls take memory anew.  VB_ECUDA without a
+ * device.                                                                    */
+vb_status vbarms_memory_trim(uint64_t keep_bytes);
 
 /* Number of device allocations this library has made since it was loaded
  * (all threads, all handles; every allocation of the library is counted).

@@ -830,6 +830,10 @@ uint64_t vbarms_launch_count(void) { return g_launch_count.load(); }
 
 uint64_t vbarms_alloc_count(void) { return g_alloc_count.load(); }
 
+vb_status vbarms_memory_trim(uint64_t keep_bytes) {
+  return guarded([&] { pool_trim((size_t)keep_bytes); });
+}
+
 vb_status vbarms_prec_ilut_chain(vbarms_prec M, int64_t* links) {
   if (!M) return set_err(VB_EINVAL, "NULL handle");
   if (links) *links = M->impl->ilut_info().chain;

@@ -108,6 +108,8 @@ __device__ __forceinline__ int ld_relaxed_gpu(const int32_t* p) {
 // unknowns: 68 ms of 558 went into mapping memory anew; a batch of 24 matrices:
 // 27 of 148; 16 subdomains of 360 000 unknowns, set up and solved: 19 of 88).
 cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s);
+// All unused memory of the current device's pool but keep bytes goes back.
+void pool_trim(size_t keep);
 
 // One per handle, its first member (destroyed after the buffers), attached to
 // the handle's device and stream.  A device's pool keeps at most an eighth of its

@@ -1,4 +1,5 @@
 // Host/device plumbing: status word readback, prefix sums, partitions.
+#include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
@@ -100,6 +101,21 @@ PoolUser::~PoolUser() {
     if (cur != dev) (void)cudaSetDevice(cur);
   }
   (void)cudaGetLastError();
+}
+
+void pool_trim(size_t keep) {
+  const int dev = current_device();
+  if (dev >= kPoolDevices) return;
+  cudaMemPool_t pool = nullptr;
+  {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    pool = g_pool[dev].pool;
+  }
+  if (!pool) return;
+  VB_CUDA(cudaDeviceSynchronize());  // buffers freed in the order of any stream
+  uint64_t used = 0;
+  VB_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used));
+  VB_CUDA(cudaMemPoolTrimTo(pool, used + std::min<uint64_t>(keep, UINT64_MAX - used)));
 }
 
 void check_status(int* dst, cudaStream_t s, const char* where) {

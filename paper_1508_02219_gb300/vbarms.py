@@ -86,6 +86,7 @@ def lib():
                 "vbarms_apply_static_max_bytes": (C.c_uint64, []),
                 "vbarms_apply_static_need": (i32, [vp, P(C.c_uint64)]),
                 "vbarms_alloc_count": (C.c_uint64, []),
+                "vbarms_memory_trim": (i32, [C.c_uint64]),
                 "vbarms_prec_ilut_geometry": (i32, [vp, P(i32), P(i32), P(i32), P(i32), P(d)]),
                 "vbarms_prec_pivot_tiles": (i32, [vp, i32, vp, vp, P(i32)]),
                 "vbarms_prec_ilut_chain": (i32, [vp, P(i64)]),
@@ -443,6 +444,12 @@ def exported_symbols() -> list[str]:
     txt = open(hdr).read()
     txt = re.sub(r"/\*.*?\*/", "", txt, flags=re.S)
     return sorted(set(re.findall(r"\b(vbarms_\w+|fgmres_solve)\s*\(", txt)))
+
+
+def memory_trim(keep_bytes: int = 0) -> None:
+    """Give back what the library's memory pool of the current device holds
+    unused, all but keep_bytes (waits for the device)."""
+    _check(lib().vbarms_memory_trim(int(keep_bytes)))
 
 
 def launch_count() -> int:
