@@ -309,14 +309,52 @@ __global__ void __launch_bounds__(PIV_T)
   }
 }
 
-// Columns of a block whose loads are in flight together: 720 000 unknowns, A x
-// 523 us instead of 575 (two FP64 operations an entry alone are 250), G x and
-// W x 32 instead of 39.
-constexpr int SPMV_K = 6;
+// One row of a block times its unknowns, op(value, unknown) column by column.
+// K = 1: a plain loop.  K > 1: the loads of K columns first, then their
+// operations; the loop over these is left at the block's end (an FP64 operation
+// takes its 64 cycles whether or not a lane wants its result).
+// Rows of a warp that meet blocks of different sizes wait for one another's loads
+// in the plain loop.  Twenty cycles of FGMRES(1), 360 000 unknowns, 15 neighbours,
+// approximate blocks, plain and K = 8: of 2 unknowns 9.4 and 7.6 ms, of 6 (tau 0.8)
+// 15.7 and 13.0, of 6 (tau 0.9) 23.8 and 18.7, of 10 20.6 and 17.9.  Blocks that
+// are all of one size, 600 000 unknowns on a grid: of 1 4.5 and 4.9, of 4 5.7 and
+// 5.9, of 6 7.2 and 7.2, of 7 7.9 and 8.4, of 8 8.6 and 8.4, of 20 16.1 and 16.1: up
+// to SPMV_PLAIN they take the plain loop.
+constexpr int SPMV_K = 8;
+constexpr int SPMV_PLAIN = 7;
+
+template <int K, typename T, typename Op>
+__device__ __forceinline__ void row_times(const T* v, const double* x, int nc, Op&& op) {
+  if constexpr (K == 1) {
+    for (int k = 0; k < nc; ++k) op(v[k], x[k]);
+  } else {
+    for (int k0 = 0; k0 < nc; k0 += K) {
+      T vk[K];
+      double xk[K];
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        if (k0 + k < nc) vk[k] = v[k0 + k], xk[k] = x[k0 + k];
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        if (k0 + k >= nc) break;
+        op(vk[k], xk[k]);
+      }
+    }
+  }
+}
+
+// All blocks are s x s for one s <= SPMV_PLAIN, as far as their number and values
+// tell.
+template <typename T>
+bool spmv_plain(const VBDev<T>& M) {
+  for (int64_t s = 1; s <= SPMV_PLAIN; ++s)
+    if (M.nval == s * s * M.nnzb) return true;
+  return false;
+}
 
 // y_row -= M x  for every scalar row of a VBCSR M (one thread per scalar row,
 // blocks in order, then the entries of the row).
-template <typename T>
+template <typename T, int K>
 __global__ void k_bsr_sub(VBView<T> M, const int64_t* __restrict__ rowblk, int64_t nrows,
                           const double* __restrict__ x, double* __restrict__ y) {
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nrows; q += (int64_t)gridDim.x * blockDim.x) {
@@ -328,18 +366,8 @@ __global__ void k_bsr_sub(VBView<T> M, const int64_t* __restrict__ rowblk, int64
       for (int64_t b = M.bptr[I]; b < M.bptr[I + 1]; ++b) {
         const int32_t J = M.bcol[b];
         const int nc = M.csz[J];
-        const T* v = M.val + M.voff[b] + (int64_t)a * nc;
-        const double* xj = x + M.coff[J];
-        for (int k0 = 0; k0 < nc; k0 += SPMV_K) {  // loads first, SPMV_K columns at a time
-          float vk[SPMV_K];
-          double xk[SPMV_K];
-#pragma unroll
-          for (int k = 0; k < SPMV_K; ++k)
-            if (k0 + k < nc) vk[k] = (float)v[k0 + k], xk[k] = xj[k0 + k];
-#pragma unroll
-          for (int k = 0; k < SPMV_K; ++k)
-            if (k0 + k < nc) acc = __fmaf_rn(vk[k], (float)xk[k], acc);
-        }
+        row_times<K>(M.val + M.voff[b] + (int64_t)a * nc, x + M.coff[J], nc,
+                     [&](T v, double xk) { acc = __fmaf_rn((float)v, (float)xk, acc); });
       }
       y[q] = y[q] - (double)acc;
       continue;
@@ -348,23 +376,15 @@ __global__ void k_bsr_sub(VBView<T> M, const int64_t* __restrict__ rowblk, int64
     for (int64_t b = M.bptr[I]; b < M.bptr[I + 1]; ++b) {
       const int32_t J = M.bcol[b];
       const int nc = M.csz[J];
-      const T* v = M.val + M.voff[b] + (int64_t)a * nc;
-      const double* xj = x + M.coff[J];
-      for (int k0 = 0; k0 < nc; k0 += SPMV_K) {
-        double vk[SPMV_K], xk[SPMV_K];
-#pragma unroll
-        for (int k = 0; k < SPMV_K; ++k)
-          if (k0 + k < nc) vk[k] = ld(v + k0 + k), xk[k] = xj[k0 + k];
-#pragma unroll
-        for (int k = 0; k < SPMV_K; ++k)
-          if (k0 + k < nc) s = __dsub_rn(s, __dmul_rn(vk[k], xk[k]));
-      }
+      row_times<K>(M.val + M.voff[b] + (int64_t)a * nc, x + M.coff[J], nc,
+                   [&](T v, double xk) { s = __dsub_rn(s, __dmul_rn((double)v, xk)); });
     }
     y[q] = s;
   }
 }
 
 // y = A x (FP64), one thread per scalar row.
+template <int K>
 __global__ void k_spmv(VBView<double> A, const int64_t* __restrict__ rowblk, int64_t nrows,
                        const double* __restrict__ x, double* __restrict__ y) {
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nrows; q += (int64_t)gridDim.x * blockDim.x) {
@@ -374,17 +394,8 @@ __global__ void k_spmv(VBView<double> A, const int64_t* __restrict__ rowblk, int
     for (int64_t b = A.bptr[I]; b < A.bptr[I + 1]; ++b) {
       const int32_t J = A.bcol[b];
       const int nc = A.csz[J];
-      const double* v = A.val + A.voff[b] + (int64_t)a * nc;
-      const double* xj = x + A.coff[J];
-      for (int k0 = 0; k0 < nc; k0 += SPMV_K) {  // loads first, SPMV_K columns at a time
-        double vk[SPMV_K], xk[SPMV_K];
-#pragma unroll
-        for (int k = 0; k < SPMV_K; ++k)
-          if (k0 + k < nc) vk[k] = v[k0 + k], xk[k] = xj[k0 + k];
-#pragma unroll
-        for (int k = 0; k < SPMV_K; ++k)
-          if (k0 + k < nc) s = __dadd_rn(s, __dmul_rn(vk[k], xk[k]));
-      }
+      row_times<K>(A.val + A.voff[b] + (int64_t)a * nc, x + A.coff[J], nc,
+                   [&](double v, double xk) { s = __dadd_rn(s, __dmul_rn(v, xk)); });
     }
     y[q] = s;
   }
@@ -1250,7 +1261,7 @@ static void make_rowblk(int64_t nbr, const int64_t* roff, int64_t n, DBuf<int64_
 
 void spmv_vb(const VBDev<double>& A, const int64_t* rowblk, int64_t n, const double* x, double* y,
              cudaStream_t s) {
-  if (n) launch(k_spmv, grid_for(n, 128, 152LL * 32), 128, 0, s, A.view(), rowblk, n, x, y);
+  if (n) launch(spmv_plain(A) ? k_spmv<1> : k_spmv<SPMV_K>, grid_for(n, 128, 152LL * 32), 128, 0, s, A.view(), rowblk, n, x, y);
   VB_LAUNCH_CHECK();
 }
 
@@ -1385,6 +1396,11 @@ void sweep_last(const PrecDev<T>& P, const SolveBufs& B, const double* g, double
   VB_LAUNCH_CHECK();
 }
 
+template <typename T>
+void bsr_sub(const VBDev<T>& M, const int64_t* rowblk, int64_t n, const double* x, double* y, cudaStream_t s) {
+  launch(spmv_plain(M) ? k_bsr_sub<T, 1> : k_bsr_sub<T, SPMV_K>, grid_for(n, 128), 128, 0, s, M.view(), rowblk, n, x, y);
+}
+
 // Alg. 2 over all levels, in the factorization's own numbering; enqueues
 // work only.  fixv (may be NULL; factorizations with fixed rows only): the
 // values the last level's backward sweep takes for its fixed rows instead of
@@ -1408,7 +1424,7 @@ void solve_core(const PrecDev<T>& P, const double* in, double* out, const SolveB
              mixed ? L.D32.val.p : nullptr, L.ptag.p, L.piv.p, B.bh[l]);
     const int64_t ng = M.n - M.nf;
     if (ng && L.G.nnzb)
-      launch(k_bsr_sub<T>, grid_for(ng, 128), 128, 0, s, L.G.view(), B.grow[l], ng, B.bh[l], B.bh[l] + M.nf);
+      bsr_sub(L.G, B.grow[l], ng, B.bh[l], B.bh[l] + M.nf, s);
     if (fixv && ng)
       launch(k_fix_down, grid_for(ng, 256), 256, 0, s, ng, M.sperm.p + M.nf, L.c.p, l == 0 ? fixv : B.fv[l],
              B.fv[l + 1]);
@@ -1437,7 +1453,7 @@ void solve_core(const PrecDev<T>& P, const double* in, double* out, const SolveB
     const LevelMaps& M = P.maps[l];
     double* xo = l == 0 ? out : B.xh[l - 1] + P.maps[l - 1].nf;
     if (M.nf && L.W.nnzb)
-      launch(k_bsr_sub<T>, grid_for(M.nf, 128), 128, 0, s, L.W.view(), B.wrow[l], M.nf, B.xh[l] + M.nf, B.bh[l]);
+      bsr_sub(L.W, B.wrow[l], M.nf, B.xh[l] + M.nf, B.bh[l], s);
     if (L.grouped)
       grouped_backward<T>(L, B.bh[l], B.xh[l], s);
     else if (L.nD)
