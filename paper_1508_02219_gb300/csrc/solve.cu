@@ -72,6 +72,7 @@ __device__ __forceinline__ double tri_div(double a, double b, double y, double z
     const double q = __fma_rn(a, y, __dmul_rn(a, z));
     return __fma_rn(__fma_rn(-b, q, a), y, q);
   }
+  if (__double2hiint(y) != 0 && __double_as_longlong(a) << 1 == 0) return __dmul_rn(a, y);  // a zero
   return __ddiv_rn(a, b);
 }
 
@@ -80,7 +81,8 @@ __device__ __forceinline__ double tri_div(double a, double b, double y, double z
 // the warp together.  One thread's walk through the largest block, one global
 // load after another, was what each launch waited for (720 000 unknowns, up to
 // 20 rows, eight launches in an application: 60 us each, 19 forward and 45
-// backward now, where an FP64 division still costs 256 cycles a row).
+// backward now, where an FP64 division still costs 256 cycles a row).  PivShape
+// says where a thread to a block is still the better way.
 constexpr int PIV_R = 8;
 
 template <typename TL>
@@ -232,14 +234,31 @@ __device__ __forceinline__ void pivot_backward_warp(const TL* __restrict__ lu, i
 
 constexpr int PIV_T = 128;  // threads per block of the two kernels below
 
-// Pivot blocks per warp: few when the chip has warps to spare, so that a warp
-// meets few large blocks one after the other (an FP64 operation costs the same
-// for 8 lanes as for 32).
-inline int piv_per(int64_t nD) { return nD <= 32768 ? 8 : 32; }
-inline unsigned piv_grid(int64_t nD) { return grid_for(nD, PIV_T / 32 * piv_per(nD)); }
+// How a launch deals out nD pivot blocks: per of them to a warp (fewer than 8
+// while the quarters of the SMs, 608, have no more than two warps each, so that a
+// warp meets few large blocks one after the other; an FP64 operation costs the same
+// for 8 lanes as for 32), and whether the large ones are solved by a thread each all
+// the same.  That is the cheaper way from three blocks a warp on, if most are large
+// (nval values: more than PIV_R rows on average): 32 chains share their operations'
+// time.  One application, two levels, FP32, blocks of one size on a grid; with a
+// thread, with a warp for every block (8 or 32 a warp) and with this rule: 16 rows,
+// 30 000 unknowns 0.27, 0.34 and 0.16 ms; 20 rows, 160 000 unknowns (about 3 000
+// blocks a launch) 0.29, 0.34 (four a warp) and 0.27, 1.0 million 0.52, 1.22 and
+// 0.44.  160 000 nodes of 6 (20 600 blocks, most of them small), 8 and 32 a warp:
+// 3.36 and 3.47 ms; 320 000 nodes (41 500 blocks) 4.35 and 4.32.
+struct PivShape {
+  int per;
+  bool threads;
+  PivShape(int64_t nD, int64_t nval) {
+    per = nD <= 1216 ? 1 : nD <= 2432 ? 2 : nD <= 4864 ? 4 : nD <= 32768 ? 8 : 32;
+    threads = nD > 2432 && nval > nD * PIV_R * PIV_R;
+    if (threads) per = 32;
+  }
+};
+inline unsigned piv_grid(int64_t nD, const PivShape& p) { return grid_for(nD, PIV_T / 32 * p.per); }
 
 __global__ void __launch_bounds__(PIV_T)
-    k_pivot_fwd(int64_t nD, int per, const int32_t* __restrict__ sz, const int64_t* __restrict__ roff,
+    k_pivot_fwd(int64_t nD, int per, bool threads, const int32_t* __restrict__ sz, const int64_t* __restrict__ roff,
                 const int64_t* __restrict__ voff, const double* __restrict__ lu64, const float* __restrict__ lu32,
                 const int32_t* __restrict__ ptag, const int32_t* __restrict__ piv, double* __restrict__ u) {
   const int lane = threadIdx.x & 31;
@@ -254,7 +273,7 @@ __global__ void __launch_bounds__(PIV_T)
         pivot_forward_reg<float>(lu32 + voff[y], piv + roff[y], m, u + roff[y]);
       else
         pivot_forward_reg<double>(lu64 + voff[y], piv + roff[y], m, u + roff[y]);
-    } else if (m > 32) {
+    } else if (m > 32 || (m > PIV_R && threads)) {
       if (f32)
         pivot_forward<float>(lu32 + voff[y], piv + roff[y], m, u + roff[y]);
       else
@@ -262,7 +281,7 @@ __global__ void __launch_bounds__(PIV_T)
     }
     __syncwarp();
     const unsigned f = __ballot_sync(0xffffffffu, f32);
-    for (unsigned w = __ballot_sync(0xffffffffu, m > PIV_R && m <= 32); w; w &= w - 1) {
+    for (unsigned w = __ballot_sync(0xffffffffu, !threads && m > PIV_R && m <= 32); w; w &= w - 1) {
       const int o = __ffs(w) - 1, mo = __shfl_sync(0xffffffffu, m, o);
       if (f >> o & 1)
         pivot_forward_warp<float>(lu32 + voff[y0 + o], piv + roff[y0 + o], mo, u + roff[y0 + o], lane);
@@ -273,7 +292,7 @@ __global__ void __launch_bounds__(PIV_T)
 }
 
 __global__ void __launch_bounds__(PIV_T)
-    k_pivot_bwd(int64_t nD, int per, const int32_t* __restrict__ sz, const int64_t* __restrict__ roff,
+    k_pivot_bwd(int64_t nD, int per, bool threads, const int32_t* __restrict__ sz, const int64_t* __restrict__ roff,
                 const int64_t* __restrict__ voff, const double* __restrict__ lu64, const float* __restrict__ lu32,
                 const int32_t* __restrict__ ptag, const double* __restrict__ u, double* __restrict__ x) {
   __shared__ double stage[PIV_T / 32][32 * 33];
@@ -290,7 +309,7 @@ __global__ void __launch_bounds__(PIV_T)
         pivot_backward_reg<float>(lu32 + voff[y], m, u + roff[y], x + roff[y]);
       else
         pivot_backward_reg<double>(lu64 + voff[y], m, u + roff[y], x + roff[y]);
-    } else if (m > 32) {
+    } else if (m > 32 || (m > PIV_R && threads)) {
       for (int a = 0; a < m; ++a) x[roff[y] + a] = u[roff[y] + a];
       if (f32)
         pivot_backward<float>(lu32 + voff[y], m, x + roff[y]);
@@ -299,7 +318,7 @@ __global__ void __launch_bounds__(PIV_T)
     }
     __syncwarp();
     const unsigned f = __ballot_sync(0xffffffffu, f32);
-    for (unsigned w = __ballot_sync(0xffffffffu, m > PIV_R && m <= 32); w; w &= w - 1) {
+    for (unsigned w = __ballot_sync(0xffffffffu, !threads && m > PIV_R && m <= 32); w; w &= w - 1) {
       const int o = __ffs(w) - 1, mo = __shfl_sync(0xffffffffu, m, o);
       if (f >> o & 1)
         pivot_backward_warp<float>(lu32 + voff[y0 + o], mo, u + roff[y0 + o], x + roff[y0 + o], S, lane);
@@ -1419,9 +1438,11 @@ void solve_core(const PrecDev<T>& P, const double* in, double* out, const SolveB
     if (M.n) launch(k_gather_scale, grid_for(M.n, 256), 256, 0, s, M.n, M.sperm.p, L.r.p, b, B.bh[l]);
     if (L.grouped)
       grouped_forward<T>(L, B.bh[l], s);
-    else if (L.nD)
-      launch(k_pivot_fwd, piv_grid(L.nD), PIV_T, 0, s, L.nD, piv_per(L.nD), L.D.rsz.p, L.D.roff.p, L.D.voff.p, L.D.val.p,
-             mixed ? L.D32.val.p : nullptr, L.ptag.p, L.piv.p, B.bh[l]);
+    else if (L.nD) {
+      const PivShape ps(L.nD, L.D.nval);
+      launch(k_pivot_fwd, piv_grid(L.nD, ps), PIV_T, 0, s, L.nD, ps.per, ps.threads, L.D.rsz.p, L.D.roff.p, L.D.voff.p,
+             L.D.val.p, mixed ? L.D32.val.p : nullptr, L.ptag.p, L.piv.p, B.bh[l]);
+    }
     const int64_t ng = M.n - M.nf;
     if (ng && L.G.nnzb)
       bsr_sub(L.G, B.grow[l], ng, B.bh[l], B.bh[l] + M.nf, s);
@@ -1456,9 +1477,11 @@ void solve_core(const PrecDev<T>& P, const double* in, double* out, const SolveB
       bsr_sub(L.W, B.wrow[l], M.nf, B.xh[l] + M.nf, B.bh[l], s);
     if (L.grouped)
       grouped_backward<T>(L, B.bh[l], B.xh[l], s);
-    else if (L.nD)
-      launch(k_pivot_bwd, piv_grid(L.nD), PIV_T, 0, s, L.nD, piv_per(L.nD), L.D.rsz.p, L.D.roff.p, L.D.voff.p, L.D.val.p,
-             mixed ? L.D32.val.p : nullptr, L.ptag.p, B.bh[l], B.xh[l]);
+    else if (L.nD) {
+      const PivShape ps(L.nD, L.D.nval);
+      launch(k_pivot_bwd, piv_grid(L.nD, ps), PIV_T, 0, s, L.nD, ps.per, ps.threads, L.D.rsz.p, L.D.roff.p, L.D.voff.p,
+             L.D.val.p, mixed ? L.D32.val.p : nullptr, L.ptag.p, B.bh[l], B.xh[l]);
+    }
     if (M.n) launch(k_scatter_scale, grid_for(M.n, 256), 256, 0, s, M.n, M.sperm.p, L.c.p, B.xh[l], xo);
     VB_LAUNCH_CHECK();
   }
