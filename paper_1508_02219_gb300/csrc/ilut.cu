@@ -216,44 +216,69 @@ __device__ __forceinline__ long long norm_key(double f2) { return __double_as_lo
 __device__ __forceinline__ long long norm_key(float f2) { return (long long)__float_as_int(f2); }
 
 // x[perm[j]] <- x[j] for one row of length m, in place: every cycle of the
-// permutation is turned from its smallest place.
+// permutation is turned from its smallest place (seen: the places below 128 that
+// were turned; beyond, a walk along the cycle tells).
 template <typename T, typename F>
 __device__ __forceinline__ void row_permute(T* x, int m, F&& perm) {
+  unsigned long long seen0 = 0, seen1 = 0;
 #pragma unroll 1
   for (int j = 0; j < m; ++j) {
     int q = perm(j);
-    while (q > j && q < m) q = perm(q);
-    if (q != j) continue;  // j is not the smallest place of its cycle
+    if (q == j) continue;
+    if (j < 64 ? seen0 >> j & 1 : j < 128 && (seen1 >> (j - 64) & 1)) continue;
+    if (j >= 128) {
+      while (q > j && q < m) q = perm(q);
+      if (q != j) continue;  // j is not the smallest place of its cycle
+    }
     T v = x[j];
 #pragma unroll 1
     for (q = perm(j); q != j && q >= 0 && q < m; q = perm(q)) {
       const T t = x[q];
       x[q] = v;
       v = t;
+      if (q < 64)
+        seen0 |= 1ull << q;
+      else if (q < 128)
+        seen1 |= 1ull << (q - 64);
     }
     x[j] = v;
   }
 }
 
-// x (one row of length m) <- x (P^T L U)^{-1} = x U^{-1} L^{-1} P, with the
-// factored pivot block read through L2 (written by another warp).
-template <typename T, typename TL>
-__device__ __noinline__ void ainv_right_row(const TL* lu, int S, const int32_t* pv, int m, T* x) {
+// x (one row of length m) <- x (P^T L U)^{-1} = x U^{-1} L^{-1} P, arithmetic in
+// TL, lu(q, j) the factored pivot block and perm(j) its permutation, UN loads in
+// flight.
+template <int UN, typename TL, typename T, typename L, typename F>
+__device__ __forceinline__ void ainv_row(T* x, int m, L&& lu, F&& perm) {
 #pragma unroll 1
   for (int j = 0; j < m; ++j) {
     TL s = (TL)x[j];
-#pragma unroll 1
-    for (int q = 0; q < j; ++q) s = msub<TL>(s, (TL)x[q], __ldcg(lu + q * S + j));
-    x[j] = (T)(s / __ldcg(lu + j * S + j));
+#pragma unroll UN
+    for (int q = 0; q < j; ++q) s = msub<TL>(s, (TL)x[q], lu(q, j));
+    x[j] = (T)(s / lu(j, j));
   }
 #pragma unroll 1
   for (int j = m - 1; j >= 0; --j) {
     TL s = (TL)x[j];
-#pragma unroll 1
-    for (int q = j + 1; q < m; ++q) s = msub<TL>(s, (TL)x[q], __ldcg(lu + q * S + j));
+#pragma unroll UN
+    for (int q = j + 1; q < m; ++q) s = msub<TL>(s, (TL)x[q], lu(q, j));
     x[j] = (T)s;
   }
-  row_permute(x, m, [&](int j) { return __ldcg(pv + j); });
+  row_permute(x, m, perm);
+}
+
+// The pivot block read through L2 (written by another warp); pm: the permutation
+// on chip, or NULL and in place at pg.  One load after another took most of a link
+// where blocks are large: 300 block rows of 28 to 32 scalars FP32 196 ms, 76 with
+// eight in flight (and those of update_general); small blocks are quicker without.
+template <typename T, typename TL>
+__device__ __noinline__ void ainv_right_row(const TL* lu, int S, const int* pm, const int32_t* pg, int m, T* x) {
+  auto at = [&](int q, int j) { return __ldcg(lu + q * S + j); };
+  auto perm = [&](int j) { return pm ? pm[j] : __ldcg(pg + j); };
+  if (m <= 8)
+    ainv_row<1, TL>(x, m, at, perm);
+  else
+    ainv_row<8, TL>(x, m, at, perm);
 }
 
 // Workspace hash: keys[h] = -2 - slot, -1 = empty; the column of a slot is
@@ -285,8 +310,8 @@ __device__ __forceinline__ int ws_lookup(const int* keys, const int* scol, uint3
 constexpr int MAX_SLOTS = 4096;  // largest workspace (blocks of one working row)
 
 // Warp-cooperative copy with eight independent loads in flight per lane.
-template <typename T>
-__device__ __noinline__ void warp_copy(T* __restrict__ dst, const T* __restrict__ src, int64_t n, int lane) {
+template <typename TD, typename T>
+__device__ __noinline__ void warp_copy(TD* __restrict__ dst, const T* __restrict__ src, int64_t n, int lane) {
 #pragma unroll 1
   for (int64_t e0 = lane; e0 < n; e0 += 32 * 8) {
     T v[8];
@@ -298,7 +323,7 @@ __device__ __noinline__ void warp_copy(T* __restrict__ dst, const T* __restrict_
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int64_t e = e0 + 32 * u;
-      if (e < n) dst[e] = v[u];
+      if (e < n) dst[e] = (TD)v[u];
     }
   }
 }
@@ -348,25 +373,16 @@ __device__ __forceinline__ float fro2_f32(const T* __restrict__ v, int n) {
   return s;
 }
 
-// x (one row of length m) <- x (P^T L U)^{-1} from a staged pivot block
-// (values of type TS, arithmetic in TL); x lives in shared memory.
+// The same from a staged pivot block (values of type TS); x may live in shared
+// memory.
 template <typename T, typename TL, typename TS>
 __device__ __noinline__ void ainv_right_row_sh(const TS* lu, int S, const int* pv, int m, T* x) {
-#pragma unroll 1
-  for (int j = 0; j < m; ++j) {
-    TL s = (TL)x[j];
-#pragma unroll 1
-    for (int q = 0; q < j; ++q) s = msub<TL>(s, (TL)x[q], (TL)lu[q * S + j]);
-    x[j] = (T)(s / (TL)lu[j * S + j]);
-  }
-#pragma unroll 1
-  for (int j = m - 1; j >= 0; --j) {
-    TL s = (TL)x[j];
-#pragma unroll 1
-    for (int q = j + 1; q < m; ++q) s = msub<TL>(s, (TL)x[q], (TL)lu[q * S + j]);
-    x[j] = (T)s;
-  }
-  row_permute(x, m, [&](int j) { return pv[j]; });
+  auto at = [&](int q, int j) { return (TL)lu[q * S + j]; };
+  auto perm = [&](int j) { return pv[j]; };
+  if (m <= 8)
+    ainv_row<1, TL>(x, m, at, perm);
+  else
+    ainv_row<8, TL>(x, m, at, perm);
 }
 
 // |x| as an integer key: non-negative IEEE values order like their bit
@@ -396,15 +412,17 @@ __device__ __forceinline__ float div_rn<float>(float a, float b) {
 // then the lanes form the multipliers and update the trailing block, so every
 // element receives the operations of the sequential algorithm in its order.
 // Pivot rows go to gpiv (and pvs when not null).  Returns false when a pivot
-// column is exactly zero.
-template <typename TL>
+// column is exactly zero.  FAR: a lies in global memory, where one element after
+// another cost a trip to L2 each (30 block rows of 100 to 128 scalars FP64 642 ms,
+// 577 with four rows in flight and the copies of the block too).
+template <typename TL, bool FAR = false>
 __device__ __noinline__ bool gepp_warp(TL* a, int n, int* pvs, int32_t* gpiv, int lane) {
 #pragma unroll 1
   for (int kk = 0; kk < n; ++kk) {
     // the largest |a_ik|, its upper word first, the lowest row on ties
     unsigned long long key = 0;  // |a| + 1, 0: no row
     int idx = 0x7fffffff;
-#pragma unroll 1
+#pragma unroll(FAR ? 4 : 1)
     for (int ii = kk + lane; ii < n; ii += 32) {
       const unsigned long long v = (unsigned long long)abs_key(a[ii * n + kk]) + 1ull;
       if (v > key) {
@@ -440,13 +458,31 @@ __device__ __noinline__ bool gepp_warp(TL* a, int n, int* pvs, int32_t* gpiv, in
       *l = div_rn<TL>(*l, d);
     }
     __syncwarp();
+    if (FAR) {  // lanes over columns, four rows in flight
 #pragma unroll 1
-    for (int e = lane; e < w * w; e += 32) {
-      int r = (int)((float)e * rw), c = e - r * w;  // e / w, corrected
-      if (c < 0) --r, c += w;
-      if (c >= w) ++r, c -= w;
-      const int ii = kk + 1 + r, jj = kk + 1 + c;
-      a[ii * n + jj] = msub<TL>(a[ii * n + jj], a[ii * n + kk], a[kk * n + jj]);
+      for (int jj = kk + 1 + lane; jj < n; jj += 32) {
+        const TL u = a[kk * n + jj];
+        int ii = kk + 1;
+#pragma unroll 1
+        for (; ii + 4 <= n; ii += 4) {
+          TL acc[4], l[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t) acc[t] = a[(ii + t) * n + jj], l[t] = a[(ii + t) * n + kk];
+#pragma unroll
+          for (int t = 0; t < 4; ++t) a[(ii + t) * n + jj] = msub<TL>(acc[t], l[t], u);
+        }
+#pragma unroll 1
+        for (; ii < n; ++ii) a[ii * n + jj] = msub<TL>(a[ii * n + jj], a[ii * n + kk], u);
+      }
+    } else {
+#pragma unroll 1
+      for (int e = lane; e < w * w; e += 32) {
+        int r = (int)((float)e * rw), c = e - r * w;  // e / w, corrected
+        if (c < 0) --r, c += w;
+        if (c >= w) ++r, c -= w;
+        const int ii = kk + 1 + r, jj = kk + 1 + c;
+        a[ii * n + jj] = msub<TL>(a[ii * n + jj], a[ii * n + kk], a[kk * n + jj]);
+      }
     }
     __syncwarp();
   }
@@ -1143,11 +1179,17 @@ __device__ __noinline__ void copy_blocks(int n, int sz, int so, long long dof, c
 // A factored pivot block (rows S apart) and the reciprocals of its diagonal into
 // a record.
 template <typename TL>
-__device__ __noinline__ void put_pivot(const TL* lu, int S, int n, TL* o, TL* rcp, int lane) {
+__device__ __noinline__ void put_pivot(const TL* __restrict__ lu, int S, int n, TL* __restrict__ o,
+                                       TL* __restrict__ rcp, int lane) {
+  if (S == n) {
+#pragma unroll 4
+    for (int e = lane; e < n * n; e += 32) o[e] = lu[e];
+  } else {
 #pragma unroll 1
-  for (int e = lane; e < n * n; e += 32) {
-    const int a = e / n;
-    o[e] = lu[a * S + e - a * n];
+    for (int e = lane; e < n * n; e += 32) {
+      const int a = e / n;
+      o[e] = lu[a * S + e - a * n];
+    }
   }
 #pragma unroll 1
   for (int a = lane; a < n; a += 32) {
@@ -1242,7 +1284,7 @@ __device__ __noinline__ void update_general(CopyTab& tab, int nq, int off, int c
   const int sz = ni * nj;
   if (missing) {
     T* z = wv + off;
-#pragma unroll 1
+#pragma unroll 4
     for (int e = 0; e < sz; ++e) z[e] = (T)0;
   }
   int incl = sz;
@@ -1294,7 +1336,7 @@ __device__ __noinline__ void update_general(CopyTab& tab, int nq, int off, int c
 #pragma unroll 1
         for (int r = 0; r < nk; ++r) av = msub<T>(av, m[a4[u] * nk + r], U[r * nj4[u] + jj4[u]]);
       } else {
-#pragma unroll 1
+#pragma unroll 8
         for (int r = 0; r < nk; ++r) av = msub<T>(av, m[a4[u] * nk + r], __ldcg(U + r * nj4[u] + jj4[u]));
       }
       *dst[u] = av;
@@ -1586,6 +1628,13 @@ __global__ void __launch_bounds__(256, 1)
           for (int r = 0; r < nk; ++r) M.mt[r * np + lane] = (T)0;
         }
       } else {
+        const int* pm = nullptr;  // a record read in place: its permutation, on chip
+        if (!staged && nk <= PVMAX) {
+#pragma unroll 1
+          for (int a = lane; a < nk; a += 32) M.perm[a] = __ldcg(rperm + a);
+          __syncwarp();
+          pm = M.perm;
+        }
 #pragma unroll 1
         for (int a = lane; a < ni; a += 32) {
           if (staged) {
@@ -1596,9 +1645,9 @@ __global__ void __launch_bounds__(256, 1)
               ainv_right_row_sh<T, float, T>(reinterpret_cast<const T*>(rec + RL.lu), S, rperm, nk, m + a * nk);
           } else {
             if (lu64)
-              ainv_right_row<T, double>(reinterpret_cast<const double*>(rec + RL.lu), S, rperm, nk, m + a * nk);
+              ainv_right_row<T, double>(reinterpret_cast<const double*>(rec + RL.lu), S, pm, rperm, nk, m + a * nk);
             else
-              ainv_right_row<T, T>(reinterpret_cast<const T*>(rec + RL.lu), S, rperm, nk, m + a * nk);
+              ainv_right_row<T, T>(reinterpret_cast<const T*>(rec + RL.lu), S, pm, rperm, nk, m + a * nk);
           }
         }
       }
@@ -1803,16 +1852,17 @@ __global__ void __launch_bounds__(256, 1)
       if (btag1 == (int)k) btag1 = -1;
     }
     record_wait<0>();  // every record fetched ahead has been used, unless the row failed
-    // A row that ends in the global workspace has its slot metadata copied
-    // to the shared working-row region (unused by such a row) when it fits,
-    // so that the scans of the finish read on-chip data; its values stay in
-    // the global workspace.
-    bool meta_sh = false;
+    // A row that ends in the global workspace has its slot metadata copied to the
+    // end of the shared working-row region (unused by such a row) when it fits, so
+    // that the scans of the finish read on-chip data; its values stay in the global
+    // workspace.  The rest of the region, right behind the stage buffers, takes a
+    // large pivot block (200 block rows of 33 to 40 scalars FP32 181 ms, 156 with it).
+    int region_end = in_sh ? g.o_vals : g.o_lc;  // end of what is free behind the stage buffers
     if (!in_sh && status_local == 0) {
       const int region = g.o_lc - g.o_vals;  // vals, hash and slot arrays of the shared workspace
       if (ns * 24 <= region) {
-        meta_sh = true;
-        long long* mf2 = reinterpret_cast<long long*>(wb + g.o_vals);
+        region_end = g.o_vals + ((region - ns * 24) & ~15);
+        long long* mf2 = reinterpret_cast<long long*>(wb + region_end);
         int* mcol = reinterpret_cast<int*>(mf2 + ns);
         int* mst = mcol + ns;
         int* mncl = mst + ns;
@@ -1922,7 +1972,7 @@ __global__ void __launch_bounds__(256, 1)
       if (lane == 0) roff16 = atomicAdd(P.ctr + 2, (unsigned long long)(rbytes / 16));
     }
     // GEPP of the diagonal block, in registers, in shared memory when it fits
-    // (the stage buffers' free part), else in place.  FP64 factor: FP64 in the
+    // (the stage buffers' free part, and the space behind them), else in place.  FP64 factor: FP64 in the
     // oracle's operation order.  Mixed factor: FP32 GEPP and 1-norm condition
     // estimate (explicit inverse columns); a block above the threshold, larger
     // than 32, or singular in FP32 is factored again in FP64 and tagged.
@@ -1934,18 +1984,17 @@ __global__ void __launch_bounds__(256, 1)
     if (status_local == 0) {
       const T* srcd = wv + soff[dslot];
       unsigned char* gb = stage0 + gb_at;
-      const int gcap = 2 * g.stage - gb_at;
+      const int gcap = region_end - g.o_stage - gb_at;
       int* pvs = ni <= PVMAX ? M.pv : nullptr;
       int32_t* gpiv = piv + A.roff[i];
       bool ok = true;
       if constexpr (F32) {
         tag64 = true;
-        float norm1 = 0.f;
-#pragma unroll 1
-        for (int jj = lane; jj < ni; jj += 32) {
+        float norm1 = 0.f;  // (a larger block is factored in FP64)
+        if (lane < ni && ni <= 32) {
           float sum = 0.f;
 #pragma unroll 1
-          for (int ii = 0; ii < ni; ++ii) sum += fabsf(srcd[ii * ni + jj]);
+          for (int ii = 0; ii < ni; ++ii) sum += fabsf(srcd[ii * ni + lane]);
           norm1 = fmaxf(norm1, sum);
         }
         norm1 = warp_max_f(norm1);
@@ -1977,11 +2026,12 @@ __global__ void __launch_bounds__(256, 1)
         __syncwarp();
       }
       if (tag64) {
-        double* a = ni * ni * 8 <= gcap ? reinterpret_cast<double*>(gb) : dg + dgoff[i];
-#pragma unroll 1
+        const bool far = ni * ni * 8 > gcap;
+        double* a = far ? dg + dgoff[i] : reinterpret_cast<double*>(gb);
+#pragma unroll 4
         for (int e = lane; e < ni * ni; e += 32) a[e] = (double)srcd[e];
         __syncwarp();
-        ok = gepp_warp<double>(a, ni, pvs, gpiv, lane);
+        ok = far ? gepp_warp<double, true>(a, ni, pvs, gpiv, lane) : gepp_warp<double>(a, ni, pvs, gpiv, lane);
         lu_g64 = a;
       }
       __syncwarp();
@@ -2083,20 +2133,21 @@ __global__ void __launch_bounds__(256, 1)
     // ---- what no other row reads: the pivot block as the solve takes it, then
     // the L part
     if (status_local == 0) {
+      if (!lu_sm && tag64) {
+        double* d = dg + dgoff[i];
+        if (lu_g64 != d) {
 #pragma unroll 1
-      for (int e = lane; e < ni * ni; e += 32) {
-        if (lu_sm) {
+          for (int e = lane; e < ni * ni; e += 32) d[e] = lu_g64[e];
+        }
+        if (mixed) {
+#pragma unroll 4
+          for (int e = lane; e < ni * ni; e += 32) dg32[dgoff[i] + e] = (float)lu_g64[e];
+        }
+      } else {
+#pragma unroll 1
+        for (int e = lane; e < ni * ni; e += 32) {
           const int a = e / ni;
-          const float v = (float)M.lu[a * NSMALL + e - a * ni];
-          dg32[dgoff[i] + e] = v;
-          dg[dgoff[i] + e] = (double)v;
-        } else if (tag64) {
-          const double v = lu_g64[e];
-          dg[dgoff[i] + e] = v;
-          if (mixed) dg32[dgoff[i] + e] = (float)v;
-        } else {
-          const int a = e / ni;
-          const float v = (float)lu_g[a * lu_str + e - a * ni];
+          const float v = lu_sm ? (float)M.lu[a * NSMALL + e - a * ni] : (float)lu_g[a * lu_str + e - a * ni];
           dg32[dgoff[i] + e] = v;
           dg[dgoff[i] + e] = (double)v;
         }
@@ -2190,12 +2241,10 @@ __global__ void __launch_bounds__(256, 1)
       P.lstart[i] = status_local == 0 ? (int64_t)lb : 0;
       P.lcnt[i] = status_local == 0 ? nL : 0;
     }
-    // clear the hash positions this row used (and the shared hash when the
-    // finish staged metadata over it)
-    if (in_sh || meta_sh) {
+    // clear the shared hash, over which the finish of a row in global memory
+    // staged its metadata and its pivot block, and the positions such a row used
 #pragma unroll 1
-      for (int q = lane; q < g.hash; q += 32) sh_keys[q] = -1;
-    }
+    for (int q = lane; q < g.hash; q += 32) sh_keys[q] = -1;
     if (!in_sh) {
 #pragma unroll 1
       for (int q = lane; q < ns; q += 32)
