@@ -65,3 +65,25 @@ def test_columns_that_every_lane_loads_again(precision):
         yo = Po.apply(x)
         tol = 1e-12 if precision == "fp64" else 9 * n * 2.0 ** -24
         assert np.linalg.norm(_apply(V, P, x) - yo) <= tol * np.linalg.norm(yo)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("lo,hi", [(33, 33), (63, 65), (95, 98), (120, 128)])
+def test_pivot_blocks_of_up_to_128_rows(lo, hi, precision):
+    """Blocks of one to four rows a lane, interchanges in every third and in random
+    ones."""
+    V = vb()
+    m = list(_matrix(lo, hi, 8, 1, seed=lo))
+    bsz, bptr, bcol, voff, val = m
+    rng = np.random.default_rng(hi)
+    for i in range(1, 8, 2):
+        b = int(bptr[i] + np.searchsorted(bcol[bptr[i]:bptr[i + 1]], i))
+        d = val[voff[b]:voff[b + 1]].reshape(bsz[i], bsz[i])
+        d[:] = d[rng.permutation(bsz[i])]
+    n = int(bsz.sum())
+    P = V.vbarms_factor(V.vbarms_vbsr_from_blocks(*m), 0, 0.0, -1, precision=precision)
+    x = np.random.default_rng(3).standard_normal(n)
+    yo = oracle.Prec(oracle.VBMat(m[0], m[0], *m[1:]), 0, 0.0, -1).apply(x)
+    # the bounds above
+    tol = 1e-12 if precision == "fp64" else 9 * n * 2.0 ** -24
+    assert np.linalg.norm(_apply(V, P, x) - yo) <= tol * np.linalg.norm(yo)
