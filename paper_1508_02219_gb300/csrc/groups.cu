@@ -174,7 +174,12 @@ __global__ void __launch_bounds__(32) k_gr_greedy(int64_t p, const int32_t* __re
 // supernodes in groups of four, four levels, 7 875 groups: 23.4 ms before; 13.2
 // with one warp; 11.2 to 11.8 with a second that reads ahead (three or seven that do:
 // 11.1).
-constexpr int64_t GR_SHMAX = 880000;  // supernodes whose mask leaves half of the SM's 256 KB to L1
+// Both greedies on the first level (the ordering's time, groups of four): 93 000
+// supernodes 10.8 ms with the mask on chip and 20.7 with marks in global memory,
+// 374 000 42.9 and 88.1, 785 000 92 and 192.  The line is where two masks would fill
+// the shared memory; one mask is still the better way beyond it (1.12 million: 133
+// ms against the 281 that they take).
+constexpr int64_t GR_SHMAX = 880000;
 
 __global__ void k_gr_elig(int64_t p, const double* __restrict__ w, double ddtol, const int32_t* __restrict__ fixed,
                           uint32_t* __restrict__ elig) {

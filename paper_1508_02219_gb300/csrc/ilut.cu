@@ -34,12 +34,12 @@
 // of 2 KB and 128 registers, the records of more than about ten U blocks (FP64:
 // four) were read in place from L2, one dependent load after another, and half
 // of the rows worked in global memory: 32 us a link (FP64 42 to 66).  Now 7
-// warps an SM (FP64 5, wide rows 3) have all their registers and keep records
-// and rows on chip; a step's update takes a column per lane, divisions by pivot
+// warps an SM (FP64 5, wide rows 3) have up to 255 registers a thread (FP32: 64
+// bytes spilled, FP64 none) and keep records and rows on chip; a step's update takes a column per lane, divisions by pivot
 // entries are corrected products with their reciprocals, the pivot search and
 // the reciprocals overlap, and FP64 drop tests are decided in FP32 where that
 // is certain.  The kernel's time before and now: 3.0 million unknowns FP32 710
-// and 376 ms, 360 000 FP64 498 and 261 ms, 48 000 at tau 0.9 786 and 253 ms.
+// and 385 ms, 360 000 FP64 498 and 261 ms, 48 000 at tau 0.9 786 and 254 ms.
 //
 // A wait that runs out sets VB_ETIMEOUT and raises an abort flag; a row that
 // failed publishes kRowFailed so that its dependants stop too.  Overflowing a
@@ -2455,16 +2455,20 @@ void ilut_last(LastDev<T>& X, double t, int lfil, bool mixed, double cond_thr, u
   // prefix of the ticket order is factored exactly on its own), the fastest
   // kept per device, precision and class of row sizes for the rest of the
   // process; small matrices take the first.  What counts is that records and
-  // working rows stay on chip; the rows in flight then matter little (3.0
-  // million unknowns FP32, the whole factorization when the chosen shape read 644
-  // ms, which is 474 now; slots / value bytes / stage bytes: 64 / 6 144 / 3 072, 8 warps an SM, 709 ms; 128 / 8 192 / 4 096, 8
-  // warps, 671; 128 / 12 288 / 4 096, 7 warps, 644; 128 / 16 384 / 6 144, 5
-  // warps, 677).  FP64 rows hold twice the bytes (360 000 unknowns: 128 / 8 192
-  // / 6 144, 7 warps, 382 ms; 128 / 16 384 / 6 144, 5 warps, 339); rows of many
-  // small blocks need slots (48 000 unknowns at tau 0.9: 512 / 8 192 / 4 096
-  // 527 ms; 512 / 16 384 487; 768 / 16 384, 3 warps, 454).  The prefix is 1/64
-  // of the tickets (2 048 to 16 384), so the timings add at most about 5 % to
-  // the first factorization of a class.
+  // working rows stay on chip; the rows in flight then matter little.  Shapes as
+  // slots / value bytes / stage bytes.  3.0 million unknowns FP32, whole
+  // factorizations with an earlier finish of the rows (the chosen shape's takes 475
+  // ms now): 64 / 6 144 / 3 072, 8 warps an SM, 709 ms; 128 / 8 192 / 4 096, 8
+  // warps, 671; 128 / 12 288 / 4 096, 7 warps, 644; 128 / 16 384 / 6 144, 5 warps,
+  // 677.  FP64 rows hold twice the bytes (360 000 unknowns: 128 / 8 192 / 6 144, 7
+  // warps, 382 ms; 128 / 16 384 / 6 144, 5 warps, 339).  Rows of many small blocks
+  // need slots: 48 000 unknowns at tau 0.9, this kernel, FP32 and FP64: 512 / 16 384
+  // / 4 096, 4 warps, 290 and 586 ms; 768 / 16 384 / 4 096, 3 warps, 255 and 556.
+  // (Fewer and larger workspaces measured shorter chains there still: 768 / 24 576 /
+  // 4 096 242 and 517, 1 024 / 32 768 / 8 192, 2 warps, 239 and 486; not timed where
+  // more than one chain is in flight.)  The prefix is 1/64 of the tickets (2 048 to
+  // 16 384), so the timings add at most about 5 % to the first factorization of a
+  // class.
   DBuf<unsigned long long> rstat(2, s);
   rstat.zero();
   launch(k_row_stats, grid_for(p, 256), 256, 0, s, p, A.bptr.p, rstat.p);

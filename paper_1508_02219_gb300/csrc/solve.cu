@@ -1048,10 +1048,11 @@ __device__ __noinline__ void tri_pivot_large(const TL* __restrict__ lu, const in
 // 0.35 us forward and 0.8 us backward in FP32 (products of the last arrival
 // 330 cycles, sum over the owners 160, subtraction 100, pivot solve 700), and
 // several times that in FP64, whose operations take 64 cycles each.  One
-// application, with flags, fences and one-lane pivot solves before and now:
-// 3.0 million unknowns FP32 (2 650 levels each way) 34.9 and 11.6 ms; 48 000
-// unknowns at tau 0.9 FP32 (5 100 and 6 190 levels) 60.6 and 17.1 ms; 360 000
-// unknowns FP64 (1 930 levels) 51.8 and 15.6 ms; 18 000 FP64 10.2 and 3.3 ms.
+// application's two sweeps, with flags, fences and one-lane pivot solves before and
+// now: 3.0 million unknowns FP32 (2 650 levels each way) 33.2 and 9.6 ms; 48 000
+// unknowns at tau 0.9 FP32 (5 100 and 6 190 levels) 60.0 and 16.7 ms; 360 000
+// unknowns FP64 (1 930 levels) 51 and 14.9 ms; 18 000 FP64 (the whole application)
+// 10.2 and 3.2 ms.
 template <typename T, bool BWD, typename R>
 __global__ void __launch_bounds__(TRI_W * 32, TRI_B)
     k_tri(VBView<T> M, const int64_t* __restrict__ dgoff, const double* __restrict__ lu64,
@@ -1190,6 +1191,9 @@ __global__ void __launch_bounds__(TRI_W * 32, TRI_B)
           if constexpr (sizeof(T) == sizeof(float)) {  // FP32 pivot blocks belong to FP32 factors only
             bool ok = false;
             float x = 0.f;
+            // in line up to 6 rows only (applications of 200 000 unknowns in blocks of
+            // 4, 6 and 8, two levels: up to 6 0.449, 0.466, 0.455 ms; up to 8 0.449,
+            // 0.470, 0.436; none 0.477, 0.493, 0.455)
             if (ni <= 6 && fast) x = tri_pivot_f32<6, 8, true>(sm.lu, sm.ry, sm.rz, ni, src, uf, lane, &ok);
             if (!ok) x = tri_pivot_f32_wide(sm.lu, sm.ry, sm.rz, ni, src, fast, uf, lane);
             if constexpr (narrow)
